@@ -80,10 +80,11 @@ extern "C" {
 #define KIN_LAYOUT_LANE 1 /* one lane integrates one cell (the paper's thread-per-ODE
                              design, Section 3): per-cell arrays in the workspace or in
                              shared memory (kin_opts.staging) */
-#define KIN_LAYOUT_WARP 2 /* one warp integrates one cell: its 32 lanes share the
-                             reactions and species of f; the cell's concentrations and
-                             rates of progress live in shared memory. staging is
-                             ignored; for RKC, occupancy selects the register budget
+#define KIN_LAYOUT_WARP 2 /* one warp (or half of one, or up to four: the library's
+                             choice by the state's size) integrates one cell: its
+                             lanes share the reactions and species of f; the cell's
+                             concentrations and rates of progress live in shared
+                             memory. staging is ignored; for RKC, occupancy selects the register budget
                              (KIN_OCC_HIGH: for up to 64 state components 48
                              registers and 40 warps per SM, or 80 registers and 24
                              warps with the energy equation); block_threads may be up

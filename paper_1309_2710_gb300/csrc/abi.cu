@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "codegen.h"
+#include "int_tables.h"
 #include "kin_dev.cuh"
 #include "seg_tables.h"
 
@@ -59,6 +60,7 @@ struct Grid {
     int threads, blocks;  // persistent grid
     int64_t nslots;
     int layout;           // KIN_LAYOUT_LANE or KIN_LAYOUT_WARP (resolved)
+    int lanes;            // lanes per cell (1 in the lane layout)
 };
 
 // Automatic layout: one warp per cell for large mechanisms (a lane's working
@@ -69,6 +71,25 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm)
     if (o->layout != KIN_LAYOUT_AUTO) return o->layout;
     if (m->nR > KIN_WARP_MIN_REACTIONS) return KIN_LAYOUT_WARP;
     return cells < (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
+}
+
+// Lanes that integrate one cell in the warp layout: half a warp for states of
+// at most 16 components (RKCK; RKC in isothermal FP64), a warp, and in
+// isothermal FP64 RKC two warps above 32 components and four above 64. An
+// evaluation is a chain of short phases, so more lanes shorten it, and the
+// FP64 pipe's vector work per cell stays the same (fewer slots per lane on more
+// warps). Measured on GB300, 2 or 4 warps against 1: 53 species, 256 / 4,096 /
+// 20,000 cells 10.4 against 18.9, 37.7 against 43.9, 157.9 against 159.4 ms;
+// 111 species, 200 / 8,000 cells 42 against 175, 231 against 323 ms. One warp
+// where the block size does not hold whole groups, and with KIN_OCC_HIGH, whose
+// 48-register kernels exist for single warps.
+int cell_lanes(const kin_opts* o, int nV, int threads)
+{
+    const bool f64 = o->method == KIN_RKC && o->precision == KIN_FP64 && !o->energy;
+    if (nV <= 16) return o->method == KIN_RKCK || f64 ? 16 : 32;
+    if (!f64 || o->occupancy || nV <= 32) return 32;
+    const int g = nV <= 64 ? 64 : 128;
+    return threads % g ? 32 : g;
 }
 
 int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
@@ -87,24 +108,26 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
         return fail(KIN_EUNSUPPORTED, "the energy equation needs the mechanism's cp and Hf");
     const int layout = resolve_layout(m, o, cells, nsm);
     int threads = o->block_threads > 0 ? o->block_threads : 128;
-    int occ = 0, cap = 0;
+    int occ = 0, cap = 0, lanes = 1;
     if (layout == KIN_LAYOUT_WARP) {
         if (threads % 32 != 0 || threads > 256) return fail(KIN_EINVAL, "block_threads must be a multiple of 32 and <= 256");
-        const int cell_lanes = warp_cell_lanes(o->method, m->nS + o->energy);
-        const size_t sm = warp_smem(m->dev, o->precision, o->energy, threads) * (32 / cell_lanes);
+        lanes = cell_lanes(o, m->nS + o->energy, threads);
+        // the layout's limit on a mechanism: C and Omega of a block's cells in
+        // shared memory (the FP64 f's own words need no more)
+        const size_t sm = (size_t)((m->nS + m->nR + 3) & ~3) * 8 * (threads / std::min(lanes, 32));
         if (sm > (size_t)maxsm)
             return fail(KIN_EUNSUPPORTED, "warp layout needs %zu bytes of shared memory per block (max %d)", sm, maxsm);
         const int nV = m->nS + o->energy;
         if (o->method == KIN_RKCK) {
-            e = o->precision == KIN_MIXED ? occ_warp_rkck_f32(m->dev, nV, o->energy, threads, &occ)
-                                          : occ_warp_rkck_f64(m->dev, nV, o->energy, threads, &occ);
+            e = o->precision == KIN_MIXED ? occ_warp_rkck_f32(m->dev, nV, lanes, o->energy, threads, &occ)
+                                          : occ_warp_rkck_f64(m->dev, nV, lanes, o->energy, threads, &occ);
         } else {
-            using OccFn = cudaError_t (*)(const MechDev&, int, int, int*);
+            using OccFn = cudaError_t (*)(const MechDev&, int, int, int, int*);
             // [energy][precision][occupancy]
             static const OccFn fns[2][2][2] = {
                 {{occ_warp_f64_o0, occ_warp_f64_o1}, {occ_warp_f32_o0, occ_warp_f32_o1}},
                 {{occ_warp_f64_en_o0, occ_warp_f64_en_o1}, {occ_warp_f32_en_o0, occ_warp_f32_en_o1}}};
-            e = fns[o->energy][o->precision == KIN_MIXED][o->occupancy ? 1 : 0](m->dev, nV, threads, &occ);
+            e = fns[o->energy][o->precision == KIN_MIXED][o->occupancy ? 1 : 0](m->dev, nV, lanes, threads, &occ);
         }
         cap = occ;  // as many as fit
     } else {
@@ -126,6 +149,7 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
     g->blocks = nsm * bps;
     g->nslots = (int64_t)g->blocks * threads;
     g->layout = layout;
+    g->lanes = lanes;
     return KIN_OK;
 }
 
@@ -464,6 +488,33 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
         }
     const size_t oEll32 = put(ell32.data(), sizeof(CsrW32) * ell_n);
     const size_t oEll64 = put(ell64.data(), sizeof(CsrW64) * ell_n);
+    // the integer FP64 f (int_tables.h), for each group size that the mechanism
+    // can take; eight rounds of reactions a chunk, so that the words of a
+    // 53-species / 634-reaction cell (7.4 KB for a warp) leave room for 16 warps
+    // per SM beside the tables in L1
+    IntGather ig[INT_NTAB];
+    size_t oIg[INT_NTAB][4];
+    const int ig_lanes[INT_NTAB] = {16, 32, 64, 128};
+    const bool ig_use[INT_NTAB] = {nS <= 16, true, nS > 32 && nS <= 64, nS > 64};
+    for (int v = 0; v < INT_NTAB; ++v) {
+        if (!ig_use[v]) continue;
+        const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, 8 * ig_lanes[v]));
+        ig[v] = build_int_gather(nS, nR, ptr.data(), crxp.data(), cnu.data(), chunk, ig_lanes[v]);
+        oIg[v][0] = put(ig[v].step0.data(), 4 * ig[v].step0.size());
+        oIg[v][1] = put(ig[v].ent.data(), 4 * ig[v].ent.size());
+        oIg[v][2] = put(ig[v].slot0.data(), 4 * ig[v].slot0.size());
+        oIg[v][3] = put(ig[v].part.data(), 4 * ig[v].part.size());
+    }
+    std::vector<int32_t> effI((size_t)(nS + 1) / 2 * nM * 4, 0), effX(nM);
+    for (int row = 0; row < nM; ++row) {
+        std::vector<int32_t> hi(nS), lo(nS);
+        effX[row] = int_efficiencies(nS, d->eff + (size_t)rxn[perm[nPlain + row]].row * nS, hi.data(), lo.data());
+        for (int k = 0; k < nS; ++k) {
+            effI[((size_t)(k / 2) * nM + row) * 4 + 2 * (k % 2)] = hi[k];
+            effI[((size_t)(k / 2) * nM + row) * 4 + 2 * (k % 2) + 1] = lo[k];
+        }
+    }
+    const size_t oEffI = put(effI.data(), 4 * effI.size()), oEffX = put(effX.data(), 4 * effX.size());
     // the segmented FP32 gather of the 32-lane isothermal f, where the packed
     // entries apply and its partial sums fit in the FP32 half of the warp's
     // shared words, past C and Omega
@@ -516,6 +567,15 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.seg_slot0 = use_seg ? (const int32_t*)(b + oSegF) : nullptr;
     M.seg_part = use_seg ? (const int32_t*)(b + oSegP) : nullptr;
     M.seg_K = use_seg ? seg.K : 0;
+    for (int v = 0; v < INT_NTAB; ++v) {
+        M.ig[v] = IntDev{};
+        if (!ig_use[v]) continue;
+        M.ig[v] = IntDev{ig[v].nchunk, ig[v].chunk, ig[v].nslots, (const int32_t*)(b + oIg[v][0]),
+                         (const uint32_t*)(b + oIg[v][1]), (const int32_t*)(b + oIg[v][2]),
+                         (const int32_t*)(b + oIg[v][3])};
+    }
+    M.effI = (const int4*)(b + oEffI);
+    M.effX = (const int32_t*)(b + oEffX);
     M.effV64 = (const double*)(b + oEffV64);
     M.effV32 = (const float*)(b + oEffV32);
     M.rxw = (const uint32_t*)(b + oRxw);
@@ -604,9 +664,7 @@ int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, 
     if (!is_device_ptr(ws)) return fail(KIN_EINVAL, "workspace must be device memory");
     // never more lanes (warps in the warp layout) than cells
     int blocks = g.blocks;
-    const int per_block = g.layout == KIN_LAYOUT_WARP
-                              ? g.threads / warp_cell_lanes(o->method, m->nS + o->energy)
-                              : g.threads;
+    const int per_block = g.threads / g.lanes;
     const int64_t want = (total + per_block - 1) / per_block;
     if (want < blocks) blocks = (int)want;
     const int64_t nslots = (int64_t)blocks * g.threads;
@@ -623,6 +681,7 @@ int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, 
                                  g.layout == KIN_LAYOUT_WARP ? 0 : nslots, total);
     P.energy = o->energy;
     P.nV = m->nS + o->energy;
+    P.lanes = g.lanes;
     P.sigma_method = sig;
     P.cell_ev = sig == KIN_SIGMA_POWER ? (double*)(base + w.ev) : nullptr;
     P.queue = (unsigned long long*)(base + w.header);

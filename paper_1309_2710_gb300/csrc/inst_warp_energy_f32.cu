@@ -10,9 +10,9 @@ cudaError_t launch_warp_f32_en_o0(Launch& L, int blocks, int threads, cudaStream
     return warp_launch<float, 0, true>(L, blocks, threads, st);
 }
 
-cudaError_t occ_warp_f32_en_o0(const MechDev& M, int nV, int threads, int* bps)
+cudaError_t occ_warp_f32_en_o0(const MechDev& M, int nV, int lanes, int threads, int* bps)
 {
-    return warp_occ<float, 0, true>(M, nV, KIN_MIXED, threads, bps);
+    return warp_occ<float, 0, true>(M, nV, lanes, KIN_MIXED, threads, bps);
 }
 
 }  // namespace kin

@@ -10,9 +10,9 @@ cudaError_t launch_warp_f64_en_o0(Launch& L, int blocks, int threads, cudaStream
     return warp_launch<double, 0, true>(L, blocks, threads, st);
 }
 
-cudaError_t occ_warp_f64_en_o0(const MechDev& M, int nV, int threads, int* bps)
+cudaError_t occ_warp_f64_en_o0(const MechDev& M, int nV, int lanes, int threads, int* bps)
 {
-    return warp_occ<double, 0, true>(M, nV, KIN_FP64, threads, bps);
+    return warp_occ<double, 0, true>(M, nV, lanes, KIN_FP64, threads, bps);
 }
 
 }  // namespace kin

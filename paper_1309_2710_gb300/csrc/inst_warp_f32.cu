@@ -9,9 +9,9 @@ cudaError_t launch_warp_f32_o0(Launch& L, int blocks, int threads, cudaStream_t 
     return warp_launch<float, 0, false>(L, blocks, threads, st);
 }
 
-cudaError_t occ_warp_f32_o0(const MechDev& M, int nV, int threads, int* bps)
+cudaError_t occ_warp_f32_o0(const MechDev& M, int nV, int lanes, int threads, int* bps)
 {
-    return warp_occ<float, 0, false>(M, nV, KIN_MIXED, threads, bps);
+    return warp_occ<float, 0, false>(M, nV, lanes, KIN_MIXED, threads, bps);
 }
 
 }  // namespace kin

@@ -10,9 +10,9 @@ cudaError_t launch_warp_f64_o1(Launch& L, int blocks, int threads, cudaStream_t 
     return warp_launch<double, 1, false>(L, blocks, threads, st);
 }
 
-cudaError_t occ_warp_f64_o1(const MechDev& M, int nV, int threads, int* bps)
+cudaError_t occ_warp_f64_o1(const MechDev& M, int nV, int lanes, int threads, int* bps)
 {
-    return warp_occ<double, 1, false>(M, nV, KIN_FP64, threads, bps);
+    return warp_occ<double, 1, false>(M, nV, lanes, KIN_FP64, threads, bps);
 }
 
 }  // namespace kin

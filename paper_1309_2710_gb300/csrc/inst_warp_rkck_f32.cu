@@ -11,10 +11,10 @@ cudaError_t launch_warp_rkck_f32(Launch& L, int blocks, int threads, cudaStream_
                     : warp_rkck_launch<float, false>(L, blocks, threads, st);
 }
 
-cudaError_t occ_warp_rkck_f32(const MechDev& M, int nV, int energy, int threads, int* bps)
+cudaError_t occ_warp_rkck_f32(const MechDev& M, int nV, int lanes, int energy, int threads, int* bps)
 {
-    return energy ? warp_rkck_occ<float, true>(M, nV, KIN_MIXED, threads, bps)
-                  : warp_rkck_occ<float, false>(M, nV, KIN_MIXED, threads, bps);
+    return energy ? warp_rkck_occ<float, true>(M, nV, lanes, KIN_MIXED, threads, bps)
+                  : warp_rkck_occ<float, false>(M, nV, lanes, KIN_MIXED, threads, bps);
 }
 
 }  // namespace kin

@@ -11,10 +11,10 @@ cudaError_t launch_warp_rkck_f64(Launch& L, int blocks, int threads, cudaStream_
                     : warp_rkck_launch<double, false>(L, blocks, threads, st);
 }
 
-cudaError_t occ_warp_rkck_f64(const MechDev& M, int nV, int energy, int threads, int* bps)
+cudaError_t occ_warp_rkck_f64(const MechDev& M, int nV, int lanes, int energy, int threads, int* bps)
 {
-    return energy ? warp_rkck_occ<double, true>(M, nV, KIN_FP64, threads, bps)
-                  : warp_rkck_occ<double, false>(M, nV, KIN_FP64, threads, bps);
+    return energy ? warp_rkck_occ<double, true>(M, nV, lanes, KIN_FP64, threads, bps)
+                  : warp_rkck_occ<double, false>(M, nV, lanes, KIN_FP64, threads, bps);
 }
 
 }  // namespace kin

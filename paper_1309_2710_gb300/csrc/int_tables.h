@@ -1,0 +1,128 @@
+// int_tables.h -- host tables of the warp layout's FP64 f in integer arithmetic
+// (plain C++, no CUDA: the library builds them at mechanism upload, and a CPU
+// test compiles this header on its own to check them).
+//
+// Gather (Eq. (E:spec-rate), omega_i = sum_j nu_ij Omega_j): the rates of
+// progress are 128-bit fixed-point words in shared memory, CHUNK reactions at
+// a time, and omega_i is a sum of such words. Species i has two rows, 2 i for
+// its positive and 2 i + 1 for its negative coefficients, so that every entry
+// counts once (a coefficient of 2 is two entries) and the inner loop only adds.
+// Within a chunk the entries, row by row, are cut into G equal runs of
+// K = ceil(n / G), one per lane (G lanes evaluate f for one cell); a lane
+// writes one partial sum per row it touches (a "flush") into consecutive
+// slots, and the species' owner adds the slots of its positive row and
+// subtracts those of its negative one, which follow them. Integer sums are
+// exact, so their order does not matter.
+//
+// An entry is a 32-bit word: the reaction's place in the chunk, and bit 16 set
+// where the lane flushes after it. Padding entries name the place after the
+// last, which holds zero. The
+// entries of a run that belong to one row are ordered so that the eight lanes
+// of a 128-byte wavefront read words in distinct 16-byte banks where they can
+// (bank = place mod 8).
+//
+// Third-body sums (Eq. (E:rxn-rate), [M] = sum_k eff_k C_k): a row's
+// efficiencies as integers eff_k 2^(54 - x), x the exponent of the row's
+// largest (one more above 128 species, which keeps the sums of 30 x 25-bit
+// products below 2^63), cut into 30 high and 25 low bits.
+#pragma once
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <vector>
+
+namespace kin {
+
+constexpr uint32_t INT_POS_MASK = 0xffffu;
+constexpr uint32_t INT_FLUSH = 0x10000u;
+
+struct IntGather {
+    int nchunk = 0, chunk = 0;
+    int nslots = 0;                 // partial-sum slots of the fullest chunk
+    std::vector<int32_t> step0;     // [nchunk + 1] first step of each chunk
+    std::vector<uint32_t> ent;      // [steps][G] entries
+    std::vector<int32_t> slot0;     // [nchunk][G] first slot of each lane
+    std::vector<int32_t> part;      // [nchunk][nS] first slot << 16 | positive slots << 8 | negative slots
+};
+
+// ptr/pos/nu: species-major rows of net coefficients; pos is the reaction's
+// permuted position, nu an integer in -2..2.
+inline IntGather build_int_gather(int nS, int nR, const int* ptr, const int* pos, const double* nu,
+                                  int chunk, int G)
+{
+    IntGather t;
+    t.chunk = chunk;
+    t.nchunk = (nR + chunk - 1) / chunk;
+    t.step0.assign(1, 0);
+    std::vector<std::vector<std::vector<int>>> rows(t.nchunk, std::vector<std::vector<int>>(2 * nS));
+    for (int i = 0; i < nS; ++i)
+        for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
+            const int c = pos[e] / chunk, at = pos[e] % chunk, n = (int)std::abs(nu[e]);
+            for (int k = 0; k < n; ++k) rows[c][2 * i + (nu[e] < 0.0)].push_back(at);
+        }
+    for (int c = 0; c < t.nchunk; ++c) {
+        int n = 0;
+        for (auto& r : rows[c]) n += (int)r.size();
+        const int K = (n + G - 1) / G, base = (int)t.ent.size();
+        t.step0.push_back(t.step0.back() + K);
+        t.ent.resize(base + (size_t)K * G, (uint32_t)chunk);
+        std::vector<int32_t> part(nS, 0), slot0(G, 0);
+        struct Seg { std::vector<int> left; };
+        std::vector<std::vector<Seg>> lane(G);
+        int row = 0, at = 0, slots = 0;
+        for (int l = 0; l < G; ++l) {
+            slot0[l] = slots;
+            for (int room = K; room > 0 && row < 2 * nS;) {
+                const int have = (int)rows[c][row].size() - at;
+                if (have == 0) { ++row; at = 0; continue; }
+                const int take = std::min(room, have);
+                if (part[row / 2] == 0) part[row / 2] = slots << 16;
+                part[row / 2] += row % 2 ? 1 : 1 << 8;
+                ++slots;
+                lane[l].push_back(Seg{{rows[c][row].begin() + at, rows[c][row].begin() + at + take}});
+                at += take;
+                room -= take;
+            }
+        }
+        t.nslots = std::max(t.nslots, slots);
+        std::vector<size_t> cur(G, 0);
+        for (int k = 0; k < K; ++k) {
+            std::vector<int> used(8 * ((G + 7) / 8), 0);
+            for (int l = 0; l < G; ++l) {
+                if (cur[l] >= lane[l].size()) continue;
+                std::vector<int>& L = lane[l][cur[l]].left;
+                int* u = &used[8 * (l / 8)];
+                size_t best = 0;
+                for (size_t q = 1; q < L.size(); ++q)
+                    if (u[L[q] % 8] < u[L[best] % 8]) best = q;
+                const int p = L[best];
+                L.erase(L.begin() + best);
+                u[p % 8]++;
+                t.ent[base + (size_t)k * G + l] = (uint32_t)p | (L.empty() ? INT_FLUSH : 0u);
+                if (L.empty()) ++cur[l];
+            }
+        }
+        t.slot0.insert(t.slot0.end(), slot0.begin(), slot0.end());
+        t.part.insert(t.part.end(), part.begin(), part.end());
+    }
+    return t;
+}
+
+// A row's efficiencies as 55-bit integers: hi (30 bits, signed) and lo (25
+// bits) of round(eff 2^(54 - x)). Returns x.
+inline int int_efficiencies(int nS, const double* eff, int32_t* hi, int32_t* lo)
+{
+    double top = 0.0;
+    for (int k = 0; k < nS; ++k) top = std::max(top, std::fabs(eff[k]));
+    int x = 0;
+    if (top > 0.0) std::frexp(top, &x), --x;
+    if (nS > 128) ++x;
+    for (int k = 0; k < nS; ++k) {
+        const int64_t E = (int64_t)std::nearbyint(std::ldexp(eff[k], 54 - x));
+        hi[k] = (int32_t)(E >> 25);
+        lo[k] = (int32_t)(E & ((1 << 25) - 1));
+    }
+    return x;
+}
+
+}  // namespace kin

@@ -1,0 +1,136 @@
+// intf.cuh -- FP64 arithmetic of the source term on the integer pipes.
+//
+// GB300 runs one FP64 warp instruction per SM sub-partition every 64 cycles
+// (DFMA, DADD, DMUL and 64-bit conversions alike; 628 G FMA/s on the chip),
+// against 2 cycles for a 32 x 32 + 64 bit multiply-add (IMAD.WIDE) and for a
+// 32-bit shift or add. The rates of progress and their sums, nine tenths of
+// an FP64 evaluation of f, therefore run faster as integers than on the FP64
+// pipe, and that pipe is left to the state vectors and the step control,
+// which run beside them:
+//  * a factor (rate constant, concentration) is a 63-bit left-aligned
+//    mantissa and an exponent, exact for every normal double; a product
+//    keeps the top 62 bits of the mantissas' product (three IMAD.WIDE, 6
+//    cycles for a DMUL's 64);
+//  * a rate of progress is placed into a 128-bit fixed-point word whose unit
+//    is 2^-101 or less of the largest rate of the evaluation, so every sum of
+//    rates is exact (four 32-bit adds) but for the words' own last bits;
+//  * a third-body sum multiplies 55-bit integer efficiencies by the
+//    concentrations as 55-bit fractions of the total.
+// Every product, sum and third-body sum is at least as accurate as its FP64
+// form: 2^-57 per product against 2^-53, no rounding in the sums. States
+// outside the range of the fixed-point forms (not finite, or a concentration
+// below -2^-9 of the total) take a plain FP64 evaluation instead.
+#pragma once
+#ifndef __CUDACC_RTC__
+#include <cstdint>
+#endif
+
+namespace kin {
+
+typedef unsigned long long im_u64;
+
+// Exponent words: bit 31 the sign, the rest the exponent biased by 1023 as in
+// the double; the value is mantissa * 2^(e - IM_BIAS).
+constexpr int IM_BIAS = 1023 + 62;
+
+// Top 64 of the 128 bits of a * b, less at most 3 units; a, b < 2^63.
+__device__ __forceinline__ im_u64 im_mul(im_u64 a, im_u64 b)
+{
+    const uint32_t a1 = (uint32_t)(a >> 32), a0 = (uint32_t)a, b1 = (uint32_t)(b >> 32), b0 = (uint32_t)b;
+    im_u64 t = (im_u64)a1 * b0;
+    t = (im_u64)a0 * b1 + t;
+    return (im_u64)a1 * b1 + (t >> 32);
+}
+
+// Mantissa and exponent word of a double (a denormal becomes zero).
+__device__ __forceinline__ void im_split(double v, im_u64& m, uint32_t& e)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t x = (hi >> 20) & 0x7ffu;
+    e = x | (hi & 0x80000000u);
+    const im_u64 n = ((im_u64)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    m = x ? n << 10 : 0ull;
+}
+
+// The same of a positive double; zero and denormals read as about 2^-1023.
+__device__ __forceinline__ void im_split_k(double v, im_u64& m, uint32_t& e)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    e = hi >> 20;
+    m = (((im_u64)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 10;
+}
+
+__device__ __forceinline__ bool im_finite_k(double v) { return ((uint32_t)__double2hiint(v) >> 20) < 0x7ffu; }
+__device__ __forceinline__ bool im_finite_k(float v) { return (__float_as_uint(v) >> 23) < 0xffu; }
+
+// 64-bit shifts by any unsigned amount (64 and more give zero).
+__device__ __forceinline__ im_u64 im_shl(im_u64 v, uint32_t n)
+{
+    im_u64 r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+__device__ __forceinline__ im_u64 im_shr(im_u64 v, uint32_t n)
+{
+    im_u64 r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+
+struct im_u128 {
+    im_u64 lo, hi;
+};
+
+__device__ __forceinline__ void im_add(im_u128& a, im_u64 lo, im_u64 hi)
+{
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(lo), "l"(hi));
+}
+__device__ __forceinline__ void im_sub(im_u128& a, im_u64 lo, im_u64 hi)
+{
+    asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(lo), "l"(hi));
+}
+
+// Q * 2^L as a 128-bit word, Q < 2^61, L <= 63; bits below the unit drop.
+__device__ __forceinline__ im_u128 im_place(im_u64 Q, int L)
+{
+    im_u128 r;
+    r.lo = im_shl(Q, (uint32_t)L) | im_shr(Q, (uint32_t)-L);
+    r.hi = im_shr(Q, (uint32_t)(64 - L));
+    return r;
+}
+
+// a * 2^x as a double, rounded once (a signed).
+__device__ __forceinline__ double im_double(im_u128 a, int x)
+{
+    const bool neg = (long long)a.hi < 0;
+    if (neg) {
+        im_u128 z{0ull, 0ull};
+        im_sub(z, a.lo, a.hi);
+        a = z;
+    }
+    if (a.hi == 0ull) {  // far below the largest rate: 64 bits up
+        a.hi = a.lo;
+        a.lo = 0ull;
+        x -= 64;
+        if (a.hi == 0ull) return 0.0;
+    }
+    const int z = __clzll((long long)a.hi);
+    im_u64 v = a.hi;
+    if (z) v = (v << z) | (a.lo >> (64 - z));
+    const double d = (double)v;  // [2^63, 2^64]
+    const int n = (__double2hiint(d) >> 20) + x + 64 - z;
+    if (n <= 0) return 0.0;
+    const int hi = n >= 0x7ff ? 0x7ff00000 : ((__double2hiint(d) & 0xfffff) | (n << 20));
+    const double r = __hiloint2double(hi, n >= 0x7ff ? 0 : __double2loint(d));
+    return neg ? -r : r;
+}
+
+// Bits a word of the largest rate (e = the evaluation's scale) is shifted up:
+// Q < 2^61, so it stays below 2^(61 + 43 + 8) where the scale is 8 octaves too
+// low, which leaves 15 bits for a row's entries and the sign.
+constexpr int IM_UP = 43, IM_GUARD = 8, IM_SLACK = 16;
+
+// Exponent that stands for a rate that is not finite.
+constexpr int IM_OUT = 1 << 20;
+
+}  // namespace kin

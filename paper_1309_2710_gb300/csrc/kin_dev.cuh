@@ -40,6 +40,18 @@ struct CsrW64 {
     int32_t pos, pad;
 };
 
+// Tables of the FP64 f in integer arithmetic (int_tables.h).
+struct IntDev {
+    int nchunk, chunk, nslots;
+    const int32_t* step0;   // [nchunk + 1]
+    const uint32_t* ent;    // [steps][G]
+    const int32_t* slot0;   // [nchunk][G]
+    const int32_t* part;    // [nchunk][nS]
+};
+// One set per number of lanes that share a cell (16: states of at most 16
+// components; 64 and 128: more than 32 and 64).
+enum IntTab : int { INT_G16 = 0, INT_G32, INT_G64, INT_G128, INT_NTAB };
+
 // Species slots of 32 in the warp layout's ELL gather tables.
 constexpr int ELL_SLOTS = (KIN_MAX_SPECIES + 31) / 32;
 
@@ -74,6 +86,9 @@ struct MechDev {
     const int32_t* seg_slot0;  // [32] first partial slot of each lane
     const int32_t* seg_part;   // [nS] first slot << 8 | slot count; -1: empty row
     int seg_K;
+    IntDev ig[INT_NTAB];
+    const int4* effI;      // [(nS + 1) / 2][nM] integer efficiencies {hi, lo} of two species
+    const int32_t* effX;   // [nM] their exponents
     // efficiencies by non-plain reaction in permutation order (row), species
     // in 16-byte groups: [k / V][row][k % V], V = 2 (FP64) or 4 (FP32), the
     // last group zero-padded
@@ -115,6 +130,7 @@ struct Launch {
     int method, precision, max_steps, n_inst, sigma_method;
     int energy;  // 1: T is state component nS (Eq. (E:energy))
     int nV;      // state length: nS + energy
+    int lanes;   // warp layout: lanes per cell
     int64_t nslots;                 // lanes of the persistent grid
     int64_t total;                  // cells over all instances
     unsigned long long* queue;      // next position in `order`
@@ -180,31 +196,22 @@ cudaError_t launch_warp_f64_o0(Launch& L, int blocks, int threads, cudaStream_t 
 cudaError_t launch_warp_f64_o1(Launch& L, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_warp_f32_o0(Launch& L, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_warp_f32_o1(Launch& L, int blocks, int threads, cudaStream_t st);
-cudaError_t occ_warp_f64_o0(const MechDev& M, int nV, int threads, int* bps);
-cudaError_t occ_warp_f64_o1(const MechDev& M, int nV, int threads, int* bps);
-cudaError_t occ_warp_f32_o0(const MechDev& M, int nV, int threads, int* bps);
-cudaError_t occ_warp_f32_o1(const MechDev& M, int nV, int threads, int* bps);
+cudaError_t occ_warp_f64_o0(const MechDev& M, int nV, int lanes, int threads, int* bps);
+cudaError_t occ_warp_f64_o1(const MechDev& M, int nV, int lanes, int threads, int* bps);
+cudaError_t occ_warp_f32_o0(const MechDev& M, int nV, int lanes, int threads, int* bps);
+cudaError_t occ_warp_f32_o1(const MechDev& M, int nV, int lanes, int threads, int* bps);
 cudaError_t launch_warp_f64_en_o0(Launch& L, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_warp_f64_en_o1(Launch& L, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_warp_f32_en_o0(Launch& L, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_warp_f32_en_o1(Launch& L, int blocks, int threads, cudaStream_t st);
-cudaError_t occ_warp_f64_en_o0(const MechDev& M, int nV, int threads, int* bps);
-cudaError_t occ_warp_f64_en_o1(const MechDev& M, int nV, int threads, int* bps);
-cudaError_t occ_warp_f32_en_o0(const MechDev& M, int nV, int threads, int* bps);
-cudaError_t occ_warp_f32_en_o1(const MechDev& M, int nV, int threads, int* bps);
+cudaError_t occ_warp_f64_en_o0(const MechDev& M, int nV, int lanes, int threads, int* bps);
+cudaError_t occ_warp_f64_en_o1(const MechDev& M, int nV, int lanes, int threads, int* bps);
+cudaError_t occ_warp_f32_en_o0(const MechDev& M, int nV, int lanes, int threads, int* bps);
+cudaError_t occ_warp_f32_en_o1(const MechDev& M, int nV, int lanes, int threads, int* bps);
 cudaError_t launch_warp_rkck_f64(Launch& L, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_warp_rkck_f32(Launch& L, int blocks, int threads, cudaStream_t st);
-cudaError_t occ_warp_rkck_f64(const MechDev& M, int nV, int energy, int threads, int* bps);
-cudaError_t occ_warp_rkck_f32(const MechDev& M, int nV, int energy, int threads, int* bps);
-// Dynamic shared memory of a 32-lane warp's worth of cell groups per block of
-// `threads` (RKC: one cell per warp; RKCK with 16-lane groups: multiply by 2).
-size_t warp_smem(const MechDev& M, int precision, int energy, int threads);
-
-// Lanes that integrate one cell in the warp-per-cell layout: a whole warp,
-// or half of one (two cells per warp) for RKCK on states of at most 16
-// components.
-inline int warp_cell_lanes(int method, int nV) { return method == KIN_RKCK && nV <= 16 ? 16 : 32; }
-
+cudaError_t occ_warp_rkck_f64(const MechDev& M, int nV, int lanes, int energy, int threads, int* bps);
+cudaError_t occ_warp_rkck_f32(const MechDev& M, int nV, int lanes, int energy, int threads, int* bps);
 // Record `code` and a printf-style message as the calling thread's last
 // error (kin_last_error); returns `code`.
 int set_last_error(int code, const char* fmt, ...);

@@ -4,14 +4,16 @@
 // With one lane per cell, every lane keeps its own concentrations, rates of
 // progress and rate constants: ~(2 n_R + n_S) words per cell, which for
 // hundreds of reactions spills out of L1/L2 and turns every f evaluation into
-// a stream from HBM. Here one warp integrates one cell:
-//  * the 32 lanes split the reactions (rates of progress, rounds of 32) and
-//    the species (state vectors in registers: species l + 32 r in slot r of
-//    lane l; stoichiometric gather over the species-major CSR);
-//  * the cell's concentrations and rates of progress live in shared memory
-//    (n_S + n_R words per warp); its rate constants, computed once per call
-//    since T is fixed, live in the workspace cell-major and are read
-//    coalesced (the working set of the resident cells stays in L2);
+// a stream from HBM. Here a group of G lanes integrates one cell (a warp; in
+// isothermal FP64 half a warp to four warps, cell_lanes in abi.cu):
+//  * the lanes split the reactions (rates of progress, rounds of G) and
+//    the species (state vectors in registers: species l + G r in slot r of
+//    lane l);
+//  * f in FP64 runs on the integer pipes (warp_int.cuh); in mixed precision and
+//    with the energy equation its concentrations and rates of progress live in
+//    shared memory (n_S + n_R words per warp). A cell's rate constants, computed
+//    once per call since T is fixed, live in the workspace cell-major and are
+//    read coalesced (the working set of the resident cells stays in L2);
 //  * reactions are visited in a fixed permutation (plain, then third-body,
 //    then falloff) so that a round of 32 lanes mixes the dense efficiency dot
 //    products with plain reactions at most once; the efficiency rows are
@@ -24,43 +26,12 @@
 // The method, its decisions and the statistics are those of the lane-per-cell
 // kernel (Section 2.3 and the readings listed with it).
 #pragma once
+#include "int_tables.h"
 #include "kernels.cuh"
 #include "seg_tables.h"
+#include "warp_int.cuh"
 
 namespace kin {
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Butterfly sum over a group of G lanes (a whole warp, or a 16-lane half
-// that owns one cell); mask names the group's lanes.
-template <int G, typename T>
-__device__ __forceinline__ T group_sum(T v, unsigned mask)
-{
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-    return v;
-}
-
-template <int G>
-__device__ __forceinline__ double group_max(double v, unsigned mask)
-{
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(mask, v, o));
-    return v;
-}
-
-__device__ __forceinline__ double warp_max(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
 
 template <typename R>
 struct EllT;
@@ -122,12 +93,27 @@ __device__ __forceinline__ double eff_dot<double>(const MechDev& M, int row, con
     return m0 + m1;
 }
 
-// Shared words per warp: C [nS] and Omega [nR], padded to 4, sized for FP64
-// (the mixed-precision path evaluates f in FP32 for its RK stages and in FP64
-// for its spectral-radius estimates, over the same words).
+// The FP64 f's tables for groups of G lanes.
+template <int G>
+__host__ __device__ __forceinline__ const IntDev& int_tab(const MechDev& M)
+{
+    return M.ig[G == 16 ? INT_G16 : G == 32 ? INT_G32 : G == 64 ? INT_G64 : INT_G128];
+}
+
+// Shared FP64 words of C [nS] and Omega [nR] in the energy and FP32 forms of
+// f, padded to 4.
 __host__ __device__ __forceinline__ int warp_smem_elems(const MechDev& M)
 {
     return (M.nS + M.nR + 3) & ~3;
+}
+
+// Shared FP64 words of a group's f: the integer arrays of the FP64 f, or C and
+// Omega (the mixed-precision path evaluates f in FP32 for its RK stages and in
+// FP64 for its spectral-radius estimates, over the same words).
+template <typename R, bool EN, int G>
+__host__ __device__ __forceinline__ int warp_f_words(const MechDev& M)
+{
+    return EN || sizeof(R) == 4 ? warp_smem_elems(M) : int_smem_words(M, int_tab<G>(M));
 }
 
 // The cell's rate constants in shared memory too: f reads every k_j once per
@@ -148,15 +134,18 @@ __host__ __device__ __forceinline__ int warp_k_words(const MechDev& M)
     return (warp_smem_elems(M) + kw) * 8 <= WARP_K_SMEM_MAX_BYTES ? kw : 0;
 }
 
-// Shared FP64 words per cell group: C and Omega, then the staged k (if any).
-template <typename R, bool EN>
+// Shared FP64 words per cell group: f's, the staged k (if any), the reductions'.
+template <typename R, int NR, bool EN, int G>
 __host__ __device__ __forceinline__ int warp_group_words(const MechDev& M)
 {
-    return warp_smem_elems(M) + warp_k_words<R, EN>(M);
+    return (warp_f_words<R, EN, G>(M) + warp_k_words<R, EN>(M) + 2 * group_set_words<NR, G>() + 1) & ~1;
 }
 
-// f for the warp's cell (Eqs. (E:mass), (E:spec-rate), (E:rxn-rate)) in
-// arithmetic type R. Kc are the cell's rate constants (stored as KT) in
+// f for the mixed-precision path's cell (Eqs. (E:mass), (E:spec-rate),
+// (E:rxn-rate)) in arithmetic type R: FP32 for the RK stages, FP64 for the
+// spectral-radius estimates. (The FP64 path's f is warp_feval_int. The mixed
+// path keeps this one for both: its FP32 f turns any change of rounding in an
+// estimate into differences of 3e-8 in the result.) Kc are the cell's rate constants (stored as KT) in
 // reaction-permutation order followed by k0/kinf per falloff ordinal (written
 // earlier in the same pre-pass kernel, so not read through the read-only
 // cache); C and OM are the warp's shared arrays. Ctot and invCtot (the total
@@ -394,7 +383,7 @@ __device__ __forceinline__ double reg_get(const double (&v)[NR], int r)
     return o;
 }
 
-template <typename R, int NR, bool EN>
+template <typename R, int NR, bool EN, int G>
 struct WarpRKC {
     const Launch& L;
     const MechDev& M;
@@ -402,58 +391,93 @@ struct WarpRKC {
     R* OM;
     double* C64;   // the same shared words as C and OM, for the FP64 evaluations
     double* OM64;
-    R* Ks;         // the warp's staged rate constants, or null
+    R* Ks;         // the group's staged rate constants, or null
     const R* Kc;
     int lane, nV;  // nV: state length, nS + 1 with the energy equation
+    Group<G> grp;
+    unsigned mask; // the group's lanes in this warp
+    int scale;     // of the integer FP64 f, kept from one evaluation to the next
+    bool kfin;     // the cell's rate constants are finite
     double Ctot, invCtot, atol, rtol, p;
     R CtotR, invCtotR;   // the same in the rate type
     int nfe, nsig, nfs;  // f evaluations, sigma estimates, f evaluations inside them
     double y[NR], f0[NR], w1[NR], w2[NR], fx[NR], x[NR], ev[NR];
 
-    __device__ explicit WarpRKC(const Launch& l) : L(l), M(l.M), Kc(nullptr), lane(threadIdx.x & 31), nV(l.nV)
+    __device__ explicit WarpRKC(const Launch& l)
+        : L(l), M(l.M), Kc(nullptr), lane(threadIdx.x & (G - 1)), nV(l.nV), grp(nullptr, group_set_words<NR, G>()), mask(group_mask<G>()), scale(0), kfin(true)
     {
-        C64 = reinterpret_cast<double*>(kin_smem) + (size_t)(threadIdx.x >> 5) * warp_group_words<R, EN>(M);
+        C64 = reinterpret_cast<double*>(kin_smem) + (size_t)(threadIdx.x / G) * warp_group_words<R, NR, EN, G>(M);
+        grp.red = C64 + warp_f_words<R, EN, G>(M) + warp_k_words<R, EN>(M);
         OM64 = C64 + M.nS;
         C = reinterpret_cast<R*>(C64);
         OM = C + M.nS;
-        Ks = warp_k_words<R, EN>(M) ? reinterpret_cast<R*>(C64 + warp_smem_elems(M)) : nullptr;
+        Ks = warp_k_words<R, EN>(M) ? reinterpret_cast<R*>(C64 + warp_f_words<R, EN, G>(M)) : nullptr;
     }
 
-    __device__ __forceinline__ bool valid(int r) const { return lane + 32 * r < nV; }
+    __device__ __forceinline__ bool valid(int r) const { return lane + G * r < nV; }
+
+    // a * b + c and a * b of the state vectors. In the FP64 path the fused and
+    // the separate operations are named, so that every group size rounds alike;
+    // the mixed path leaves the choice to the compiler.
+    __device__ __forceinline__ static double mul_add(double a, double b, double c)
+    {
+        if constexpr (sizeof(R) == 8) return fma(a, b, c);
+        else return c + a * b;
+    }
+    __device__ __forceinline__ static double mul(double a, double b)
+    {
+        if constexpr (sizeof(R) == 8) return __dmul_rn(a, b);
+        else return a * b;
+    }
 
     __device__ __forceinline__ void f(const double (&in)[NR], double (&o)[NR])
     {
-        if constexpr (EN) warp_feval_energy<R, NR>(M, p, C, OM, in, o, lane);
-        else warp_feval<R, R, NR>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane);
+        if constexpr (EN) warp_feval_energy<R, NR, G>(M, p, C, OM, in, o, lane, mask);
+        else if constexpr (sizeof(R) == 4) warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
+        else f64(in, o);
         nfe++;
+    }
+
+    // The isothermal f of the FP64 path.
+    __device__ __forceinline__ void f64(const double (&in)[NR], double (&o)[NR])
+    {
+        const IntDev& I = int_tab<G>(M);
+        warp_feval_int<NR, G>(M, I, IntSmem(M, I, C64), Kc, kfin, Ctot, invCtot, scale, in, o, lane, grp);
     }
 
     // f in FP64 for the spectral-radius estimates (FP32 rounding noise in
     // f(y + v) - f(y) would swamp the difference; see SIG_SQRT_U).
     __device__ __forceinline__ void fs(const double (&in)[NR], double (&o)[NR])
     {
-        if constexpr (EN)
-            warp_feval_energy<double, NR>(M, p, C64, OM64, in, o, lane);
+        if constexpr (EN) warp_feval_energy<double, NR, G>(M, p, C64, OM64, in, o, lane, mask);
         else if constexpr (sizeof(R) == 4)
-            warp_feval<double, R, NR>(M, Kc, C64, OM64, Ctot, invCtot, in, o, lane);
-        else
-            warp_feval<double, double, NR>(M, Kc, C, OM, Ctot, invCtot, in, o, lane);
+            warp_feval<double, R, NR, G>(M, Kc, C64, OM64, Ctot, invCtot, in, o, lane, mask);
+        else f64(in, o);
         nfe++;
         nfs++;
     }
 
     // Weighted RMS norm, Eq. (E:rmsE), of d with T_i = atol + rtol max(|a_i|, |b_i|).
-    __device__ double rms(const double (&d)[NR], const double (&a)[NR], const double (&b)[NR]) const
+    __device__ double rms(const double (&d)[NR], const double (&a)[NR], const double (&b)[NR])
     {
         double acc = 0.0;
+        if constexpr (sizeof(R) == 8) {
+            double q[NR];
 #pragma unroll
-        for (int r = 0; r < NR; ++r)
-            if (valid(r)) {
-                const double sc = atol + rtol * fmax(fabs(a[r]), fabs(b[r]));
-                const double q = ddiv(d[r], sc);
-                acc += q * q;
-            }
-        return dsqrt(ddiv(warp_sum(acc), (double)nV));
+            for (int r = 0; r < NR; ++r)
+                q[r] = valid(r) ? ddiv(d[r], fma(rtol, fmax(fabs(a[r]), fabs(b[r])), atol)) : 0.0;
+            acc = grp.sum_sq(q);
+        } else {
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                if (valid(r)) {
+                    const double sc = atol + rtol * fmax(fabs(a[r]), fabs(b[r]));
+                    const double q = ddiv(d[r], sc);
+                    acc += q * q;
+                }
+            acc = group_sum<G>(acc, mask);
+        }
+        return dsqrt(ddiv(acc, (double)nV));
     }
 
     // FP64 f(y), the base of the spectral-radius differences: f0 in the FP64
@@ -469,13 +493,20 @@ struct WarpRKC {
     __device__ double power_setup()
     {
         double yn = 0.0, vn = 0.0;
+        if constexpr (sizeof(R) == 8) {
+            yn = grp.sum_sq(y);
+            vn = grp.sum_sq(ev);
+        } else {
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            yn += y[r] * y[r];
-            vn += ev[r] * ev[r];
+            for (int r = 0; r < NR; ++r) {
+                yn += y[r] * y[r];
+                vn += ev[r] * ev[r];
+            }
+            yn = group_sum<G>(yn, mask);
+            vn = group_sum<G>(vn, mask);
         }
-        yn = dsqrt(warp_sum(yn));
-        vn = dsqrt(warp_sum(vn));
+        yn = dsqrt(yn);
+        vn = dsqrt(vn);
         const double dyn = yn > 0.0 ? SIG_SQRT_U * yn : SIG_SQRT_U;
         if (!(vn > 0.0) || !isfinite(vn)) {
 #pragma unroll
@@ -484,7 +515,7 @@ struct WarpRKC {
         }
         const double sc0 = ddiv(dyn, vn);
 #pragma unroll
-        for (int r = 0; r < NR; ++r) ev[r] = ev[r] * sc0;
+        for (int r = 0; r < NR; ++r) ev[r] = mul(ev[r], sc0);
         return dyn;
     }
 
@@ -518,8 +549,8 @@ struct WarpRKC {
 #pragma unroll
                 for (int r = 0; r < NR; ++r) x[r] = y[r] + ev[r];
             } else {  // Gershgorin column k
-                const int kr = k >> 5, kl = k & 31;
-                const double yk = __shfl_sync(0xffffffffu, reg_get(y, kr), kl);
+                const int kr = k / G, kl = k % G;
+                const double yk = grp.from(reg_get(y, kr), kl);
                 eps = SIG_SQRT_U * fmax(fabs(yk), atol);
 #pragma unroll
                 for (int r = 0; r < NR; ++r) x[r] = (r == kr && lane == kl) ? yk + eps : y[r];
@@ -536,17 +567,24 @@ struct WarpRKC {
             }
             if (pw) {
                 double wn = 0.0;
+                if constexpr (sizeof(R) == 8) {
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    fx[r] = fx[r] - sig_base(r);
-                    wn += fx[r] * fx[r];
+                    for (int r = 0; r < NR; ++r) fx[r] = fx[r] - sig_base(r);
+                    wn = grp.sum_sq(fx);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        fx[r] = fx[r] - sig_base(r);
+                        wn += fx[r] * fx[r];
+                    }
+                    wn = group_sum<G>(wn, mask);
                 }
-                wn = dsqrt(warp_sum(wn));
+                wn = dsqrt(wn);
                 sig = ddiv(wn, dyn);
                 if (!(wn > 0.0) || !isfinite(wn)) break;
                 const double sc = ddiv(dyn, wn);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) ev[r] = fx[r] * sc;
+                for (int r = 0; r < NR; ++r) ev[r] = mul(fx[r], sc);
                 if (k >= 1 && fabs(sig - prev) <= 0.01 * sig) break;
                 prev = sig;
                 if (k + 1 >= 20) break;
@@ -559,7 +597,7 @@ struct WarpRKC {
                     double m = 0.0;
 #pragma unroll
                     for (int r = 0; r < NR; ++r) m = fmax(m, rs[r]);
-                    return warp_max(m);
+                    return grp.max(m);
                 }
             }
         }
@@ -619,7 +657,7 @@ struct WarpRKC {
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 w2[r] = y[r];
-                w1[r] = y[r] + m1 * f0[r];
+                w1[r] = mul_add(m1, f0[r], y[r]);
             }
             for (int j = 2;; ++j) {
                 f(w1, fx);  // f(w_{j-1}); after the last stage, f(w_s)
@@ -628,24 +666,40 @@ struct WarpRKC {
                 const double mu = c[0], nu = c[1], mt = c[2] * hh, gt = c[3] * hh, c0 = c[4];
 #pragma unroll
                 for (int r = 0; r < NR; ++r) {
-                    const double wn = c0 * y[r] + mu * w1[r] + nu * w2[r] + mt * fx[r] + gt * f0[r];
+                    double wn;
+                    if constexpr (sizeof(R) == 8)
+                        wn = fma(gt, f0[r], fma(mt, fx[r], fma(nu, w2[r], fma(mu, w1[r], __dmul_rn(c0, y[r])))));
+                    else
+                        wn = c0 * y[r] + mu * w1[r] + nu * w2[r] + mt * fx[r] + gt * f0[r];
                     w2[r] = w1[r];
                     w1[r] = wn;
                 }
             }
             attempts++;
             double acc = 0.0;
+            if constexpr (sizeof(R) == 8) {
+                double q[NR];
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
-                if (valid(r)) {
-                    const double d = 0.8 * (y[r] - w1[r]) + 0.4 * hh * (f0[r] + fx[r]);
-                    const double sc = atol + rtol * fmax(fabs(y[r]), fabs(w1[r]));
-                    const double q = d * rcp_newton(sc);
-                    acc += q * q;
+                for (int r = 0; r < NR; ++r) {
+                    const double d = fma(0.8, y[r] - w1[r], __dmul_rn(0.4 * hh, f0[r] + fx[r]));
+                    const double sc = fma(rtol, fmax(fabs(y[r]), fabs(w1[r])), atol);
+                    q[r] = valid(r) ? __dmul_rn(d, rcp_newton(sc)) : 0.0;
                 }
+                acc = grp.sum_sq(q);
+            } else {
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (valid(r)) {
+                        const double d = 0.8 * (y[r] - w1[r]) + 0.4 * hh * (f0[r] + fx[r]);
+                        const double sc = atol + rtol * fmax(fabs(y[r]), fabs(w1[r]));
+                        const double q = d * rcp_newton(sc);
+                        acc += q * q;
+                    }
+                acc = group_sum<G>(acc, mask);
+            }
             // x = ||Delta||^2; z = x^(-1/6) = err^(-1/3) (see the lane kernel)
             // (one evaluation of the power serves both branches)
-            const double xe = warp_sum(acc) * invN;
+            const double xe = acc * invN;
             // (the mixed-precision path keeps the FP32 power, within 4 ulp: a
             // step-size factor, with the FP32 rates' precision)
             double z = 0.0;
@@ -710,17 +764,17 @@ struct WarpBounds {
     static constexpr int min_blocks = NR == 8 ? (OCC ? 2 : 1) : (OCC && NR <= 2 ? (EN ? 3 : 5) : 2);
 };
 
-// Pre-pass, one warp per cell (grid-stride over cells): the cell's rate
+// Pre-pass, one group of G lanes per cell (grid-stride over cells): the cell's rate
 // constants (stored cell-major for the main kernel), f(y0), sigma and the
 // initial step h1 (Section 2.3).
-template <typename R, int NR, int OCC, bool EN>
+template <typename R, int NR, int OCC, bool EN, int G>
 __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp_init_kernel(const __grid_constant__ Launch L)
 {
-    WarpRKC<R, NR, EN> W(L);
+    WarpRKC<R, NR, EN, G> W(L);
     const MechDev& M = L.M;
     const int lane = W.lane, nK = M.nR + M.nFO, nS = M.nS, nV = L.nV;
-    const int64_t nwarps = L.nslots >> 5;
-    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < L.total; g += nwarps) {
+    const int64_t ngroups = L.nslots / G;
+    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; g < L.total; g += ngroups) {
         const int ii = find_inst(L, g);
         const InstDev& I = L.inst[ii];
         const int64_t c = g - L.start[ii];
@@ -742,33 +796,38 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
             R* kc = reinterpret_cast<R*>(L.cell_k) + g * nK;
             R* ks = W.Ks ? W.Ks : kc;
             const double lnT = log(T), invT = ddiv(1.0, T);
-            for (int q = lane; q < M.nR; q += 32) {
+            bool kfin = true;
+            for (int q = lane; q < M.nR; q += G) {
                 const int j = M.rxn_perm[q];
                 const double a = M.lnA[j] + M.beta[j] * lnT - M.EaR[j] * invT;
                 const R k = Tab<R>::ex(a);
                 kc[q] = k;
                 ks[q] = k;
+                if (sizeof(R) == 8) kfin &= im_finite_k(k);
                 const int fo = M.rxnp[q].fo;
                 if (fo >= 0) {
                     const double a0 = M.lnA0[j] + M.beta0[j] * lnT - M.Ea0R[j] * invT;
                     const R k0 = Tab<R>::ex(a0 - a);
                     kc[M.nR + fo] = k0;
                     ks[M.nR + fo] = k0;
+                    if (sizeof(R) == 8) kfin &= im_finite_k(k0);
                 }
             }
-            __syncwarp();
+            W.grp.sync();
             W.Kc = ks;
+            if (sizeof(R) == 8) W.kfin = W.grp.all(kfin);
+            W.scale = 0;
         }
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-            const int i = lane + 32 * r;
+            const int i = lane + G * r;
             W.y[r] = i < nS ? I.Y[(int64_t)i * I.ldY + c] : (i == nS && EN ? T : 0.0);
         }
         W.f(W.y, W.f0);
         bool fin = true;
 #pragma unroll
         for (int r = 0; r < NR; ++r) fin &= isfinite(W.f0[r]);
-        fin = __all_sync(0xffffffffu, fin);
+        fin = W.grp.all(fin);
         uint8_t st = fin ? 0 : KIN_CELL_NONFINITE;
         double sig = 0.0, h = I.dt;
         if (fin) {
@@ -779,7 +838,7 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
                 double h0 = sig > 0.0 ? ddiv(1.0, sig) : I.dt;
                 if (h0 > I.dt) h0 = I.dt;
 #pragma unroll
-                for (int r = 0; r < NR; ++r) W.x[r] = W.y[r] + h0 * W.f0[r];
+                for (int r = 0; r < NR; ++r) W.x[r] = W.mul_add(h0, W.f0[r], W.y[r]);
                 W.f(W.x, W.fx);
 #pragma unroll
                 for (int r = 0; r < NR; ++r) W.x[r] = h0 * (W.fx[r] - W.f0[r]);  // Delta_0
@@ -793,8 +852,8 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
 #pragma unroll
         for (int r = 0; r < NR; ++r)
             if (W.valid(r)) {
-                L.cell_f0[g * nV + lane + 32 * r] = W.f0[r];
-                if (L.cell_ev) L.cell_ev[g * nV + lane + 32 * r] = W.ev[r];
+                L.cell_f0[g * nV + lane + G * r] = W.f0[r];
+                if (L.cell_ev) L.cell_ev[g * nV + lane + G * r] = W.ev[r];
             }
         if (lane == 0) {
             L.cell_sig[g] = sig;
@@ -808,16 +867,16 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
 
 // Persistent main kernel: each warp takes cells from the queue in the
 // longest-first order and integrates them one after another.
-template <typename R, int NR, int OCC, bool EN>
+template <typename R, int NR, int OCC, bool EN, int G>
 __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp_integrate_kernel(const __grid_constant__ Launch L)
 {
-    WarpRKC<R, NR, EN> W(L);
+    WarpRKC<R, NR, EN, G> W(L);
     const MechDev& M = L.M;
     const int lane = W.lane, nK = M.nR + M.nFO, nS = M.nS, nV = L.nV;
     for (;;) {
         unsigned long long q = 0;
         if (lane == 0) q = atomicAdd(L.queue, 1ull);
-        q = __shfl_sync(0xffffffffu, q, 0);
+        q = W.grp.from(q, 0);
         if (q >= (unsigned long long)L.total) return;
         const int64_t g = L.order[q];
         const int ii = find_inst(L, g);
@@ -843,17 +902,21 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
                 W.Kc = nullptr;
             } else {
                 const R* kg = reinterpret_cast<const R*>(L.cell_k) + g * nK;
-                if (W.Ks) {  // stage the cell's k (the last f of the previous cell ended in a sync)
-                    for (int q = lane; q < nK; q += 32) W.Ks[q] = kg[q];
-                    __syncwarp();
-                    W.Kc = W.Ks;
-                } else {
-                    W.Kc = kg;
-                }
+                bool kfin = true;
+                if (W.Ks || sizeof(R) == 8)
+                    for (int q = lane; q < nK; q += G) {
+                        const R k = kg[q];
+                        if (sizeof(R) == 8) kfin &= im_finite_k(k);
+                        if (W.Ks) W.Ks[q] = k;  // staged (the last f of the previous cell ended in a sync)
+                    }
+                if (sizeof(R) == 8) W.kfin = W.grp.all(kfin);
+                W.scale = 0;
+                if (W.Ks) W.grp.sync();
+                W.Kc = W.Ks ? W.Ks : kg;
             }
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
-                const int i = lane + 32 * r;
+                const int i = lane + G * r;
                 const bool v = i < nV;
                 W.y[r] = i < nS ? I.Y[(int64_t)i * I.ldY + c] : (v ? T : 0.0);
                 W.f0[r] = v ? L.cell_f0[g * nV + i] : 0.0;
@@ -862,7 +925,7 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
             code = W.run(I.dt, L.cell_sig[g], L.cell_h[g], nacc, nrej);
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
-                const int i = lane + 32 * r;
+                const int i = lane + G * r;
                 if (i < nS) I.Y[(int64_t)i * I.ldY + c] = W.y[r];
                 else if (i == nS && EN) I.T[c] = W.y[r];
             }
@@ -879,12 +942,6 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
             }
         }
     }
-}
-
-template <typename R, bool EN>
-inline size_t warp_smem_bytes(const MechDev& M, int threads)
-{
-    return (size_t)warp_group_words<R, EN>(M) * (threads / 32) * 8;
 }
 
 // ---------------------------------------------------- RKCK, warp per cell --
@@ -906,8 +963,12 @@ struct WarpRKCK {
     R* OM;
     R* Ks;  // the group's staged rate constants, or null
     const R* Kc;
+    double* base;   // the group's shared words
     int lane, nV;
+    Group<G> grp;
     unsigned mask;  // the group's lanes
+    int scale;      // of the integer FP64 f, kept from one evaluation to the next
+    bool kfin;      // the cell's rate constants are finite
     double Ctot, invCtot, atol, rtol, p;
     R CtotR, invCtotR;  // the same in the rate type
     int nfe;
@@ -915,12 +976,12 @@ struct WarpRKCK {
 
     __device__ explicit WarpRKCK(const Launch& l)
         : L(l), M(l.M), Kc(nullptr), lane(threadIdx.x & (G - 1)), nV(l.nV),
-          mask(G == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16)))
+          grp(nullptr, group_set_words<NR, G>()), mask(group_mask<G>()), scale(0), kfin(true)
     {
-        double* base = reinterpret_cast<double*>(kin_smem) + (size_t)(threadIdx.x / G) * warp_group_words<R, EN>(M);
+        base = reinterpret_cast<double*>(kin_smem) + (size_t)(threadIdx.x / G) * warp_group_words<R, NR, EN, G>(M);
         C = reinterpret_cast<R*>(base);
         OM = C + M.nS;
-        Ks = warp_k_words<R, EN>(M) ? reinterpret_cast<R*>(base + warp_smem_elems(M)) : nullptr;
+        Ks = warp_k_words<R, EN>(M) ? reinterpret_cast<R*>(base + warp_f_words<R, EN, G>(M)) : nullptr;
     }
 
     __device__ __forceinline__ bool valid(int r) const { return lane + G * r < nV; }
@@ -928,7 +989,10 @@ struct WarpRKCK {
     __device__ __forceinline__ void f(const double (&in)[NR], double (&o)[NR])
     {
         if constexpr (EN) warp_feval_energy<R, NR, G>(M, p, C, OM, in, o, lane, mask);
-        else warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
+        else if constexpr (sizeof(R) == 4) warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
+        else
+            warp_feval_int<NR, G>(M, int_tab<G>(M), IntSmem(M, int_tab<G>(M), base), Kc, kfin, Ctot, invCtot,
+                                     scale, in, o, lane, grp);
         nfe++;
     }
 
@@ -1037,18 +1101,25 @@ __global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const _
             // previous cell's last f ended in a sync of the group)
             R* kc = W.Ks ? W.Ks : reinterpret_cast<R*>(L.cell_k) + g * nK;
             const double lnT = log(T), invT = ddiv(1.0, T);
+            bool kfin = true;
             for (int qq = lane; qq < M.nR; qq += G) {
                 const int j = M.rxn_perm[qq];
                 const double a = M.lnA[j] + M.beta[j] * lnT - M.EaR[j] * invT;
-                kc[qq] = Tab<R>::ex(a);
+                const R k = Tab<R>::ex(a);
+                kc[qq] = k;
+                if (sizeof(R) == 8) kfin &= im_finite_k(k);
                 const int fo = M.rxnp[qq].fo;
                 if (fo >= 0) {
                     const double a0 = M.lnA0[j] + M.beta0[j] * lnT - M.Ea0R[j] * invT;
-                    kc[M.nR + fo] = Tab<R>::ex(a0 - a);
+                    const R k0 = Tab<R>::ex(a0 - a);
+                    kc[M.nR + fo] = k0;
+                    if (sizeof(R) == 8) kfin &= im_finite_k(k0);
                 }
             }
             __syncwarp(W.mask);
             W.Kc = kc;
+            if (sizeof(R) == 8) W.kfin = __all_sync(W.mask, kfin);
+            W.scale = 0;
         }
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
@@ -1083,18 +1154,16 @@ __global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const _
     }
 }
 
-inline int rkck_group(int nV) { return warp_cell_lanes(KIN_RKCK, nV); }
-
-template <typename R, bool EN>
-inline size_t group_smem_bytes(const MechDev& M, int threads, int G)
+template <typename R, int NR, bool EN, int G>
+inline size_t group_smem_bytes(const MechDev& M, int threads)
 {
-    return (size_t)warp_group_words<R, EN>(M) * (threads / G) * 8;
+    return (size_t)warp_group_words<R, NR, EN, G>(M) * (threads / G) * 8;
 }
 
 template <typename R, int NR, bool EN, int G>
 inline cudaError_t warp_rkck_launch_nr(Launch& L, int blocks, int threads, cudaStream_t st)
 {
-    const size_t sm = group_smem_bytes<R, EN>(L.M, threads, G);
+    const size_t sm = group_smem_bytes<R, NR, EN, G>(L.M, threads);
     cudaError_t e = cudaFuncSetAttribute(warp_rkck_kernel<R, NR, EN, G>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -1105,71 +1174,86 @@ inline cudaError_t warp_rkck_launch_nr(Launch& L, int blocks, int threads, cudaS
 template <typename R, int NR, bool EN, int G>
 inline cudaError_t warp_rkck_occ_nr(const MechDev& M, int threads, int* bps)
 {
-    const size_t sm = group_smem_bytes<R, EN>(M, threads, G);
+    const size_t sm = group_smem_bytes<R, NR, EN, G>(M, threads);
     cudaError_t e = cudaFuncSetAttribute(warp_rkck_kernel<R, NR, EN, G>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, warp_rkck_kernel<R, NR, EN, G>, threads, sm);
 }
 
-template <typename R, int NR, int OCC, bool EN>
+template <typename R, int NR, int OCC, bool EN, int G>
 inline cudaError_t warp_launch_nr(Launch& L, int blocks, int threads, cudaStream_t st)
 {
-    const size_t sm = warp_smem_bytes<R, EN>(L.M, threads);
-    cudaError_t e = cudaFuncSetAttribute(warp_init_kernel<R, NR, OCC, EN>,
+    const size_t sm = group_smem_bytes<R, NR, EN, G>(L.M, threads);
+    cudaError_t e = cudaFuncSetAttribute(warp_init_kernel<R, NR, OCC, EN, G>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(warp_integrate_kernel<R, NR, OCC, EN>,
+        e = cudaFuncSetAttribute(warp_integrate_kernel<R, NR, OCC, EN, G>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    warp_init_kernel<R, NR, OCC, EN><<<blocks, threads, sm, st>>>(L);
+    warp_init_kernel<R, NR, OCC, EN, G><<<blocks, threads, sm, st>>>(L);
     e = launch_sort(L, st);
     if (e != cudaSuccess) return e;
-    warp_integrate_kernel<R, NR, OCC, EN><<<blocks, threads, sm, st>>>(L);
+    warp_integrate_kernel<R, NR, OCC, EN, G><<<blocks, threads, sm, st>>>(L);
     return cudaGetLastError();
 }
 
-template <typename R, int NR, int OCC, bool EN>
+template <typename R, int NR, int OCC, bool EN, int G>
 inline cudaError_t warp_occ_nr(const MechDev& M, int precision, int threads, int* bps)
 {
-    const size_t sm = warp_smem_bytes<R, EN>(M, threads);
-    cudaError_t e = cudaFuncSetAttribute(warp_integrate_kernel<R, NR, OCC, EN>,
+    const size_t sm = group_smem_bytes<R, NR, EN, G>(M, threads);
+    cudaError_t e = cudaFuncSetAttribute(warp_integrate_kernel<R, NR, OCC, EN, G>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, warp_integrate_kernel<R, NR, OCC, EN>,
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, warp_integrate_kernel<R, NR, OCC, EN, G>,
                                                          threads, sm);
 }
 
-// Register-vector width for a state of n components (component l + 32 r, r < NR).
-__host__ __device__ inline int warp_nr(int n) { return n <= 32 ? 1 : n <= 64 ? 2 : n <= 128 ? 4 : 8; }
+// Register-vector width of a state of n components on groups of G lanes
+// (component l + G r, r < NR).
+__host__ __device__ inline int warp_nr(int n, int G)
+{
+    const int r = (n + G - 1) / G;
+    return r <= 2 ? r : r <= 4 ? 4 : 8;
+}
+
+// The instantiation for groups of `lanes` lanes: FN<NR, G>.
+#define KIN_WARP_DISPATCH(FN, n, lanes)                                     \
+    if constexpr (sizeof(R) == 8 && !EN) {                                  \
+        if (lanes == 16) return FN(1, 16);                                  \
+        if constexpr (OCC == 0) {                                           \
+            if (lanes == 64) return FN(1, 64);                              \
+            if (lanes == 128) return warp_nr(n, 128) == 1 ? FN(1, 128) : FN(2, 128); \
+        }                                                                   \
+    }                                                                       \
+    switch (warp_nr(n, 32)) {                                               \
+    case 1: return FN(1, 32);                                               \
+    case 2: return FN(2, 32);                                               \
+    case 4: return FN(4, 32);                                               \
+    default: return FN(8, 32);                                              \
+    }
 
 template <typename R, int OCC, bool EN>
 inline cudaError_t warp_launch(Launch& L, int blocks, int threads, cudaStream_t st)
 {
-    switch (warp_nr(L.nV)) {
-    case 1: return warp_launch_nr<R, 1, OCC, EN>(L, blocks, threads, st);
-    case 2: return warp_launch_nr<R, 2, OCC, EN>(L, blocks, threads, st);
-    case 4: return warp_launch_nr<R, 4, OCC, EN>(L, blocks, threads, st);
-    default: return warp_launch_nr<R, 8, OCC, EN>(L, blocks, threads, st);
-    }
+#define KIN_FN(NR, G) warp_launch_nr<R, NR, OCC, EN, G>(L, blocks, threads, st)
+    KIN_WARP_DISPATCH(KIN_FN, L.nV, L.lanes)
+#undef KIN_FN
 }
 
 template <typename R, int OCC, bool EN>
-inline cudaError_t warp_occ(const MechDev& M, int nV, int precision, int threads, int* bps)
+inline cudaError_t warp_occ(const MechDev& M, int nV, int lanes, int precision, int threads, int* bps)
 {
-    switch (warp_nr(nV)) {
-    case 1: return warp_occ_nr<R, 1, OCC, EN>(M, precision, threads, bps);
-    case 2: return warp_occ_nr<R, 2, OCC, EN>(M, precision, threads, bps);
-    case 4: return warp_occ_nr<R, 4, OCC, EN>(M, precision, threads, bps);
-    default: return warp_occ_nr<R, 8, OCC, EN>(M, precision, threads, bps);
-    }
+#define KIN_FN(NR, G) warp_occ_nr<R, NR, OCC, EN, G>(M, precision, threads, bps)
+    KIN_WARP_DISPATCH(KIN_FN, nV, lanes)
+#undef KIN_FN
 }
 
 template <typename R, bool EN>
 inline cudaError_t warp_rkck_launch(Launch& L, int blocks, int threads, cudaStream_t st)
 {
-    if (rkck_group(L.nV) == 16) return warp_rkck_launch_nr<R, 1, EN, 16>(L, blocks, threads, st);
-    switch (warp_nr(L.nV)) {
+    if (L.lanes == 16) return warp_rkck_launch_nr<R, 1, EN, 16>(L, blocks, threads, st);
+    switch (warp_nr(L.nV, 32)) {
     case 1: return warp_rkck_launch_nr<R, 1, EN, 32>(L, blocks, threads, st);
     case 2: return warp_rkck_launch_nr<R, 2, EN, 32>(L, blocks, threads, st);
     case 4: return warp_rkck_launch_nr<R, 4, EN, 32>(L, blocks, threads, st);
@@ -1178,11 +1262,11 @@ inline cudaError_t warp_rkck_launch(Launch& L, int blocks, int threads, cudaStre
 }
 
 template <typename R, bool EN>
-inline cudaError_t warp_rkck_occ(const MechDev& M, int nV, int precision, int threads, int* bps)
+inline cudaError_t warp_rkck_occ(const MechDev& M, int nV, int lanes, int precision, int threads, int* bps)
 {
     (void)precision;
-    if (rkck_group(nV) == 16) return warp_rkck_occ_nr<R, 1, EN, 16>(M, threads, bps);
-    switch (warp_nr(nV)) {
+    if (lanes == 16) return warp_rkck_occ_nr<R, 1, EN, 16>(M, threads, bps);
+    switch (warp_nr(nV, 32)) {
     case 1: return warp_rkck_occ_nr<R, 1, EN, 32>(M, threads, bps);
     case 2: return warp_rkck_occ_nr<R, 2, EN, 32>(M, threads, bps);
     case 4: return warp_rkck_occ_nr<R, 4, EN, 32>(M, threads, bps);

@@ -1,0 +1,499 @@
+// warp_int.cuh -- the warp layout's isothermal FP64 f on the integer pipes
+// (intf.cuh has the arithmetic, int_tables.h the tables).
+//
+// One group of G lanes evaluates f for one cell. Concentrations live in
+// shared memory as mantissas and exponents; the lanes split the reactions of
+// a chunk, leave each rate of progress as a 128-bit word in shared memory,
+// and gather the words of the chunk into partial sums per species, G equal
+// runs of the chunk's entries. Chunks keep the words of a large mechanism from
+// taking the shared memory that resident groups and L1 need.
+//
+// An evaluation is bound by the latency of its phases, not by a pipe (cycles
+// of one evaluation of 53 species / 634 reactions, two warps, 8 cells per
+// SM: mixture 2165, products and third-body sums 8390, gather 8391, the rest
+// 1780; the FP64 f it replaced took 43 K with one warp, 354 FP64 instructions
+// of 64 cycles among them). So a lane's next reaction words, the gather's next
+// entries and eight efficiencies of a third-body sum are fetched ahead.
+// Whole calls on GB300, before and after: 53 / 634 RKC, 4,096 cells 76.9 ->
+// 38.4 ms; 111 / 1566 RKC, 16 instances of 2,000 cells in all 1067 -> 222 ms;
+// 13 / 54 RKC, 1,000 cells 3.70 -> 3.11 ms; 9 / 38 RKCK, 4,096 cells 0.715 ->
+// 0.457 ms. Error of whole results against plain FP64: unchanged (1e-13, the
+// finite differences of the spectral radius).
+#pragma once
+#include "intf.cuh"
+#include "kernels.cuh"
+
+namespace kin {
+
+// The lanes of this thread's group within its warp.
+template <int G>
+__device__ __forceinline__ unsigned group_mask()
+{
+    return G >= 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
+}
+
+// Butterfly sum over a group of G lanes (a whole warp, or a 16-lane half
+// that owns one cell); mask names the group's lanes.
+template <int G, typename T>
+__device__ __forceinline__ T group_sum(T v, unsigned mask)
+{
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+    return v;
+}
+
+template <int G>
+__device__ __forceinline__ double group_max(double v, unsigned mask)
+{
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(mask, v, o));
+    return v;
+}
+
+// A group of G lanes that evaluates one cell: a half warp, a warp, or several
+// warps of a block. Reductions leave every lane with the same bits, and the
+// sums do not depend on G: component l + 32 r is added at lane l in the order
+// of r, then the 32 (16) lanes in butterfly order. Across warps the components
+// go through shared words and the group's named barrier; the words alternate
+// between two sets, so that one barrier per reduction is enough (a set is
+// written again only after the barrier of the reduction in between).
+template <int G>
+struct Group {
+    static constexpr int WARPS = G / 32;
+    unsigned mask;
+    double* red;  // [2][set_words]
+    int set, set_words;
+
+    __device__ explicit Group(double* r, int words) : mask(group_mask<G>()), red(r), set(0), set_words(words) {}
+
+    __device__ __forceinline__ void sync() const
+    {
+        if constexpr (G <= 32) __syncwarp(mask);
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / G), "n"(G) : "memory");
+    }
+    __device__ __forceinline__ double* next_set()
+    {
+        double* b = red + set * set_words;
+        set ^= 1;
+        return b;
+    }
+    // One value per warp, seen by all.
+    template <typename T>
+    __device__ __forceinline__ const T* exchange(T v)
+    {
+        static_assert(sizeof(T) <= 8, "one shared word per warp");
+        T* t = reinterpret_cast<T*>(next_set());
+        if ((threadIdx.x & 31) == 0) t[(threadIdx.x % G) >> 5] = v;
+        sync();
+        return t;
+    }
+    // Sum of v, or of its squares, over the components (lane + G r). (__dadd_rn:
+    // no product in v is fused into the sum, which only some G could.)
+    template <bool SQ, int NR>
+    __device__ __forceinline__ double sum_of(const double (&v)[NR])
+    {
+        double s = 0.0;
+        if constexpr (G <= 32) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) s = SQ ? fma(v[r], v[r], s) : __dadd_rn(s, v[r]);
+        } else {
+            double* b = next_set();
+#pragma unroll
+            for (int r = 0; r < NR; ++r) b[threadIdx.x % G + G * r] = v[r];
+            sync();
+#pragma unroll
+            for (int r = 0; r < NR * WARPS; ++r) {
+                const double u = b[(threadIdx.x & 31) + 32 * r];
+                s = SQ ? fma(u, u, s) : __dadd_rn(s, u);
+            }
+        }
+        return group_sum<(G < 32 ? G : 32)>(s, mask);
+    }
+    template <int NR>
+    __device__ __forceinline__ double sum(const double (&v)[NR])
+    {
+        return sum_of<false>(v);
+    }
+    template <int NR>
+    __device__ __forceinline__ double sum_sq(const double (&v)[NR])
+    {
+        return sum_of<true>(v);
+    }
+    __device__ __forceinline__ double max(double v)
+    {
+        v = group_max<(G < 32 ? G : 32)>(v, mask);
+        if constexpr (G > 32) {
+            const double* b = exchange(v);
+            v = b[0];
+#pragma unroll
+            for (int w = 1; w < WARPS; ++w) v = fmax(v, b[w]);
+        }
+        return v;
+    }
+    __device__ __forceinline__ int imax(int v)
+    {
+        v = __reduce_max_sync(mask, v);
+        if constexpr (G > 32) {
+            const int* b = exchange(v);
+            v = b[0];
+#pragma unroll
+            for (int w = 1; w < WARPS; ++w) v = ::max(v, b[w]);
+        }
+        return v;
+    }
+    __device__ __forceinline__ bool all(bool v)
+    {
+        if constexpr (G <= 32) return __all_sync(mask, v);
+        else return imax(!v) == 0;
+    }
+    // v of the group's lane k
+    template <typename T>
+    __device__ __forceinline__ T from(T v, int k)
+    {
+        if constexpr (G <= 32) return __shfl_sync(mask, v, k, G);
+        else {
+            double* b = next_set();
+            if ((int)(threadIdx.x % G) == k) *reinterpret_cast<T*>(b) = v;
+            sync();
+            return *reinterpret_cast<const T*>(b);
+        }
+    }
+};
+// Shared words of one set of a group's reductions, NR components per lane.
+template <int NR, int G>
+__host__ __device__ constexpr int group_set_words() { return G > 32 ? NR * G : 0; }
+
+// The group's shared arrays.
+struct IntSmem {
+    ulonglong2* OM;  // [chunk + 1] rates of progress of a chunk, and a zero word
+    ulonglong2* P;   // [nslots] partial sums
+    int2* CF;        // [nS, even] concentrations as 55-bit fractions: 30 high, 25 low bits
+    im_u64* CM;      // [nS + 1] mantissas, after the constant 1 that empty slots read
+    uint32_t* CE;    // [nS + 1] exponent words
+
+    __device__ IntSmem(const MechDev& M, const IntDev& I, double* base)
+    {
+        OM = reinterpret_cast<ulonglong2*>(base);
+        P = OM + I.chunk + 1;
+        CF = reinterpret_cast<int2*>(P + I.nslots);
+        CM = reinterpret_cast<im_u64*>(CF + ((M.nS + 1) & ~1));
+        CE = reinterpret_cast<uint32_t*>(CM + M.nS + 1);
+    }
+};
+
+// Shared FP64 words of a group, a multiple of 4.
+__host__ __device__ __forceinline__ int int_smem_words(const MechDev& M, const IntDev& I)
+{
+    const int w = 2 * (I.chunk + 1 + I.nslots) + ((M.nS + 1) & ~1) + M.nS + 1 + (M.nS + 2) / 2;
+    return (w + 3) & ~3;
+}
+
+// A concentration back from its mantissa.
+__device__ __forceinline__ double int_conc(const IntSmem& S, int k)
+{
+    const im_u64 m = S.CM[k] >> 10;
+    const uint32_t e = S.CE[k];
+    return __hiloint2double((int)((e & 0x80000000u) | ((e & 0x7ffu) << 20) | ((uint32_t)(m >> 32) & 0xfffffu)),
+                            (int)(uint32_t)m);
+}
+
+// [M] of an efficiency row in FP64, from concentrations c[k + 1] given by get.
+template <typename Get>
+__device__ double int_row_dot(const MechDev& M, int row, Get get)
+{
+    const double2* __restrict__ a = reinterpret_cast<const double2*>(M.effV64) + row;
+    double m = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < M.nS; ++k) {
+        const double2 e = a[(int64_t)(k >> 1) * M.nM];
+        m += ((k & 1) ? e.y : e.x) * get(k + 1);
+    }
+    return m;
+}
+
+static __device__ __noinline__ double int_row_dot_slow(const MechDev& M, int row, const IntSmem& S)
+{
+    return int_row_dot(M, row, [&](int k) { return int_conc(S, k); });
+}
+
+// sum_j nu_ij Omega_j of species i in plain FP64, one term after another, from
+// the concentrations c[k + 1] in shared memory (c[0] = 1): for states outside
+// the integer forms' range. Such states are trial points that blew up, so
+// this code is small rather than fast.
+static __device__ __noinline__ double int_general_sum(const MechDev& M, const double* Kc, const double* c, int i)
+{
+    const int nP = M.nR - M.nM, nF = M.nR - M.nFO;
+    double w = 0.0;
+#pragma unroll 1
+    for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
+        const int q = M.csrp_rxn[e];
+        const uint32_t r = M.rxw[q];
+        double v = Kc[q] * c[r & 0xffffu] * c[r >> 16];
+        if (q >= nP) {
+            const double Mc = int_row_dot(M, q - nP, [&](int k) { return c[k]; });
+            if (q < nF) {
+                v *= Mc;
+            } else {
+                const double Pr = Kc[M.nR + (q - nF)] * Mc;
+                v *= ddiv(Pr, 1.0 + Pr);
+            }
+        }
+        w += M.csr_nu[e] * v;
+    }
+    return w;
+}
+
+// Pr / (1 + Pr): the reciprocal by two Newton steps and one correction of the
+// quotient (within an ulp; an IEEE division is a third longer).
+__device__ __forceinline__ double falloff_factor(double Pr)
+{
+    const double d = 1.0 + Pr, r = Tab<double>::inv(d), q = Pr * r;
+    const double z = fma(r, fma(-q, d, Pr), q);
+    return isfinite(z) ? z : ddiv(Pr, d);
+}
+
+// f of such a state, from its concentrations (the group's lanes together).
+template <int NR, int G>
+__device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, const double* Kc, const double (&c)[NR],
+                                            double invrho, double (&out)[NR], int lane, const Group<G>& grp)
+{
+    double* cs = reinterpret_cast<double*>(S.CM);
+    if (lane == 0) cs[0] = 1.0;
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        if (lane + G * r < M.nS) cs[lane + G * r + 1] = c[r];
+    grp.sync();
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        out[r] = i < M.nS ? __dmul_rn(int_general_sum(M, Kc, cs, i), M.W[i] * invrho) : 0.0;
+    }
+    grp.sync();
+}
+
+// f for the group's cell. `scale` is the exponent of the largest rate of the
+// cell's previous evaluation (kept by the caller, any value at the first); an
+// evaluation whose rates outgrow it by more than IM_GUARD octaves is repeated
+// with its own. kfin: the cell's rate constants are finite.
+template <int NR, int G>
+__device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I, const IntSmem& S, const double* Kc,
+                                               bool kfin, double Ctot, double invCtot, int& scale,
+                                               const double (&x)[NR], double (&out)[NR], int lane, Group<G>& grp)
+{
+    const int nS = M.nS, nR = M.nR, nM = M.nM;
+    double c[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        c[r] = i < nS ? x[r] * M.invW[i] : 0.0;
+    }
+    const double s = grp.sum(c);
+    const double rho = Ctot * Tab<double>::inv(s);
+    const uint32_t top = (uint32_t)__double2hiint(Ctot);
+    const int eT = (int)(top >> 20);
+    bool in = kfin && top - 0x00100000u < 0x7fe00000u;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        c[r] *= rho;
+        // finite, and not below -2^-9 of the total (by the high words)
+        const uint32_t hi = (uint32_t)__double2hiint(c[r]);
+        in = in && (hi < 0x7ff00000u || (hi >= 0x80000000u && (hi & 0x7fffffffu) + (9u << 20) < top));
+    }
+    const double invrho = s * invCtot;
+    if (!grp.all(in)) {
+        int_general<NR, G>(M, S, Kc, c, invrho, out, lane, grp);
+        return;
+    }
+    if (lane == 0) {
+        S.CM[0] = 1ull << 62;
+        S.CE[0] = 1023u;
+        S.OM[I.chunk] = make_ulonglong2(0ull, 0ull);
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        if (i < nS) {
+            im_u64 m;
+            uint32_t e;
+            im_split(c[r], m, e);
+            S.CM[i + 1] = m;
+            S.CE[i + 1] = e;
+            if (nM) {
+                // c 2^(55 - x), x the exponent above Ctot's: sum |F| < 3 * 2^55
+                const uint32_t down = (uint32_t)(eT - (int)(e & 0x7ffu) + 7);
+                long long F = (long long)((im_shr(m, down) + 1ull) >> 1);
+                if (e >> 31) F = -F;
+                S.CF[i] = make_int2((int)(F >> 25), (int)(F & ((1 << 25) - 1)));
+            }
+        } else if (i == nS && (nS & 1)) {
+            S.CF[i] = make_int2(0, 0);
+        }
+    }
+    grp.sync();
+    const int nP = nR - nM, nF = nR - M.nFO;
+    double wr[NR];  // W_i / rho
+#pragma unroll
+    for (int r = 0; r < NR; ++r) wr[r] = lane + G * r < nS ? __dmul_rn(M.W[lane + G * r], invrho) : 0.0;
+    im_u128 acc[NR];
+    for (;;) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r] = im_u128{0ull, 0ull};
+        int emax = -100000;
+        // K C C of reaction q, from its reactants' word and its rate constant
+        auto product = [&](uint32_t w, double k, im_u64& Q, uint32_t& e) {
+            im_split_k(k, Q, e);
+            const uint32_t a = w & 0xffffu, b = w >> 16;
+            Q = im_mul(im_mul(S.CM[a], S.CM[b]), Q);
+            e += S.CE[a] + S.CE[b];
+        };
+        auto store = [&](im_u64 Q, uint32_t e, int at) {
+            const int x = (int)(e & 0x7fffffffu);
+            if (Q) emax = max(emax, x);
+            im_u128 v = im_place(Q, min(x - scale + IM_UP, 63));
+            if (e >> 31) {
+                im_u128 z{0ull, 0ull};
+                im_sub(z, v.lo, v.hi);
+                v = z;
+            }
+            S.OM[at] = make_ulonglong2(v.lo, v.hi);
+        };
+        // the lane's reactions follow each other through the chunks, so the
+        // next one's words are on their way while this one is formed
+        uint32_t wn = 0;
+        double kn = 0.0;
+        if (lane < nR) {
+            wn = M.rxw[lane];
+            kn = Kc[lane];
+        }
+#pragma unroll 1
+        for (int ch = 0, q0 = 0; ch < I.nchunk; ++ch, q0 += I.chunk) {
+            const int q1 = min(nR, q0 + I.chunk);
+#pragma unroll 1
+            for (int q = q0 + lane; q < q1; q += G) {
+                const uint32_t w = wn;
+                const double kq = kn;
+                if (q + G < nR) {
+                    wn = M.rxw[q + G];
+                    kn = Kc[q + G];
+                }
+                im_u64 Q;
+                uint32_t e;
+                product(w, kq, Q, e);
+                if (q >= nP) {
+                    const int row = q - nP;
+                    const int4* __restrict__ E = M.effI + row;
+                    const int4* F = reinterpret_cast<const int4*>(S.CF);
+                    long long hi = 0, mid = 0;
+                    auto term = [&](const int4& u, const int4& f) {
+                        hi += (long long)u.x * f.x;
+                        mid += (long long)u.x * f.y;
+                        mid += (long long)u.y * f.x;
+                        hi += (long long)u.z * f.z;
+                        mid += (long long)u.z * f.w;
+                        mid += (long long)u.w * f.z;
+                    };
+                    const int n2 = (nS + 1) >> 1;
+                    int k = 0;
+#pragma unroll 1
+                    for (; k + 7 < n2; k += 8) {
+                        int4 u[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) u[j] = E[(int64_t)(k + j) * nM];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) term(u[j], F[k + j]);
+                    }
+#pragma unroll 4
+                    for (; k < n2; ++k) term(E[(int64_t)k * nM], F[k]);
+                    const long long U = hi + (mid >> 25);
+                    double Md = 0.0;
+                    im_u64 mm;
+                    uint32_t em;
+                    if (U < (1ll << 54)) {  // small beside its terms: the fractions are too coarse
+                        Md = int_row_dot_slow(M, row, S);
+                        im_split(Md, mm, em);
+                    } else {
+                        const int z = __clzll(U);
+                        mm = (im_u64)U << (z - 1);
+                        em = (uint32_t)(M.effX[row] + eT + 5 - z);
+                        if (q >= nF) {
+                            const double d = (double)mm;  // [2^62, 2^63]
+                            Md = __hiloint2double(__double2hiint(d) + (((int)em - IM_BIAS) << 20),
+                                                  __double2loint(d));
+                        }
+                    }
+                    if (q >= nF) {
+                        im_split(falloff_factor(__dmul_rn(Kc[nR + (q - nF)], Md)), mm, em);
+                        if ((em & 0x7ffu) == 0x7ffu) emax = IM_OUT;
+                    }
+                    Q = im_mul(Q, mm);
+                    e += em - (uint32_t)(IM_BIAS - 64);
+                }
+                store(Q, e, q - q0);
+            }
+            // the run's first entries, fetched ahead of the barrier
+            const int k0 = I.step0[ch], K = I.step0[ch + 1] - k0;
+            const uint32_t* __restrict__ ent = I.ent + (int64_t)k0 * G + lane;
+            ulonglong2* P = S.P + I.slot0[ch * G + lane];
+            int part[NR];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) part[r] = lane + G * r < nS ? I.part[ch * nS + lane + G * r] : 0;
+            uint32_t en[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) en[j] = j < K ? ent[G * j] : (uint32_t)I.chunk;
+            grp.sync();
+            im_u128 w{0ull, 0ull};
+#pragma unroll 1
+            for (int k = 0; k < K; k += 4) {
+                uint32_t e[4];
+                ulonglong2 v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    e[j] = en[j];
+                    v[j] = S.OM[e[j] & INT_POS_MASK];
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) en[j] = k + 4 + j < K ? ent[G * (k + 4 + j)] : (uint32_t)I.chunk;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    im_add(w, v[j].x, v[j].y);
+                    if (e[j] & INT_FLUSH) {
+                        *P++ = make_ulonglong2(w.lo, w.hi);
+                        w = im_u128{0ull, 0ull};
+                    }
+                }
+            }
+            grp.sync();
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const ulonglong2* p = S.P + (part[r] >> 16);
+                const int np = (part[r] >> 8) & 0xff, n = np + (part[r] & 0xff);
+#pragma unroll 1
+                for (int k = 0; k < n; ++k) {
+                    const ulonglong2 v = p[k];
+                    if (k < np) im_add(acc[r], v.x, v.y);
+                    else im_sub(acc[r], v.x, v.y);
+                }
+            }
+        }
+        emax = grp.imax(emax);
+        if (emax >= IM_OUT) {  // a falloff factor that is not finite
+            int_general<NR, G>(M, S, Kc, c, invrho, out, lane, grp);
+            return;
+        }
+        const bool fits = emax <= scale + IM_GUARD;
+        const int s0 = scale;
+        if (!fits || emax < scale - IM_SLACK) scale = max(emax, 0);
+        if (fits) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int i = lane + G * r;
+                // a word's unit at e = s0: 2^(128 + s0 - 3 IM_BIAS - IM_UP)
+                out[r] = i < nS ? __dmul_rn(im_double(acc[r], 128 + s0 - 3 * IM_BIAS - IM_UP), wr[r]) : 0.0;
+            }
+            grp.sync();  // the shared words are rewritten by the next evaluation
+            return;
+        }
+    }
+}
+
+}  // namespace kin
