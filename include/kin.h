@@ -76,7 +76,10 @@ extern "C" {
 #define KIN_LAYOUT_AUTO 0 /* library choice: KIN_LAYOUT_WARP when n_reactions >
                              KIN_WARP_MIN_REACTIONS or the call has fewer than
                              KIN_WARP_MAX_CELLS_PER_SM cells per SM of the device (too
-                             few to give every lane a cell), else KIN_LAYOUT_LANE */
+                             few to give every lane a cell); also below
+                             KIN_WARP_FP64_MAX_CELLS_PER_SM for isothermal FP64 RKC on at
+                             most 16 species, unless a launch shape, staging, register
+                             budget or f evaluation is asked for; else KIN_LAYOUT_LANE */
 #define KIN_LAYOUT_LANE 1 /* one lane integrates one cell (the paper's thread-per-ODE
                              design, Section 3): per-cell arrays in the workspace or in
                              shared memory (kin_opts.staging) */
@@ -91,6 +94,7 @@ extern "C" {
                              to 256 */
 #define KIN_WARP_MIN_REACTIONS 256
 #define KIN_WARP_MAX_CELLS_PER_SM 64
+#define KIN_WARP_FP64_MAX_CELLS_PER_SM 512
 
 /* how the lane-per-cell layout evaluates f (kin_opts.feval) */
 #define KIN_FEVAL_AUTO 0      /* the generated f for an isothermal call of at least
@@ -294,6 +298,9 @@ int kin_integrate_host(const kin_mech *m, int64_t cells, double *T, const double
  *    contents; each call clears what must start at zero. Calls that overlap
  *    on the GPU (on different streams, or from different threads) race on it:
  *    serialise them.
+ *  - The automatic layout is chosen as kin_integrate chooses it, but a call
+ *    whose cells would not fit the array in the lane layout is refused in
+ *    either.
  *  - The working memory grows with the cell count and the persistent blocks
  *    per SM. blocks_per_sm is resolved as in kin_integrate (0: as many as
  *    fit); when that workspace exceeds the array, the call steps down to the

@@ -65,16 +65,29 @@ struct Grid {
 
 // Automatic layout: one warp per cell for large mechanisms (a lane's working
 // set would stream from memory) and for calls too small to give every lane of
-// the GPU a cell; one lane per cell otherwise.
-int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm)
+// the GPU a cell; one lane per cell otherwise. `full`: without the rule below.
+int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm, bool full = true)
 {
     if (o->layout != KIN_LAYOUT_AUTO) return o->layout;
     if (m->nR > KIN_WARP_MIN_REACTIONS) return KIN_LAYOUT_WARP;
-    return cells < (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
+    if (cells < (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return KIN_LAYOUT_WARP;
+    // Isothermal FP64 RKC on small mechanisms: the warp layout's integer f, four
+    // cells to a warp, beats a lane per cell until each lane of the GPU has one
+    // (13 species: 30,000 cells 14.6 ms against 39.0, 60,000 29.1 against 52.4,
+    // 262,144 128 against 122 with the generated f). A call that names a shape or
+    // form of the lane layout keeps it.
+    const bool free_shape = o->block_threads == 0 && o->blocks_per_sm == 0 && o->staging == KIN_STAGE_GLOBAL &&
+                            o->occupancy == KIN_OCC_DEFAULT && o->feval == KIN_FEVAL_AUTO;
+    if (full && free_shape && o->method == KIN_RKC && o->precision == KIN_FP64 && !o->energy && m->nS <= 16 &&
+        cells < (int64_t)KIN_WARP_FP64_MAX_CELLS_PER_SM * nsm)
+        return KIN_LAYOUT_WARP;
+    return KIN_LAYOUT_LANE;
 }
 
 // Lanes that integrate one cell in the warp layout: half a warp for states of
-// at most 16 components (RKCK; RKC in isothermal FP64), a warp, and in
+// at most 16 components (RKCK; RKC in isothermal FP64, there a quarter above
+// 64 cells per SM: 13 species, 4,000 cells 4.0 ms with 16 lanes and 5.6 with
+// 8, 16,000 cells 9.8 and 8.6, 30,000 cells 17.9 and 14.6), a warp, and in
 // isothermal FP64 RKC two warps above 32 components and four above 64. An
 // evaluation is a chain of short phases, so more lanes shorten it, and the
 // FP64 pipe's vector work per cell stays the same (fewer slots per lane on more
@@ -83,9 +96,10 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm)
 // 111 species, 200 / 8,000 cells 42 against 175, 231 against 323 ms. One warp
 // where the block size does not hold whole groups, and with KIN_OCC_HIGH, whose
 // 48-register kernels exist for single warps.
-int cell_lanes(const kin_opts* o, int nV, int threads)
+int cell_lanes(const kin_opts* o, int nV, int threads, int64_t cells, int nsm)
 {
     const bool f64 = o->method == KIN_RKC && o->precision == KIN_FP64 && !o->energy;
+    if (nV <= 16 && f64 && !o->occupancy && cells > (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return 8;
     if (nV <= 16) return o->method == KIN_RKCK || f64 ? 16 : 32;
     if (!f64 || o->occupancy || nV <= 32) return 32;
     const int g = nV <= 64 ? 64 : 128;
@@ -111,7 +125,7 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
     int occ = 0, cap = 0, lanes = 1;
     if (layout == KIN_LAYOUT_WARP) {
         if (threads % 32 != 0 || threads > 256) return fail(KIN_EINVAL, "block_threads must be a multiple of 32 and <= 256");
-        lanes = cell_lanes(o, m->nS + o->energy, threads);
+        lanes = cell_lanes(o, m->nS + o->energy, threads, cells, nsm);
         // the layout's limit on a mechanism: C and Omega of a block's cells in
         // shared memory (the FP64 f's own words need no more)
         const size_t sm = (size_t)((m->nS + m->nR + 3) & ~3) * 8 * (threads / std::min(lanes, 32));
@@ -204,6 +218,14 @@ int kin::noalloc_opts(const kin_mech* m, const kin_opts* in, int64_t cells, int6
     int rc = check_opts(in);
     if (rc) return rc;
     kin_opts o = *in;
+    // the layout of kin_integrate's choice; its cells have to fit the array in
+    // the lane layout too where only the f evaluation and the launch shape,
+    // left to the library, make it the warp layout
+    int nsm = 1;
+    cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
+    o.layout = resolve_layout(m, in, cells, nsm);
+    const int limit = resolve_layout(m, in, cells, nsm, false);
     // Never compile here: NVRTC and loading the compiled library allocate
     // device memory. The generated f runs only where an earlier call loaded
     // it on this device; otherwise the automatic choice falls back to the
@@ -219,11 +241,17 @@ int kin::noalloc_opts(const kin_mech* m, const kin_opts* in, int64_t cells, int6
     Grid g;
     rc = grid_for(m, &o, cells, &g);  // resolves blocks_per_sm = 0 to "as many as fit"
     if (rc) return rc;
-    int nsm = 1;
-    cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     int64_t need = 0;
-    for (int bps = g.blocks / nsm; bps >= 1; --bps) {
+    if (limit != o.layout) {
+        kin_opts l = o;
+        l.layout = limit;
+        l.blocks_per_sm = 1;
+        Grid gl;
+        rc = grid_for(m, &l, cells, &gl);
+        if (rc) return rc;
+        need = ws_bytes(m, &l, gl, cells);
+    }
+    for (int bps = need > cap ? 0 : g.blocks / nsm; bps >= 1; --bps) {
         o.blocks_per_sm = bps;
         rc = grid_for(m, &o, cells, &g);
         if (rc) return rc;
@@ -494,11 +522,11 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     // per SM beside the tables in L1
     IntGather ig[INT_NTAB];
     size_t oIg[INT_NTAB][4];
-    const int ig_lanes[INT_NTAB] = {16, 32, 64, 128};
-    const bool ig_use[INT_NTAB] = {nS <= 16, true, nS > 32 && nS <= 64, nS > 64};
+    const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128};
+    const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS > 32 && nS <= 64, nS > 64};
     for (int v = 0; v < INT_NTAB; ++v) {
         if (!ig_use[v]) continue;
-        const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, 8 * ig_lanes[v]));
+        const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, 8 * ig_lanes[v])));
         ig[v] = build_int_gather(nS, nR, ptr.data(), crxp.data(), cnu.data(), chunk, ig_lanes[v]);
         oIg[v][0] = put(ig[v].step0.data(), 4 * ig[v].step0.size());
         oIg[v][1] = put(ig[v].ent.data(), 4 * ig[v].ent.size());
@@ -514,6 +542,16 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
             effI[((size_t)(k / 2) * nM + row) * 4 + 2 * (k % 2) + 1] = lo[k];
         }
     }
+    std::vector<uint64_t> imW(2 * nS);
+    std::vector<int32_t> imWe(2 * nS);
+    for (int i = 0; i < nS; ++i) {
+        imW[2 * i] = int_split(1.0L / d->W[i], &imWe[2 * i]);
+        imW[2 * i + 1] = int_split(d->W[i], &imWe[2 * i + 1]);
+    }
+    int imLow = 0;
+    for (int j = 0; j < nR; ++j)
+        if ((d->reac[2 * j] >= 0) + (d->reac[2 * j + 1] >= 0) + (rxn[j].type == KIN_RXN_THIRD_BODY) < 2) imLow = 1;
+    const size_t oImW = put(imW.data(), 8 * imW.size()), oImWe = put(imWe.data(), 4 * imWe.size());
     const size_t oEffI = put(effI.data(), 4 * effI.size()), oEffX = put(effX.data(), 4 * effX.size());
     // the segmented FP32 gather of the 32-lane isothermal f, where the packed
     // entries apply and its partial sums fit in the FP32 half of the warp's
@@ -576,6 +614,9 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     }
     M.effI = (const int4*)(b + oEffI);
     M.effX = (const int32_t*)(b + oEffX);
+    M.imW = (const ulonglong2*)(b + oImW);
+    M.imWe = (const int2*)(b + oImWe);
+    M.imLow = imLow;
     M.effV64 = (const double*)(b + oEffV64);
     M.effV32 = (const float*)(b + oEffV32);
     M.rxw = (const uint32_t*)(b + oRxw);
@@ -606,6 +647,27 @@ int kin_destroy(kin_mech* m)
     return e == cudaSuccess ? KIN_OK : cuda_fail(e, "cudaFree");
 }
 
+// The largest workspace of a call with these options: the automatic layout
+// depends on the f evaluation, which a caller may set after sizing the
+// workspace.
+static int max_ws_bytes(const kin_mech* m, const kin_opts* o, int64_t cells, int64_t* bytes)
+{
+    Grid g;
+    int rc = grid_for(m, o, cells, &g);
+    if (rc) return rc;
+    *bytes = ws_bytes(m, o, g, cells);
+    int nsm = 0;
+    const cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
+    kin_opts lane = *o;
+    lane.layout = resolve_layout(m, o, cells, nsm, false);
+    if (lane.layout == g.layout) return KIN_OK;
+    rc = grid_for(m, &lane, cells, &g);
+    if (rc) return rc;
+    *bytes = std::max(*bytes, ws_bytes(m, &lane, g, cells));
+    return KIN_OK;
+}
+
 int64_t kin_workspace_bytes(const kin_mech* m, const kin_opts* o, int64_t cells)
 {
     g_err[0] = 0;
@@ -613,10 +675,9 @@ int64_t kin_workspace_bytes(const kin_mech* m, const kin_opts* o, int64_t cells)
     if (cells < 0) return fail(KIN_EINVAL, "cells < 0");
     int rc = check_opts(o);
     if (rc) return rc;
-    Grid g;
-    rc = grid_for(m, o, cells, &g);
-    if (rc) return rc;
-    return ws_bytes(m, o, g, cells);
+    int64_t bytes = 0;
+    rc = max_ws_bytes(m, o, cells, &bytes);
+    return rc ? rc : bytes;
 }
 
 int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, const kin_opts* o,

@@ -108,6 +108,20 @@ inline IntGather build_int_gather(int nS, int nR, const int* ptr, const int* pos
     return t;
 }
 
+// 63-bit left-aligned mantissa of v > 0 and its exponent as in a double.
+inline uint64_t int_split(long double v, int* e)
+{
+    int x = 0;
+    const long double f = frexpl(v, &x);  // v = f 2^x, f in [1/2, 1)
+    uint64_t m = (uint64_t)llroundl(ldexpl(f, 62)) << 1;
+    if (m == 1ull << 63) {
+        m >>= 1;
+        ++x;
+    }
+    *e = x - 1 + 1023;
+    return m;
+}
+
 // A row's efficiencies as 55-bit integers: hi (30 bits, signed) and lo (25
 // bits) of round(eff 2^(54 - x)). Returns x.
 inline int int_efficiencies(int nS, const double* eff, int32_t* hi, int32_t* lo)

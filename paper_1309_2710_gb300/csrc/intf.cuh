@@ -12,7 +12,7 @@
 //    keeps the top 62 bits of the mantissas' product (three IMAD.WIDE, 6
 //    cycles for a DMUL's 64);
 //  * a rate of progress is placed into a 128-bit fixed-point word whose unit
-//    is 2^-101 or less of the largest rate of the evaluation, so every sum of
+//    is 2^-99 (at most 2^-83) of the largest rate of the evaluation, so every sum of
 //    rates is exact (four 32-bit adds) but for the words' own last bits;
 //  * a third-body sum multiplies 55-bit integer efficiencies by the
 //    concentrations as 55-bit fractions of the total.
@@ -63,7 +63,13 @@ __device__ __forceinline__ void im_split_k(double v, im_u64& m, uint32_t& e)
 __device__ __forceinline__ bool im_finite_k(double v) { return ((uint32_t)__double2hiint(v) >> 20) < 0x7ffu; }
 __device__ __forceinline__ bool im_finite_k(float v) { return (__float_as_uint(v) >> 23) < 0xffu; }
 
-// 64-bit shifts by any unsigned amount (64 and more give zero).
+struct im_u128 {
+    im_u64 lo, hi;
+};
+
+// 64-bit shifts by any unsigned amount (64 and more give zero), and 128-bit
+// sums (the plain forms are for host compilers).
+#ifdef __CUDACC__
 __device__ __forceinline__ im_u64 im_shl(im_u64 v, uint32_t n)
 {
     im_u64 r;
@@ -76,11 +82,6 @@ __device__ __forceinline__ im_u64 im_shr(im_u64 v, uint32_t n)
     asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
     return r;
 }
-
-struct im_u128 {
-    im_u64 lo, hi;
-};
-
 __device__ __forceinline__ void im_add(im_u128& a, im_u64 lo, im_u64 hi)
 {
     asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(lo), "l"(hi));
@@ -89,6 +90,21 @@ __device__ __forceinline__ void im_sub(im_u128& a, im_u64 lo, im_u64 hi)
 {
     asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(lo), "l"(hi));
 }
+#else
+inline im_u64 im_shl(im_u64 v, uint32_t n) { return n < 64 ? v << n : 0; }
+inline im_u64 im_shr(im_u64 v, uint32_t n) { return n < 64 ? v >> n : 0; }
+inline void im_add(im_u128& a, im_u64 lo, im_u64 hi)
+{
+    const im_u64 l = a.lo + lo;
+    a.hi += hi + (l < lo);
+    a.lo = l;
+}
+inline void im_sub(im_u128& a, im_u64 lo, im_u64 hi)
+{
+    a.hi -= hi + (a.lo < lo);
+    a.lo -= lo;
+}
+#endif
 
 // Q * 2^L as a 128-bit word, Q < 2^61, L <= 63; bits below the unit drop.
 __device__ __forceinline__ im_u128 im_place(im_u64 Q, int L)
@@ -99,8 +115,22 @@ __device__ __forceinline__ im_u128 im_place(im_u64 Q, int L)
     return r;
 }
 
-// a * 2^x as a double, rounded once (a signed).
-__device__ __forceinline__ double im_double(im_u128 a, int x)
+// r * 2^x rounded to a double, 2^52 < r < 2^63 (0 gives 0), negated if neg.
+__device__ __forceinline__ double im_round(im_u64 r, int x, bool neg)
+{
+    if (r == 0ull) return 0.0;
+    const int z = __clzll((long long)r);
+    const im_u64 m = ((r << (z - 1)) + 512ull) >> 10;  // [2^52, 2^53]
+    const int n = 1075 + x + 11 - z;
+    im_u64 b = m + ((im_u64)(uint32_t)(n - 1) << 52);  // a carry into 2^53 raises the exponent
+    if (n <= 0) b = 0ull;
+    if (n >= 0x7ff) b = 0x7ff0000000000000ull;
+    return __longlong_as_double((long long)(neg ? b | 0x8000000000000000ull : b));
+}
+
+// (a 2^x) (u 2^(eu - IM_BIAS)) (v 2^(ev - IM_BIAS)) of a signed 128-bit word and
+// two 63-bit mantissas, as a double.
+__device__ __forceinline__ double im_scaled(im_u128 a, int x, im_u64 u, int eu, im_u64 v, int ev)
 {
     const bool neg = (long long)a.hi < 0;
     if (neg) {
@@ -115,19 +145,17 @@ __device__ __forceinline__ double im_double(im_u128 a, int x)
         if (a.hi == 0ull) return 0.0;
     }
     const int z = __clzll((long long)a.hi);
-    im_u64 v = a.hi;
-    if (z) v = (v << z) | (a.lo >> (64 - z));
-    const double d = (double)v;  // [2^63, 2^64]
-    const int n = (__double2hiint(d) >> 20) + x + 64 - z;
-    if (n <= 0) return 0.0;
-    const int hi = n >= 0x7ff ? 0x7ff00000 : ((__double2hiint(d) & 0xfffff) | (n << 20));
-    const double r = __hiloint2double(hi, n >= 0x7ff ? 0 : __double2loint(d));
-    return neg ? -r : r;
+    im_u64 t = a.hi;
+    if (z) t = (t << z) | (a.lo >> (64 - z));
+    t = im_mul(t >> 1, u) << 1;
+    return im_round(im_mul(t, v), x + 64 - z + 1 + eu + ev - 2 * IM_BIAS + 127, neg);
 }
 
 // Bits a word of the largest rate (e = the evaluation's scale) is shifted up:
-// Q < 2^61, so it stays below 2^(61 + 43 + 8) where the scale is 8 octaves too
-// low, which leaves 15 bits for a row's entries and the sign.
+// Q < 2^61, so it stays below 2^(61 + 43 + 8) where the scale is IM_GUARD octaves
+// too low, which leaves 15 bits for a row's entries and the sign. The words'
+// unit is 2^-99 of the largest rate (Q >= 2^56), 2^-83 where the scale is
+// IM_SLACK octaves too high.
 constexpr int IM_UP = 43, IM_GUARD = 8, IM_SLACK = 16;
 
 // Exponent that stands for a rate that is not finite.

@@ -48,9 +48,9 @@ struct IntDev {
     const int32_t* slot0;   // [nchunk][G]
     const int32_t* part;    // [nchunk][nS]
 };
-// One set per number of lanes that share a cell (16: states of at most 16
-// components; 64 and 128: more than 32 and 64).
-enum IntTab : int { INT_G16 = 0, INT_G32, INT_G64, INT_G128, INT_NTAB };
+// One set per number of lanes that share a cell (8 and 16: states of at most
+// 16 components; 64 and 128: more than 32 and 64).
+enum IntTab : int { INT_G8 = 0, INT_G16, INT_G32, INT_G64, INT_G128, INT_NTAB };
 
 // Species slots of 32 in the warp layout's ELL gather tables.
 constexpr int ELL_SLOTS = (KIN_MAX_SPECIES + 31) / 32;
@@ -89,6 +89,9 @@ struct MechDev {
     IntDev ig[INT_NTAB];
     const int4* effI;      // [(nS + 1) / 2][nM] integer efficiencies {hi, lo} of two species
     const int32_t* effX;   // [nM] their exponents
+    const ulonglong2* imW; // [nS] 63-bit mantissas of 1 / W and W
+    const int2* imWe;      // [nS] their exponents
+    int imLow;             // 1: a reaction of fewer than two factors of concentration
     // efficiencies by non-plain reaction in permutation order (row), species
     // in 16-byte groups: [k / V][row][k % V], V = 2 (FP64) or 4 (FP32), the
     // last group zero-padded

@@ -97,7 +97,7 @@ __device__ __forceinline__ double eff_dot<double>(const MechDev& M, int row, con
 template <int G>
 __host__ __device__ __forceinline__ const IntDev& int_tab(const MechDev& M)
 {
-    return M.ig[G == 16 ? INT_G16 : G == 32 ? INT_G32 : G == 64 ? INT_G64 : INT_G128];
+    return M.ig[G == 8 ? INT_G8 : G == 16 ? INT_G16 : G == 32 ? INT_G32 : G == 64 ? INT_G64 : INT_G128];
 }
 
 // Shared FP64 words of C [nS] and Omega [nR] in the energy and FP32 forms of
@@ -401,7 +401,7 @@ struct WarpRKC {
     double Ctot, invCtot, atol, rtol, p;
     R CtotR, invCtotR;   // the same in the rate type
     int nfe, nsig, nfs;  // f evaluations, sigma estimates, f evaluations inside them
-    double y[NR], f0[NR], w1[NR], w2[NR], fx[NR], x[NR], ev[NR];
+    double y[NR], f0[NR], w1[NR], w2[NR], fx[NR], x[NR], ev[NR];  // (x: sigma() only)
 
     __device__ explicit WarpRKC(const Launch& l)
         : L(l), M(l.M), Kc(nullptr), lane(threadIdx.x & (G - 1)), nV(l.nV), grp(nullptr, group_set_words<NR, G>()), mask(group_mask<G>()), scale(0), kfin(true)
@@ -416,6 +416,16 @@ struct WarpRKC {
 
     __device__ __forceinline__ bool valid(int r) const { return lane + G * r < nV; }
 
+    __device__ __forceinline__ static unsigned long long bits(double v)
+    {
+        return (unsigned long long)__double_as_longlong(v);
+    }
+    // max(|a|, |b|) by the bits (a NaN wins): no comparison on the FP64 pipe
+    __device__ __forceinline__ static double max_abs(double a, double b)
+    {
+        const unsigned long long m = 0x7fffffffffffffffull, u = bits(a) & m, v = bits(b) & m;
+        return __longlong_as_double((long long)(u > v ? u : v));
+    }
     // a * b + c and a * b of the state vectors. In the FP64 path the fused and
     // the separate operations are named, so that every group size rounds alike;
     // the mixed path leaves the choice to the compiler.
@@ -465,7 +475,7 @@ struct WarpRKC {
             double q[NR];
 #pragma unroll
             for (int r = 0; r < NR; ++r)
-                q[r] = valid(r) ? ddiv(d[r], fma(rtol, fmax(fabs(a[r]), fabs(b[r])), atol)) : 0.0;
+                q[r] = valid(r) ? ddiv(d[r], fma(rtol, max_abs(a[r], b[r]), atol)) : 0.0;
             acc = grp.sum_sq(q);
         } else {
 #pragma unroll
@@ -609,142 +619,319 @@ struct WarpRKC {
         return M.rkc + ((int64_t)s * RKC_TAB_S + j) * RKC_TAB_W;
     }
 
-    // RKC integration over [0, dt] from the pre-pass state (y, f0, ev and the
-    // given sigma and first trial step h). Returns the cell status.
-    __device__ int run(double dt, double sig, double h, int& nacc, int& nrej)
+    // Stages of a step of hh at spectral radius sig (SMAX + 1: more than the
+    // cap). The mixed-precision path takes the square root in FP32: s is an
+    // integer, which the FP32 root changes only where 1 + sqrt(1 + 1.54 h sigma)
+    // lies within FP32 rounding of an integer, and the FP64 root is a dozen
+    // instructions on the FP64 pipe that all lanes repeat. The FP64 path takes
+    // it in FP32 too unless that lands within 5e-4 of an integer (or above the
+    // cap), where the FP64 root decides.
+    __device__ __forceinline__ static int stages(double hh, double sig)
     {
-        double t = 0.0, hprev = 0.0, cprev = 0.0;
-        int attempts = 0, since = 0;
-        bool sigma_here = true, last_rej = false, have_prev = false;
-        const double invN = ddiv(1.0, (double)nV);
-        for (;;) {
-            if (attempts >= L.max_steps) return KIN_CELL_MAXSTEPS;
-            if (since >= 25 || (last_rej && !sigma_here)) {
-                sig = sigma(false);
-                nsig++;
-                since = 0;
-                sigma_here = true;
-                if (!isfinite(sig)) return KIN_CELL_NONFINITE;
-            }
-            double hh = h;
-            bool last = false;
-            if (hh >= dt - t) {
-                hh = dt - t;
-                last = true;
-            }
-            // The mixed-precision path takes the stage count's square root in
-            // FP32: s is an integer, which the FP32 root changes only where
-            // 1 + sqrt(1 + 1.54 h sigma) lies within FP32 rounding of an
-            // integer, and the FP64 root is a dozen instructions on the FP64
-            // pipe that all 32 lanes repeat.
-            double sr;
-            if constexpr (sizeof(R) == 4)
-                sr = (double)floorf(1.0f + sqrtf(1.0f + (float)(1.54 * hh * sig)));
-            else
-                sr = floor(1.0 + dsqrt(1.0 + 1.54 * hh * sig));
-            int s;
-            if (sr < 2.0) {
-                s = 2;
-            } else if (sr > (double)SMAX) {
-                s = SMAX;
-                hh = ddiv((SMAX - 1.0) * (SMAX - 1.0) - 1.0, 1.54 * sig);
-                last = false;
-            } else {
-                s = (int)sr;
-            }
-            // w_0 = y, w_1 = y + mu~_1 h f_0, then the three-term recursion
-            const double m1 = coef(s, 1)[2] * hh;
+        if constexpr (sizeof(R) == 4) {
+            const double sr = (double)floorf(1.0f + sqrtf(1.0f + (float)(1.54 * hh * sig)));
+            return sr < 2.0 ? 2 : sr > (double)SMAX ? SMAX + 1 : (int)sr;
+        } else {
+            const double v = fma(__dmul_rn(1.54, hh), sig, 1.0);
+            const float u = 1.0f + sqrtf((float)v), k = floorf(u);
+            if (u < SMAX + 0.5f && u - k >= 5e-4f && u - k <= 1.0f - 5e-4f) return max(2, (int)k);
+            const double sr = floor(1.0 + dsqrt(v));
+            return sr < 2.0 ? 2 : sr > (double)SMAX ? SMAX + 1 : (int)sr;
+        }
+    }
+
+    // w_1 = y + mu~_1 h f_0 of a step of s stages; w_0 = y.
+    __device__ __forceinline__ void first_stage(int s, double hh)
+    {
+        const double m1 = coef(s, 1)[2] * hh;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            w2[r] = y[r];
+            w1[r] = mul_add(m1, f0[r], y[r]);
+        }
+    }
+
+    // w_j from f(w_{j-1}) in fx (the three-term recursion).
+    __device__ __forceinline__ void stage(int s, int j, double hh)
+    {
+        const double* c = coef(s, j);
+        const double mu = c[0], nu = c[1], mt = c[2] * hh, gt = c[3] * hh, c0 = c[4];
+        if (sizeof(R) == 8 && j == 2) {
+            // w_0 = y, w_1 = y + m1 f_0: w_2 = y + (mu m1 + gamma~ h) f_0 + mu~ h f_1
+            const double a = fma(mu, coef(s, 1)[2] * hh, gt);
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
-                w2[r] = y[r];
-                w1[r] = mul_add(m1, f0[r], y[r]);
+                w2[r] = w1[r];
+                w1[r] = fma(mt, fx[r], fma(a, f0[r], y[r]));
             }
-            for (int j = 2;; ++j) {
+            return;
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            double wn;
+            if constexpr (sizeof(R) == 8)
+                wn = fma(gt, f0[r], fma(mt, fx[r], fma(nu, w2[r], fma(mu, w1[r], __dmul_rn(c0, y[r])))));
+            else
+                wn = c0 * y[r] + mu * w1[r] + nu * w2[r] + mt * fx[r] + gt * f0[r];
+            w2[r] = w1[r];
+            w1[r] = wn;
+        }
+    }
+
+    // Sum of the squared weighted error components of the step that ends in w1.
+    __device__ __forceinline__ double error_sum(double hh)
+    {
+        double acc = 0.0;
+        if constexpr (sizeof(R) == 8) {
+            double q[NR];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const double d = fma(0.8, y[r] - w1[r], __dmul_rn(0.4 * hh, f0[r] + fx[r]));
+                const double sc = fma(rtol, max_abs(y[r], w1[r]), atol);
+                q[r] = valid(r) ? __dmul_rn(d, rcp_newton(sc)) : 0.0;
+            }
+            acc = grp.sum_sq(q);
+        } else {
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                if (valid(r)) {
+                    const double d = 0.8 * (y[r] - w1[r]) + 0.4 * hh * (f0[r] + fx[r]);
+                    const double sc = atol + rtol * fmax(fabs(y[r]), fabs(w1[r]));
+                    const double q = d * rcp_newton(sc);
+                    acc += q * q;
+                }
+            acc = group_sum<G>(acc, mask);
+        }
+        return acc;
+    }
+
+    // Integration state of a cell.
+    struct Cell {
+        double dt, sig, h;                  // flow step, spectral radius, next step size
+        double t, hprev, cprev, hh;
+        int attempts, since, nacc, nrej;
+        int s, j;                           // stages of the step, stage whose f comes next (j > s: f(w_s))
+        bool last, sigma_here, last_rej, have_prev;
+        // a spectral-radius estimate in progress (groups of less than a warp)
+        bool estimating, wait;
+        int k;
+        double dyn, prev, eps;
+
+        __device__ void start(double dt_, double sig_, double h_)
+        {
+            dt = dt_;
+            sig = sig_;
+            h = h_;
+            t = hprev = cprev = 0.0;
+            attempts = since = nacc = nrej = 0;
+            sigma_here = true;
+            last_rej = have_prev = estimating = false;
+        }
+        __device__ bool stale() const { return since >= 25 || (last_rej && !sigma_here); }
+    };
+
+    // The next step's size and stages, and w_1.
+    __device__ __forceinline__ void begin_step(Cell& U)
+    {
+        double hh = U.h;
+        bool last = false;
+        if (hh >= U.dt - U.t) {
+            hh = U.dt - U.t;
+            last = true;
+        }
+        int s = stages(hh, U.sig);
+        if (s > SMAX) {
+            s = SMAX;
+            hh = ddiv((SMAX - 1.0) * (SMAX - 1.0) - 1.0, 1.54 * U.sig);
+            last = false;
+        }
+        U.hh = hh;
+        U.last = last;
+        U.s = s;
+        U.j = 2;
+        first_stage(s, hh);
+    }
+
+    // Error test and step control after f(w_s). Returns a final status, or -1.
+    __device__ __forceinline__ int end_step(Cell& U, double invN)
+    {
+        const double hh = U.hh;
+        U.attempts++;
+        // x = ||Delta||^2; z = x^(-1/6) = err^(-1/3) (see the lane kernel)
+        // (one evaluation of the power serves both branches)
+        const double xe = error_sum(hh) * invN;
+        // (the mixed-precision path keeps the FP32 power, within 4 ulp: a
+        // step-size factor, with the FP32 rates' precision)
+        double z = 0.0;
+        const bool pos = bits(xe) - 1ull < 0x7fefffffffffffffull;  // 0 < xe < inf (xe is not negative)
+        if (pos) {
+            if constexpr (sizeof(R) == 4)
+                z = f32_normal(xe) ? (double)powf((float)xe, -1.0f / 6.0f) : dpow(xe, -1.0 / 6.0);
+            else
+                z = rpow6_newton(xe);
+        }
+        if (bits(xe) <= bits(1.0)) {
+            U.nacc++;
+            double fac, c3 = 0.0;
+            if (xe == 0.0) {
+                fac = 10.0;
+            } else {
+                const double z2 = z * z;
+                c3 = xe * (z2 * z2 * z);
+                if (U.have_prev && !U.last_rej && U.cprev > 0.0)
+                    fac = 0.8 * hh * U.cprev * z2 * rcp_newton(U.hprev);
+                else fac = 0.8 * z;
+            }
+            fac = fmin(10.0, fmax(0.1, fac));
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                y[r] = w1[r];
+                f0[r] = fx[r];
+            }
+            if (U.last) return KIN_CELL_OK;
+            U.t += hh;
+            U.have_prev = true;
+            U.hprev = hh;
+            U.cprev = c3;
+            U.last_rej = false;
+            U.sigma_here = false;
+            U.since++;
+            U.h = fac * hh;
+        } else {
+            U.nrej++;
+            double fac = pos ? 0.8 * z : 0.1;
+            if (fac < 0.1) fac = 0.1;
+            U.last_rej = true;
+            U.h = fac * hh;
+            if (U.h < 1e-20 * U.dt) return KIN_CELL_HMIN;
+        }
+        return -1;
+    }
+
+    // RKC integration of a started cell (y, f0 and ev from the pre-pass).
+    // Returns the cell status.
+    __device__ int run(Cell& U)
+    {
+        const double invN = ddiv(1.0, (double)nV);
+        for (;;) {
+            if (U.attempts >= L.max_steps) return KIN_CELL_MAXSTEPS;
+            if (U.stale()) {
+                U.sig = sigma(false);
+                nsig++;
+                U.since = 0;
+                U.sigma_here = true;
+                if (!isfinite(U.sig)) return KIN_CELL_NONFINITE;
+            }
+            begin_step(U);
+            for (;; ++U.j) {
                 f(w1, fx);  // f(w_{j-1}); after the last stage, f(w_s)
-                if (j > s) break;
-                const double* c = coef(s, j);
-                const double mu = c[0], nu = c[1], mt = c[2] * hh, gt = c[3] * hh, c0 = c[4];
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    double wn;
-                    if constexpr (sizeof(R) == 8)
-                        wn = fma(gt, f0[r], fma(mt, fx[r], fma(nu, w2[r], fma(mu, w1[r], __dmul_rn(c0, y[r])))));
-                    else
-                        wn = c0 * y[r] + mu * w1[r] + nu * w2[r] + mt * fx[r] + gt * f0[r];
-                    w2[r] = w1[r];
-                    w1[r] = wn;
-                }
+                if (U.j > U.s) break;
+                stage(U.s, U.j, U.hh);
             }
-            attempts++;
-            double acc = 0.0;
-            if constexpr (sizeof(R) == 8) {
-                double q[NR];
+            const int code = end_step(U, invN);
+            if (code >= 0) return code;
+        }
+    }
+
+    // ---- several cells per warp (FP64): one evaluation of f at a time ----
+    // Each call of run's loop would let the warp's groups drift apart, and a
+    // group in an estimate would keep the others waiting for its evaluations.
+    // Here every pass of the kernel's loop evaluates f once for each group, at
+    // the point its cell needs next (w1), and then does that cell's own
+    // bookkeeping.
+
+    // The point to evaluate in pass `pass`, once a step or an estimate has ended.
+    // Steps start in even passes (nearly all have two evaluations), so that the
+    // groups of a warp are in the same part of their steps and run its control
+    // together. Returns a final status, or -1.
+    __device__ __forceinline__ int next_point(Cell& U, unsigned pass)
+    {
+        if (U.attempts >= L.max_steps) return KIN_CELL_MAXSTEPS;
+        U.wait = false;
+        if (!U.stale()) {
+            U.estimating = false;
+            U.wait = pass & 1u;
+            begin_step(U);
+            return -1;
+        }
+        U.estimating = true;
+        U.k = 0;
+        U.prev = 0.0;
+        if (L.sigma_method == KIN_SIGMA_POWER) U.dyn = power_setup();
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    const double d = fma(0.8, y[r] - w1[r], __dmul_rn(0.4 * hh, f0[r] + fx[r]));
-                    const double sc = fma(rtol, fmax(fabs(y[r]), fabs(w1[r])), atol);
-                    q[r] = valid(r) ? __dmul_rn(d, rcp_newton(sc)) : 0.0;
-                }
-                acc = grp.sum_sq(q);
-            } else {
+        for (int r = 0; r < NR; ++r) w2[r] = 0.0;  // Gershgorin row sums
+        sigma_point(U);
+        return -1;
+    }
+
+    __device__ __forceinline__ void sigma_point(Cell& U)
+    {
+        if (L.sigma_method == KIN_SIGMA_POWER) {
 #pragma unroll
-                for (int r = 0; r < NR; ++r)
-                    if (valid(r)) {
-                        const double d = 0.8 * (y[r] - w1[r]) + 0.4 * hh * (f0[r] + fx[r]);
-                        const double sc = atol + rtol * fmax(fabs(y[r]), fabs(w1[r]));
-                        const double q = d * rcp_newton(sc);
-                        acc += q * q;
-                    }
-                acc = group_sum<G>(acc, mask);
-            }
-            // x = ||Delta||^2; z = x^(-1/6) = err^(-1/3) (see the lane kernel)
-            // (one evaluation of the power serves both branches)
-            const double xe = acc * invN;
-            // (the mixed-precision path keeps the FP32 power, within 4 ulp: a
-            // step-size factor, with the FP32 rates' precision)
-            double z = 0.0;
-            if (xe > 0.0 && isfinite(xe)) {
-                if constexpr (sizeof(R) == 4)
-                    z = f32_normal(xe) ? (double)powf((float)xe, -1.0f / 6.0f) : dpow(xe, -1.0 / 6.0);
-                else
-                    z = rpow6_newton(xe);
-            }
-            if (xe <= 1.0) {
-                nacc++;
-                double fac, c3 = 0.0;
-                if (xe == 0.0) {
-                    fac = 10.0;
-                } else {
-                    const double z2 = z * z;
-                    c3 = xe * (z2 * z2 * z);
-                    if (have_prev && !last_rej && cprev > 0.0)
-                        fac = 0.8 * hh * cprev * z2 * rcp_newton(hprev);
-                    else fac = 0.8 * z;
-                }
-                fac = fmin(10.0, fmax(0.1, fac));
+            for (int r = 0; r < NR; ++r) w1[r] = y[r] + ev[r];
+            return;
+        }
+        const int kr = U.k / G, kl = U.k % G;
+        const double yk = grp.from(reg_get(y, kr), kl);
+        U.eps = SIG_SQRT_U * fmax(fabs(yk), atol);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    y[r] = w1[r];
-                    f0[r] = fx[r];
-                }
-                if (last) return KIN_CELL_OK;
-                t += hh;
-                have_prev = true;
-                hprev = hh;
-                cprev = c3;
-                last_rej = false;
-                sigma_here = false;
-                since++;
-                h = fac * hh;
-            } else {
-                nrej++;
-                double fac = isfinite(xe) ? 0.8 * z : 0.1;
-                if (fac < 0.1) fac = 0.1;
-                last_rej = true;
-                h = fac * hh;
-                if (h < 1e-20 * dt) return KIN_CELL_HMIN;
+        for (int r = 0; r < NR; ++r) w1[r] = (r == kr && lane == kl) ? yk + U.eps : y[r];
+    }
+
+    // fx = f(w1) of an estimate; true when it has ended (U.sig).
+    __device__ __forceinline__ bool sigma_post(Cell& U)
+    {
+        if (L.sigma_method == KIN_SIGMA_POWER) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) fx[r] = fx[r] - f0[r];
+            const double wn = dsqrt(grp.sum_sq(fx)), sg = ddiv(wn, U.dyn);
+            U.sig = 1.2 * sg;
+            if (!(wn > 0.0) || !isfinite(wn)) return true;
+            const double sc = ddiv(U.dyn, wn);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) ev[r] = mul(fx[r], sc);
+            if (U.k >= 1 && fabs(sg - U.prev) <= 0.01 * sg) return true;
+            U.prev = sg;
+            if (++U.k >= 20) return true;
+        } else {
+            const double ie = rcp_newton(U.eps);
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                if (valid(r)) w2[r] += fabs(__dmul_rn(fx[r] - f0[r], ie));
+            if (++U.k >= nV) {
+                double m = 0.0;
+#pragma unroll
+                for (int r = 0; r < NR; ++r) m = fmax(m, w2[r]);
+                U.sig = grp.max(m);
+                return true;
             }
         }
+        sigma_point(U);
+        return false;
+    }
+
+    // What follows f(w1) = fx. Returns a final status, or -1.
+    __device__ __forceinline__ int advance(Cell& U, double invN, unsigned pass)
+    {
+        bool ended = false;
+        if (U.estimating) {
+            nfs++;
+            ended = sigma_post(U);
+            if (ended) {
+                nsig++;
+                U.since = 0;
+                U.sigma_here = true;
+                if (!isfinite(U.sig)) return KIN_CELL_NONFINITE;
+            }
+        } else if (U.j <= U.s) {
+            stage(U.s, U.j, U.hh);
+            U.j++;
+        } else {
+            const int code = end_step(U, invN);
+            if (code >= 0) return code;
+            ended = true;
+        }
+        return ended ? next_point(U, pass + 1) : -1;
     }
 };
 
@@ -865,80 +1052,144 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
     }
 }
 
-// Persistent main kernel: each warp takes cells from the queue in the
+// Take cell g into W: its constants, state and pre-pass results. Returns the
+// status that the pre-pass decided, or 0.
+template <typename R, int NR, bool EN, int G>
+__device__ __forceinline__ uint8_t warp_load_cell(WarpRKC<R, NR, EN, G>& W, const InstDev& I, int64_t g, int64_t c)
+{
+    const Launch& L = W.L;
+    const MechDev& M = W.M;
+    const int lane = W.lane, nK = M.nR + M.nFO, nS = M.nS, nV = L.nV;
+    W.nfe = L.cell_nfe[g];
+    W.nfs = L.cell_nfs[g];
+    W.nsig = 1;
+    const uint8_t pre = L.cell_st[g];
+    if (pre != 0) return pre;  // Y stays as given
+    const double T = I.T[c], p = I.p[c];
+    W.Ctot = ddiv(p * 1e-6, R_GAS * T);
+    W.invCtot = ddiv(1.0, W.Ctot);
+    W.CtotR = (R)W.Ctot;
+    W.invCtotR = (R)W.invCtot;
+    W.atol = I.atol;
+    W.rtol = I.rtol;
+    W.p = p;
+    if constexpr (EN) {
+        W.Kc = nullptr;
+    } else {
+        const R* kg = reinterpret_cast<const R*>(L.cell_k) + g * nK;
+        bool kfin = true;
+        if (W.Ks || sizeof(R) == 8)
+            for (int q = lane; q < nK; q += G) {
+                const R k = kg[q];
+                if (sizeof(R) == 8) kfin &= im_finite_k(k);
+                if (W.Ks) W.Ks[q] = k;  // staged (the last f of the previous cell ended in a sync)
+            }
+        if (sizeof(R) == 8) W.kfin = W.grp.all(kfin);
+        W.scale = 0;
+        if (W.Ks) W.grp.sync();
+        W.Kc = W.Ks ? W.Ks : kg;
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        const bool v = i < nV;
+        W.y[r] = i < nS ? I.Y[(int64_t)i * I.ldY + c] : (v ? T : 0.0);
+        W.f0[r] = v ? L.cell_f0[g * nV + i] : 0.0;
+        W.ev[r] = (v && L.cell_ev) ? L.cell_ev[g * nV + i] : 0.0;
+    }
+    return 0;
+}
+
+// Cell c's result: its state unless the pre-pass decided its status, the
+// status and the statistics.
+template <typename R, int NR, bool EN, int G>
+__device__ __forceinline__ void warp_store_cell(const WarpRKC<R, NR, EN, G>& W, const InstDev& I, int64_t c, bool state,
+                                                int code, int nacc, int nrej)
+{
+    const int lane = W.lane, nS = W.M.nS;
+    if (state) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int i = lane + G * r;
+            if (i < nS) I.Y[(int64_t)i * I.ldY + c] = W.y[r];
+            else if (i == nS && EN) I.T[c] = W.y[r];
+        }
+    }
+    if (lane == 0) {
+        if (I.status) I.status[c] = (uint8_t)code;
+        if (I.stats) {
+            int32_t* st = I.stats + KIN_NSTATS * c;
+            st[0] = W.nfe;
+            st[1] = nacc;
+            st[2] = nrej;
+            st[3] = W.nsig;
+            st[4] = W.nfs;
+        }
+    }
+}
+
+// Persistent main kernel: each group takes cells from the queue in the
 // longest-first order and integrates them one after another.
 template <typename R, int NR, int OCC, bool EN, int G>
 __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp_integrate_kernel(const __grid_constant__ Launch L)
 {
-    WarpRKC<R, NR, EN, G> W(L);
-    const MechDev& M = L.M;
-    const int lane = W.lane, nK = M.nR + M.nFO, nS = M.nS, nV = L.nV;
-    for (;;) {
-        unsigned long long q = 0;
-        if (lane == 0) q = atomicAdd(L.queue, 1ull);
-        q = W.grp.from(q, 0);
-        if (q >= (unsigned long long)L.total) return;
-        const int64_t g = L.order[q];
-        const int ii = find_inst(L, g);
-        const InstDev& I = L.inst[ii];
-        const int64_t c = g - L.start[ii];
-        int nacc = 0, nrej = 0, code;
-        W.nfe = L.cell_nfe[g];
-        W.nfs = L.cell_nfs[g];
-        W.nsig = 1;
-        const uint8_t pre = L.cell_st[g];
-        if (pre != 0) {
-            code = pre;  // decided by the pre-pass; Y stays as given
-        } else {
-            const double T = I.T[c], p = I.p[c];
-            W.Ctot = ddiv(p * 1e-6, R_GAS * T);
-            W.invCtot = ddiv(1.0, W.Ctot);
-            W.CtotR = (R)W.Ctot;
-            W.invCtotR = (R)W.invCtot;
-            W.atol = I.atol;
-            W.rtol = I.rtol;
-            W.p = p;
-            if constexpr (EN) {
-                W.Kc = nullptr;
-            } else {
-                const R* kg = reinterpret_cast<const R*>(L.cell_k) + g * nK;
-                bool kfin = true;
-                if (W.Ks || sizeof(R) == 8)
-                    for (int q = lane; q < nK; q += G) {
-                        const R k = kg[q];
-                        if (sizeof(R) == 8) kfin &= im_finite_k(k);
-                        if (W.Ks) W.Ks[q] = k;  // staged (the last f of the previous cell ended in a sync)
-                    }
-                if (sizeof(R) == 8) W.kfin = W.grp.all(kfin);
-                W.scale = 0;
-                if (W.Ks) W.grp.sync();
-                W.Kc = W.Ks ? W.Ks : kg;
+    using Warp = WarpRKC<R, NR, EN, G>;
+    Warp W(L);
+    typename Warp::Cell U;
+    if constexpr (G >= 32) {
+        for (;;) {
+            unsigned long long q = 0;
+            if (W.lane == 0) q = atomicAdd(L.queue, 1ull);
+            q = W.grp.from(q, 0);
+            if (q >= (unsigned long long)L.total) return;
+            const int64_t g = L.order[q];
+            const int ii = find_inst(L, g);
+            const InstDev& I = L.inst[ii];
+            const int64_t c = g - L.start[ii];
+            int code = warp_load_cell(W, I, g, c);
+            const bool pre = code != 0;  // decided by the pre-pass
+            U.nacc = U.nrej = 0;
+            if (!pre) {
+                U.start(I.dt, L.cell_sig[g], L.cell_h[g]);
+                code = W.run(U);
             }
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int i = lane + G * r;
-                const bool v = i < nV;
-                W.y[r] = i < nS ? I.Y[(int64_t)i * I.ldY + c] : (v ? T : 0.0);
-                W.f0[r] = v ? L.cell_f0[g * nV + i] : 0.0;
-                W.ev[r] = (v && L.cell_ev) ? L.cell_ev[g * nV + i] : 0.0;
-            }
-            code = W.run(I.dt, L.cell_sig[g], L.cell_h[g], nacc, nrej);
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int i = lane + G * r;
-                if (i < nS) I.Y[(int64_t)i * I.ldY + c] = W.y[r];
-                else if (i == nS && EN) I.T[c] = W.y[r];
-            }
+            warp_store_cell(W, I, c, !pre, code, U.nacc, U.nrej);
         }
-        if (lane == 0) {
-            if (I.status) I.status[c] = (uint8_t)code;
-            if (I.stats) {
-                int32_t* st = I.stats + KIN_NSTATS * c;
-                st[0] = W.nfe;
-                st[1] = nacc;
-                st[2] = nrej;
-                st[3] = W.nsig;
-                st[4] = W.nfs;
+    } else {
+        // the warp's groups together: one evaluation of f per pass (a group
+        // without a cell waits)
+        const double invN = ddiv(1.0, (double)W.nV);
+        bool have = false, more = true;
+        int ii = 0;
+        int64_t c = 0;
+        for (unsigned pass = 0;; ++pass) {
+            while (!have && more) {
+                unsigned long long q = 0;
+                if (W.lane == 0) q = atomicAdd(L.queue, 1ull);
+                q = W.grp.from(q, 0);
+                more = q < (unsigned long long)L.total;
+                if (!more) break;
+                const int64_t g = L.order[q];
+                ii = find_inst(L, g);
+                c = g - L.start[ii];
+                int code = warp_load_cell(W, L.inst[ii], g, c);
+                const bool pre = code != 0;
+                U.start(L.inst[ii].dt, L.cell_sig[g], L.cell_h[g]);
+                if (!pre) code = W.next_point(U, pass);
+                have = !pre && code < 0;
+                if (!have) warp_store_cell(W, L.inst[ii], c, !pre, code, 0, 0);
+            }
+            if (__all_sync(0xffffffffu, !have)) return;
+            const bool go = have && !U.wait;
+            U.wait = false;
+            if (go) W.f(W.w1, W.fx);
+            __syncwarp();
+            if (go) {
+                const int code = W.advance(U, invN, pass);
+                if (code >= 0) {
+                    warp_store_cell(W, L.inst[ii], c, true, code, U.nacc, U.nrej);
+                    have = false;
+                }
             }
         }
     }
@@ -1220,6 +1471,9 @@ __host__ __device__ inline int warp_nr(int n, int G)
 // The instantiation for groups of `lanes` lanes: FN<NR, G>.
 #define KIN_WARP_DISPATCH(FN, n, lanes)                                     \
     if constexpr (sizeof(R) == 8 && !EN) {                                  \
+        if constexpr (OCC == 0) {                                           \
+            if (lanes == 8) return FN(2, 8);                                \
+        }                                                                   \
         if (lanes == 16) return FN(1, 16);                                  \
         if constexpr (OCC == 0) {                                           \
             if (lanes == 64) return FN(1, 64);                              \

@@ -29,7 +29,7 @@ namespace kin {
 template <int G>
 __device__ __forceinline__ unsigned group_mask()
 {
-    return G >= 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
+    return G >= 32 ? 0xffffffffu : (((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1)));
 }
 
 // Butterfly sum over a group of G lanes (a whole warp, or a 16-lane half
@@ -53,7 +53,8 @@ __device__ __forceinline__ double group_max(double v, unsigned mask)
 // A group of G lanes that evaluates one cell: a half warp, a warp, or several
 // warps of a block. Reductions leave every lane with the same bits, and the
 // sums do not depend on G: component l + 32 r is added at lane l in the order
-// of r, then the 32 (16) lanes in butterfly order. Across warps the components
+// of r, then the 32 (16, 8) lanes in butterfly order (the first step of 16
+// lanes adds the components that 8 lanes hold in two slots). Across warps the components
 // go through shared words and the group's named barrier; the words alternate
 // between two sets, so that one barrier per reduction is enough (a set is
 // written again only after the barrier of the reduction in between).
@@ -95,7 +96,10 @@ struct Group {
         double s = 0.0;
         if constexpr (G <= 32) {
 #pragma unroll
-            for (int r = 0; r < NR; ++r) s = SQ ? fma(v[r], v[r], s) : __dadd_rn(s, v[r]);
+            for (int r = 0; r < NR; ++r) {
+                if constexpr (SQ && G == 32) s = fma(v[r], v[r], s);
+                else s = __dadd_rn(s, SQ ? __dmul_rn(v[r], v[r]) : v[r]);
+            }
         } else {
             double* b = next_set();
 #pragma unroll
@@ -188,13 +192,11 @@ __host__ __device__ __forceinline__ int int_smem_words(const MechDev& M, const I
     return (w + 3) & ~3;
 }
 
-// A concentration back from its mantissa.
+// A c_k / rho back from its mantissa.
 __device__ __forceinline__ double int_conc(const IntSmem& S, int k)
 {
-    const im_u64 m = S.CM[k] >> 10;
     const uint32_t e = S.CE[k];
-    return __hiloint2double((int)((e & 0x80000000u) | ((e & 0x7ffu) << 20) | ((uint32_t)(m >> 32) & 0xfffffu)),
-                            (int)(uint32_t)m);
+    return im_round(S.CM[k], (int)(e & 0x7fffffffu) - 64 - IM_BIAS, (int)e < 0);
 }
 
 // [M] of an efficiency row in FP64, from concentrations c[k + 1] given by get.
@@ -252,16 +254,16 @@ __device__ __forceinline__ double falloff_factor(double Pr)
     return isfinite(z) ? z : ddiv(Pr, d);
 }
 
-// f of such a state, from its concentrations (the group's lanes together).
+// f of such a state, from its c_k / rho (the group's lanes together).
 template <int NR, int G>
 __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, const double* Kc, const double (&c)[NR],
-                                            double invrho, double (&out)[NR], int lane, const Group<G>& grp)
+                                            double rho, double invrho, double (&out)[NR], int lane, const Group<G>& grp)
 {
     double* cs = reinterpret_cast<double*>(S.CM);
     if (lane == 0) cs[0] = 1.0;
 #pragma unroll
     for (int r = 0; r < NR; ++r)
-        if (lane + G * r < M.nS) cs[lane + G * r + 1] = c[r];
+        if (lane + G * r < M.nS) cs[lane + G * r + 1] = c[r] * rho;
     grp.sync();
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
@@ -273,56 +275,67 @@ __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, 
 
 // f for the group's cell. `scale` is the exponent of the largest rate of the
 // cell's previous evaluation (kept by the caller, any value at the first); an
-// evaluation whose rates outgrow it by more than IM_GUARD octaves is repeated
-// with its own. kfin: the cell's rate constants are finite.
+// evaluation whose largest is more than IM_GUARD octaves above it or IM_SLACK
+// below is repeated with its own. kfin: the cell's rate constants are finite.
 template <int NR, int G>
 __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I, const IntSmem& S, const double* Kc,
                                                bool kfin, double Ctot, double invCtot, int& scale,
                                                const double (&x)[NR], double (&out)[NR], int lane, Group<G>& grp)
 {
     const int nS = M.nS, nR = M.nR, nM = M.nM;
+    // c_k / rho = Y_k / W_k: in FP64 for the mixture sum, and as mantissa and
+    // exponent word (64 above the double's, so that 1 / W never takes it below
+    // zero) for everything else
     double c[NR];
+    im_u64 m[NR];
+    uint32_t e[NR];
+    int neg = -100000;
+    bool in = kfin;
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         const int i = lane + G * r;
-        c[r] = i < nS ? x[r] * M.invW[i] : 0.0;
+        c[r] = 0.0;
+        m[r] = 0ull;
+        e[r] = 0u;
+        if (i < nS) {
+            c[r] = __dmul_rn(x[r], M.invW[i]);
+            im_split(x[r], m[r], e[r]);
+            in = in && (e[r] & 0x7ffu) != 0x7ffu;
+            const int z = (int)(e[r] & 0x7ffu) + M.imWe[i].x - 1022 + 64;
+            if ((int)e[r] < 0 && m[r]) neg = max(neg, z);
+            m[r] = im_mul(m[r], M.imW[i].x) << 1;
+            e[r] = (uint32_t)z | (e[r] & 0x80000000u);
+        }
     }
     const double s = grp.sum(c);
     const double rho = Ctot * Tab<double>::inv(s);
-    const uint32_t top = (uint32_t)__double2hiint(Ctot);
+    const uint32_t top = (uint32_t)__double2hiint(s);
     const int eT = (int)(top >> 20);
-    bool in = kfin && top - 0x00100000u < 0x7fe00000u;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        c[r] *= rho;
-        // finite, and not below -2^-9 of the total (by the high words)
-        const uint32_t hi = (uint32_t)__double2hiint(c[r]);
-        in = in && (hi < 0x7ff00000u || (hi >= 0x80000000u && (hi & 0x7fffffffu) + (9u << 20) < top));
-    }
-    const double invrho = s * invCtot;
+    // finite, and no species below -2^-9 of the total
+    in = in && top - 0x00100000u < 0x7fe00000u && neg + 9 <= eT + 64;
     if (!grp.all(in)) {
-        int_general<NR, G>(M, S, Kc, c, invrho, out, lane, grp);
+        int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
         return;
     }
+    im_u64 mr, mi = 0ull;  // rho and 1 / rho
+    uint32_t er, ei = 0u;
+    im_split_k(rho, mr, er);
+    if (M.imLow) im_split_k(s * invCtot, mi, ei);
     if (lane == 0) {
         S.CM[0] = 1ull << 62;
-        S.CE[0] = 1023u;
+        S.CE[0] = 1023u + 64u;
         S.OM[I.chunk] = make_ulonglong2(0ull, 0ull);
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         const int i = lane + G * r;
         if (i < nS) {
-            im_u64 m;
-            uint32_t e;
-            im_split(c[r], m, e);
-            S.CM[i + 1] = m;
-            S.CE[i + 1] = e;
+            S.CM[i + 1] = m[r];
+            S.CE[i + 1] = e[r];
             if (nM) {
-                // c 2^(55 - x), x the exponent above Ctot's: sum |F| < 3 * 2^55
-                const uint32_t down = (uint32_t)(eT - (int)(e & 0x7ffu) + 7);
-                long long F = (long long)((im_shr(m, down) + 1ull) >> 1);
-                if (e >> 31) F = -F;
+                // 2^55 of twice the total at most: sum |F| < 3 * 2^55
+                long long F = (long long)((im_shr(m[r], (uint32_t)(eT - (int)(e[r] & 0xfffu) + 71)) + 1ull) >> 1);
+                if ((int)e[r] < 0) F = -F;
                 S.CF[i] = make_int2((int)(F >> 25), (int)(F & ((1 << 25) - 1)));
             }
         } else if (i == nS && (nS & 1)) {
@@ -331,14 +344,11 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
     }
     grp.sync();
     const int nP = nR - nM, nF = nR - M.nFO;
-    double wr[NR];  // W_i / rho
-#pragma unroll
-    for (int r = 0; r < NR; ++r) wr[r] = lane + G * r < nS ? __dmul_rn(M.W[lane + G * r], invrho) : 0.0;
     im_u128 acc[NR];
     for (;;) {
 #pragma unroll
         for (int r = 0; r < NR; ++r) acc[r] = im_u128{0ull, 0ull};
-        int emax = -100000;
+        int emax = 0;
         // K C C of reaction q, from its reactants' word and its rate constant
         auto product = [&](uint32_t w, double k, im_u64& Q, uint32_t& e) {
             im_split_k(k, Q, e);
@@ -411,15 +421,12 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                     if (U < (1ll << 54)) {  // small beside its terms: the fractions are too coarse
                         Md = int_row_dot_slow(M, row, S);
                         im_split(Md, mm, em);
+                        Md *= rho;
                     } else {
                         const int z = __clzll(U);
                         mm = (im_u64)U << (z - 1);
                         em = (uint32_t)(M.effX[row] + eT + 5 - z);
-                        if (q >= nF) {
-                            const double d = (double)mm;  // [2^62, 2^63]
-                            Md = __hiloint2double(__double2hiint(d) + (((int)em - IM_BIAS) << 20),
-                                                  __double2loint(d));
-                        }
+                        if (q >= nF) Md = im_round(mm, (int)em - IM_BIAS, false) * rho;
                     }
                     if (q >= nF) {
                         im_split(falloff_factor(__dmul_rn(Kc[nR + (q - nF)], Md)), mm, em);
@@ -427,6 +434,18 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                     }
                     Q = im_mul(Q, mm);
                     e += em - (uint32_t)(IM_BIAS - 64);
+                }
+                // the rate is rho^2 of what a plain reaction of two gives here
+                if (q >= nP || M.imLow) {
+                    int p = ((w & 0xffffu) != 0u) + (w >> 16 != 0u) + (q >= nP && q < nF) - 2;
+                    for (; p > 0; --p) {
+                        Q = im_mul(Q, mr);
+                        e += er - (uint32_t)(IM_BIAS - 64);
+                    }
+                    for (; p < 0; ++p) {
+                        Q = im_mul(Q, mi);
+                        e += ei - (uint32_t)(IM_BIAS - 64);
+                    }
                 }
                 store(Q, e, q - q0);
             }
@@ -477,18 +496,18 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         }
         emax = grp.imax(emax);
         if (emax >= IM_OUT) {  // a falloff factor that is not finite
-            int_general<NR, G>(M, S, Kc, c, invrho, out, lane, grp);
+            int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
             return;
         }
-        const bool fits = emax <= scale + IM_GUARD;
         const int s0 = scale;
-        if (!fits || emax < scale - IM_SLACK) scale = max(emax, 0);
+        const bool fits = emax <= s0 + IM_GUARD && emax >= s0 - IM_SLACK;
+        scale = emax;
         if (fits) {
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int i = lane + G * r;
-                // a word's unit at e = s0: 2^(128 + s0 - 3 IM_BIAS - IM_UP)
-                out[r] = i < nS ? __dmul_rn(im_double(acc[r], 128 + s0 - 3 * IM_BIAS - IM_UP), wr[r]) : 0.0;
+                // a word's unit at e = s0: 2^(128 + s0 - 2 * 64 - 3 IM_BIAS - IM_UP)
+                out[r] = i < nS ? im_scaled(acc[r], s0 - 3 * IM_BIAS - IM_UP, M.imW[i].y, M.imWe[i].y, mr, (int)er) : 0.0;
             }
             grp.sync();  // the shared words are rewritten by the next evaluation
             return;

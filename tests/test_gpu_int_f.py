@@ -91,3 +91,32 @@ def test_sizes_against_oracle(nS, nR, method):
     else:
         same[:] = True
     assert err[:, same].max() <= 1e-8, err[:, same].max()
+
+
+@pytest.mark.parametrize("nS,nR", [(2, 1), (9, 38), (15, 31), (16, 33)])
+def test_lanes_per_cell_do_not_change_the_bits(nS, nR):
+    """A call of many cells gives each a quarter warp, one of few half a warp."""
+    m = Mech(nS, nR, 5 * nS + nR)
+    rng = np.random.default_rng(nS)
+    n, tiles = 37, 400
+    T, p = rng.uniform(900.0, 1800.0, n), 101325.0 * rng.uniform(0.5, 20.0, n)
+    Y = rng.uniform(0.0, 1.0, (nS, n))
+    if nS > 2:
+        Y[2, 5] = -0.05 * Y[:, 5].sum()
+    Y /= Y.sum(axis=0)
+    assert n * tiles > kin.WARP_MAX_CELLS_PER_SM * torch.cuda.get_device_properties(0).multi_processor_count
+    km = kin.Mechanism(m)
+    for sigma in (kin.SIGMA_POWER, kin.SIGMA_GERSHGORIN):
+        got = []
+        for k in (1, tiles):
+            Yd = dev(np.tile(Y, (1, k)))
+            st = torch.zeros(n * k, dtype=torch.uint8, device="cuda")
+            sta = torch.zeros((n * k, kin.NSTATS), dtype=torch.int32, device="cuda")
+            kin.integrate(km, dev(np.tile(T, k)), dev(np.tile(p, k)), Yd, 1e-7, 1e-6, 1e-10, kin.RKC, status=st,
+                          stats=sta, sigma=sigma)
+            torch.cuda.synchronize()
+            got.append((Yd.cpu().numpy(), st.cpu().numpy(), sta.cpu().numpy()))
+        one, many = got
+        assert np.array_equal(np.tile(one[0], (1, tiles)), many[0])
+        assert np.array_equal(np.tile(one[1], tiles), many[1]) and np.array_equal(np.tile(one[2], (tiles, 1)), many[2])
+    km.close()

@@ -83,7 +83,7 @@ def mechanism(name):
     return r, p, 17
 
 
-@pytest.mark.parametrize("G", [16, 32])
+@pytest.mark.parametrize("G", [8, 16, 32, 128])
 @pytest.mark.parametrize("chunk", [32, 128, 256])
 @pytest.mark.parametrize("name", ["h2_9sp_rkck", "h2co_13sp_rkc", "ch4_53sp_rkc_mixed", "one", "none", "hub",
                                   "random"])
