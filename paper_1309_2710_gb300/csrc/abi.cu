@@ -98,7 +98,8 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
 // 48-register kernels exist for single warps.
 int cell_lanes(const kin_opts* o, int nV, int threads, int64_t cells, int nsm)
 {
-    const bool f64 = o->method == KIN_RKC && o->precision == KIN_FP64 && !o->energy;
+    const bool int_f = o->precision == KIN_FP64 && !o->energy, f64 = int_f && o->method == KIN_RKC;
+    if (nV <= 16 && int_f && !o->occupancy && cells <= 8 * (int64_t)nsm) return 32;
     if (nV <= 16 && f64 && !o->occupancy && cells > (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return 8;
     if (nV <= 16) return o->method == KIN_RKCK || f64 ? 16 : 32;
     if (!f64 || o->occupancy || nV <= 32) return 32;
@@ -519,14 +520,15 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     // the integer FP64 f (int_tables.h), for each group size that the mechanism
     // can take; eight rounds of reactions a chunk, so that the words of a
     // 53-species / 634-reaction cell (7.4 KB for a warp) leave room for 16 warps
-    // per SM beside the tables in L1
+    // per SM beside the tables in L1, and sixteen across warps, whose barriers
+    // cost more than the shared memory
     IntGather ig[INT_NTAB];
     size_t oIg[INT_NTAB][4];
     const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128};
     const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS > 32 && nS <= 64, nS > 64};
     for (int v = 0; v < INT_NTAB; ++v) {
         if (!ig_use[v]) continue;
-        const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, 8 * ig_lanes[v])));
+        const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, (ig_lanes[v] > 32 ? 16 : 8) * ig_lanes[v])));
         ig[v] = build_int_gather(nS, nR, ptr.data(), crxp.data(), cnu.data(), chunk, ig_lanes[v]);
         oIg[v][0] = put(ig[v].step0.data(), 4 * ig[v].step0.size());
         oIg[v][1] = put(ig[v].ent.data(), 4 * ig[v].ent.size());

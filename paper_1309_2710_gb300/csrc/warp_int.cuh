@@ -72,6 +72,24 @@ struct Group {
         if constexpr (G <= 32) __syncwarp(mask);
         else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / G), "n"(G) : "memory");
     }
+    // sync, and whether v holds for any of the group's lanes
+    __device__ __forceinline__ bool sync_any(bool v) const
+    {
+        if constexpr (G <= 32) {
+            const bool a = __any_sync(mask, v);
+            __syncwarp(mask);
+            return a;
+        } else {
+            int a;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, %3, p;\n\t"
+                "selp.s32 %0, 1, 0, q;\n\t}"
+                : "=r"(a)
+                : "r"((int)v), "r"(1 + (int)threadIdx.x / G), "n"(G)
+                : "memory");
+            return a != 0;
+        }
+    }
     __device__ __forceinline__ double* next_set()
     {
         double* b = red + set * set_words;
@@ -273,10 +291,11 @@ __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, 
     grp.sync();
 }
 
-// f for the group's cell. `scale` is the exponent of the largest rate of the
-// cell's previous evaluation (kept by the caller, any value at the first); an
-// evaluation whose largest is more than IM_GUARD octaves above it or IM_SLACK
-// below is repeated with its own. kfin: the cell's rate constants are finite.
+// f for the group's cell. `scale` is the exponent that the fixed-point words are
+// placed by, kept by the caller from one evaluation of the cell to the next
+// (any value at the first); an evaluation whose largest rate is more than
+// IM_GUARD octaves above it or IM_SLACK below is repeated with that rate's. The
+// barriers around the gather carry the two tests. kfin: the cell's rate constants are finite.
 template <int NR, int G>
 __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I, const IntSmem& S, const double* Kc,
                                                bool kfin, double Ctot, double invCtot, int& scale,
@@ -313,10 +332,6 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
     const int eT = (int)(top >> 20);
     // finite, and no species below -2^-9 of the total
     in = in && top - 0x00100000u < 0x7fe00000u && neg + 9 <= eT + 64;
-    if (!grp.all(in)) {
-        int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
-        return;
-    }
     im_u64 mr, mi = 0ull;  // rho and 1 / rho
     uint32_t er, ei = 0u;
     im_split_k(rho, mr, er);
@@ -342,13 +357,17 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
             S.CF[i] = make_int2(0, 0);
         }
     }
-    grp.sync();
+    if (grp.sync_any(!in)) {
+        int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
+        return;
+    }
     const int nP = nR - nM, nF = nR - M.nFO;
     im_u128 acc[NR];
     for (;;) {
 #pragma unroll
         for (int r = 0; r < NR; ++r) acc[r] = im_u128{0ull, 0ull};
         int emax = 0;
+        bool over = false, under = false;
         // K C C of reaction q, from its reactants' word and its rate constant
         auto product = [&](uint32_t w, double k, im_u64& Q, uint32_t& e) {
             im_split_k(k, Q, e);
@@ -459,7 +478,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
             uint32_t en[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) en[j] = j < K ? ent[G * j] : (uint32_t)I.chunk;
-            grp.sync();
+            over = grp.sync_any(emax > scale + IM_GUARD);
             im_u128 w{0ull, 0ull};
 #pragma unroll 1
             for (int k = 0; k < K; k += 4) {
@@ -481,7 +500,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                     }
                 }
             }
-            grp.sync();
+            under = !grp.sync_any(emax >= scale - IM_SLACK);
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const ulonglong2* p = S.P + (part[r] >> 16);
@@ -494,24 +513,24 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                 }
             }
         }
+        if (!over && !under) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int i = lane + G * r;
+                // a word's unit at e = scale: 2^(128 + scale - 2 * 64 - 3 IM_BIAS - IM_UP)
+                out[r] = i < nS ? im_scaled(acc[r], scale - 3 * IM_BIAS - IM_UP, M.imW[i].y, M.imWe[i].y, mr, (int)er) : 0.0;
+            }
+            // the shared words are rewritten by the next evaluation (across
+            // warps, only after the barrier of its mixture sum)
+            if constexpr (G <= 32) grp.sync();
+            return;
+        }
         emax = grp.imax(emax);
         if (emax >= IM_OUT) {  // a falloff factor that is not finite
             int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
             return;
         }
-        const int s0 = scale;
-        const bool fits = emax <= s0 + IM_GUARD && emax >= s0 - IM_SLACK;
         scale = emax;
-        if (fits) {
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int i = lane + G * r;
-                // a word's unit at e = s0: 2^(128 + s0 - 2 * 64 - 3 IM_BIAS - IM_UP)
-                out[r] = i < nS ? im_scaled(acc[r], s0 - 3 * IM_BIAS - IM_UP, M.imW[i].y, M.imWe[i].y, mr, (int)er) : 0.0;
-            }
-            grp.sync();  // the shared words are rewritten by the next evaluation
-            return;
-        }
     }
 }
 
