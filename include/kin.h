@@ -76,10 +76,13 @@ extern "C" {
 #define KIN_LAYOUT_AUTO 0 /* library choice: KIN_LAYOUT_WARP when n_reactions >
                              KIN_WARP_MIN_REACTIONS or the call has fewer than
                              KIN_WARP_MAX_CELLS_PER_SM cells per SM of the device (too
-                             few to give every lane a cell); also below
-                             KIN_WARP_FP64_MAX_CELLS_PER_SM for isothermal FP64 RKC on at
-                             most 16 species, unless a launch shape, staging, register
-                             budget or f evaluation is asked for; else KIN_LAYOUT_LANE */
+                             few to give every lane a cell); in FP64, unless a launch
+                             shape, staging, register budget or f evaluation is asked
+                             for, also RKC on 17 to 32 state components, both methods
+                             with the energy equation on at most 16, and isothermal
+                             calls on at most 16 species below
+                             KIN_WARP_RKC_MAX_CELLS_PER_SM or
+                             KIN_WARP_RKCK_MAX_CELLS_PER_SM; else KIN_LAYOUT_LANE */
 #define KIN_LAYOUT_LANE 1 /* one lane integrates one cell (the paper's thread-per-ODE
                              design, Section 3): per-cell arrays in the workspace or in
                              shared memory (kin_opts.staging) */
@@ -94,7 +97,8 @@ extern "C" {
                              to 256 */
 #define KIN_WARP_MIN_REACTIONS 256
 #define KIN_WARP_MAX_CELLS_PER_SM 64
-#define KIN_WARP_FP64_MAX_CELLS_PER_SM 512
+#define KIN_WARP_RKC_MAX_CELLS_PER_SM 704
+#define KIN_WARP_RKCK_MAX_CELLS_PER_SM 320
 
 /* how the lane-per-cell layout evaluates f (kin_opts.feval) */
 #define KIN_FEVAL_AUTO 0      /* the generated f for an isothermal call of at least

@@ -71,17 +71,24 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
     if (o->layout != KIN_LAYOUT_AUTO) return o->layout;
     if (m->nR > KIN_WARP_MIN_REACTIONS) return KIN_LAYOUT_WARP;
     if (cells < (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return KIN_LAYOUT_WARP;
-    // Isothermal FP64 RKC on small mechanisms: the warp layout's integer f, four
-    // cells to a warp, beats a lane per cell until each lane of the GPU has one
-    // (13 species: 30,000 cells 14.6 ms against 39.0, 60,000 29.1 against 52.4,
-    // 262,144 128 against 122 with the generated f). A call that names a shape or
-    // form of the lane layout keeps it.
+    // FP64 on small mechanisms: the warp layout's integer f beats a lane per cell
+    // until every lane of the GPU has more than one. GB300, warp against lane:
+    //   13 species RKC: 30,000 cells 14.6 against 39.0 ms, 100,000 51.3 against
+    //     55.3, 131,072 67.4 against 64.3 (generated f from 65,536 cells on);
+    //   9 species RKCK: 20,000 cells 1.85 against 3.24, 40,000 3.51 against 4.20,
+    //     80,000 6.83 against 5.69;
+    //   24 species RKC: 12,000 cells 10.8 against 94.9, 150,000 134 against 185;
+    //   energy equation, 13 species RKC: 20,000 cells 13.3 against 68.2, 200,000
+    //     128 against 269; 9 species RKCK: 80,000 cells 13.6 against 17.4.
+    // A call that names a shape or form of the lane layout keeps it.
     const bool free_shape = o->block_threads == 0 && o->blocks_per_sm == 0 && o->staging == KIN_STAGE_GLOBAL &&
                             o->occupancy == KIN_OCC_DEFAULT && o->feval == KIN_FEVAL_AUTO;
-    if (full && free_shape && o->method == KIN_RKC && o->precision == KIN_FP64 && !o->energy && m->nS <= 16 &&
-        cells < (int64_t)KIN_WARP_FP64_MAX_CELLS_PER_SM * nsm)
-        return KIN_LAYOUT_WARP;
-    return KIN_LAYOUT_LANE;
+    const int nV = m->nS + o->energy;
+    if (!full || !free_shape || o->precision != KIN_FP64 || nV > 32) return KIN_LAYOUT_LANE;
+    const bool rkc = o->method == KIN_RKC;
+    if (nV > 16) return rkc ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
+    const int64_t most = rkc ? KIN_WARP_RKC_MAX_CELLS_PER_SM : KIN_WARP_RKCK_MAX_CELLS_PER_SM;
+    return o->energy || cells < most * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
 }
 
 // Lanes that integrate one cell in the warp layout: half a warp for states of
@@ -98,7 +105,7 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
 // 48-register kernels exist for single warps.
 int cell_lanes(const kin_opts* o, int nV, int threads, int64_t cells, int nsm)
 {
-    const bool int_f = o->precision == KIN_FP64 && !o->energy, f64 = int_f && o->method == KIN_RKC;
+    const bool int_f = o->precision == KIN_FP64, f64 = int_f && o->method == KIN_RKC;
     if (nV <= 16 && int_f && !o->occupancy && cells <= 8 * (int64_t)nsm) return 32;
     if (nV <= 16 && f64 && !o->occupancy && cells > (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return 8;
     if (nV <= 16) return o->method == KIN_RKCK || f64 ? 16 : 32;
@@ -525,7 +532,7 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     IntGather ig[INT_NTAB];
     size_t oIg[INT_NTAB][4];
     const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128};
-    const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS > 32 && nS <= 64, nS > 64};
+    const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS >= 32 && nS <= 64, nS >= 64};
     for (int v = 0; v < INT_NTAB; ++v) {
         if (!ig_use[v]) continue;
         const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, (ig_lanes[v] > 32 ? 16 : 8) * ig_lanes[v])));
@@ -553,6 +560,21 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     int imLow = 0;
     for (int j = 0; j < nR; ++j)
         if ((d->reac[2 * j] >= 0) + (d->reac[2 * j + 1] >= 0) + (rxn[j].type == KIN_RXN_THIRD_BODY) < 2) imLow = 1;
+    std::vector<double> arr(3 * nR), arr0(3 * nFO);
+    for (int q = 0; q < nR; ++q) {
+        const int j = perm[q], fo = rxnp[q].fo;
+        arr[q] = d->lnA[j];
+        arr[nR + q] = d->beta[j];
+        arr[2 * nR + q] = EaR[j];
+        if (fo < 0) continue;
+        arr0[fo] = lnA0[j];
+        arr0[nFO + fo] = beta0[j];
+        arr0[2 * nFO + fo] = Ea0R[j];
+    }
+    uint64_t ex2[64], lnc[128];
+    int_exp_log_tables(ex2, lnc);
+    const size_t oArr = put(arr.data(), 8 * arr.size()), oArr0 = put(arr0.data(), 8 * arr0.size());
+    const size_t oEx2 = put(ex2, sizeof(ex2)), oLnc = put(lnc, sizeof(lnc));
     const size_t oImW = put(imW.data(), 8 * imW.size()), oImWe = put(imWe.data(), 4 * imWe.size());
     const size_t oEffI = put(effI.data(), 4 * effI.size()), oEffX = put(effX.data(), 4 * effX.size());
     // the segmented FP32 gather of the 32-lane isothermal f, where the packed
@@ -569,14 +591,15 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     // thermochemistry for the energy equation: cp, cp/W, Hf
     const bool thermo = d->cp && d->Hf;
     if ((d->cp != nullptr) != (d->Hf != nullptr)) return fail(KIN_EINVAL, "give both cp and Hf, or neither");
-    std::vector<double> cpW(thermo ? nS : 0);
+    std::vector<double> cpW(thermo ? nS : 0), HfW(thermo ? nS : 0);
     for (int i = 0; thermo && i < nS; ++i) {
         if (!finite_pos(d->cp[i])) return fail(KIN_EINVAL, "cp[%d] must be finite and > 0", i);
         if (!std::isfinite(d->Hf[i])) return fail(KIN_EINVAL, "Hf[%d] must be finite", i);
         cpW[i] = d->cp[i] / d->W[i];
+        HfW[i] = d->Hf[i] / d->W[i];
     }
     const size_t oCp = thermo ? put(d->cp, 8 * nS) : 0, oCpW = thermo ? put(cpW.data(), 8 * nS) : 0;
-    const size_t oHf = thermo ? put(d->Hf, 8 * nS) : 0;
+    const size_t oHf = thermo ? put(d->Hf, 8 * nS) : 0, oHfW = thermo ? put(HfW.data(), 8 * nS) : 0;
     const size_t oTab = put(nullptr, 0);
     const size_t tabBytes = sizeof(double) * RKC_TAB_S * RKC_TAB_S * RKC_TAB_W;
     host.resize(oTab + tabBytes, 0);
@@ -616,6 +639,10 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     }
     M.effI = (const int4*)(b + oEffI);
     M.effX = (const int32_t*)(b + oEffX);
+    M.arr = (const double*)(b + oArr);
+    M.arr0 = (const double*)(b + oArr0);
+    M.ex2 = (const unsigned long long*)(b + oEx2);
+    M.lnc = (const ulonglong2*)(b + oLnc);
     M.imW = (const ulonglong2*)(b + oImW);
     M.imWe = (const int2*)(b + oImWe);
     M.imLow = imLow;
@@ -630,6 +657,7 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.cp = thermo ? (const double*)(b + oCp) : nullptr;
     M.cpW = thermo ? (const double*)(b + oCpW) : nullptr;
     M.Hf = thermo ? (const double*)(b + oHf) : nullptr;
+    M.HfW = thermo ? (const double*)(b + oHfW) : nullptr;
     m->nS = nS; m->nR = nR; m->nM = nM;
     m->thermo = thermo;
     if (gen_eligible(nS, nR)) m->gen_src = gen_f_source(d);
@@ -885,8 +913,12 @@ int kin_rates(const kin_mech* m, int64_t cells, const double* T, const double* p
     if (!ws || ((uintptr_t)ws) % 256) return fail(KIN_EINVAL, "workspace must be non-NULL and 256-byte aligned");
     if (ws_size < need) return fail(KIN_ENOMEM, "workspace has %lld bytes, needs %lld", (long long)ws_size, (long long)need);
     if (!is_device_ptr(ws)) return fail(KIN_EINVAL, "workspace must be device memory");
-    cudaError_t e = launch_rates(m->dev, cells, T, p, Y, ldY, dYdt, precision, ws, g.nslots,
-                                 g.blocks, g.threads, (cudaStream_t)stream);
+    int nsm = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
+    e = precision == KIN_MIXED ? launch_rates_f32(m->dev, cells, T, p, Y, ldY, dYdt, ws, g.nslots, g.blocks, g.threads,
+                                                  (cudaStream_t)stream)
+                               : launch_rates_f64(m->dev, cells, T, p, Y, ldY, dYdt, nsm, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "rates launch");
     return KIN_OK;
 }

@@ -122,6 +122,18 @@ inline uint64_t int_split(long double v, int* e)
     return m;
 }
 
+// The tables of im_exp and im_log (intf.cuh).
+inline void int_exp_log_tables(uint64_t* ex2, uint64_t* lnc)
+{
+    for (int i = 0; i < 64; ++i) {
+        ex2[i] = (uint64_t)llroundl(ldexpl(exp2l(i / 64.0L), 61)) << 1;
+        // far enough above for m c_i >= 1 after the product's truncation
+        const uint64_t c = (uint64_t)ceill(ldexpl(64.0L / (64 + i), 62)) + 16;
+        lnc[2 * i] = c;
+        lnc[2 * i + 1] = (uint64_t)llroundl(ldexpl(-logl(ldexpl((long double)c, -62)), 59));
+    }
+}
+
 // A row's efficiencies as 55-bit integers: hi (30 bits, signed) and lo (25
 // bits) of round(eff 2^(54 - x)). Returns x.
 inline int int_efficiencies(int nS, const double* eff, int32_t* hi, int32_t* lo)

@@ -1,5 +1,5 @@
 // kernels.cu -- non-template kernels and host launchers of the integrator:
-// the f-alone kernel, the RKC coefficient table, the longest-first bucket
+// f alone in mixed precision, the RKC coefficient table, the longest-first bucket
 // sort, workspace layout, and dispatch to the per-method/precision
 // instantiations (inst_*.cu).
 #include "kernels.cuh"
@@ -41,23 +41,22 @@ __global__ void bucket_scatter_kernel(const __grid_constant__ Launch L)
     }
 }
 
-// ------------------------------------------------------------- f alone ---
-template <typename R>
+// ------------------------------------- f alone in mixed precision -------
 __global__ void rates_kernel(MechDev M, int64_t cells, const double* __restrict__ T,
                              const double* __restrict__ p, const double* Y, int64_t ldY,
-                             double* dYdt, void* lane_r, void* cell_k, int64_t nslots)
+                             double* dYdt, float* lane_r, float* cell_k, int64_t nslots)
 {
     const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (slot >= nslots) return;
-    R* rb = reinterpret_cast<R*>(lane_r) + slot;
-    Lane<R> C{rb, (int32_t)nslots}, OM{rb + (int64_t)M.nS * nslots, (int32_t)nslots};
+    float* rb = lane_r + slot;
+    Lane<float> C{rb, (int32_t)nslots}, OM{rb + (int64_t)M.nS * nslots, (int32_t)nslots};
     for (int64_t c = slot; c < cells; c += nslots) {
-        Lane<R> K{reinterpret_cast<R*>(cell_k) + c, (int32_t)cells};
-        Lane<R> KR{reinterpret_cast<R*>(cell_k) + (int64_t)M.nR * cells + c, (int32_t)cells};
-        rate_constants<R>(M, T[c], K, KR);
+        Lane<float> K{cell_k + c, (int32_t)cells};
+        Lane<float> KR{cell_k + (int64_t)M.nR * cells + c, (int32_t)cells};
+        rate_constants<float>(M, T[c], K, KR);
         const double Ctot = p[c] * 1e-6 / (R_GAS * T[c]);
-        feval<R>(M, Ctot, 1.0 / Ctot, K, KR, C, OM,
-                 Lane<double>{const_cast<double*>(Y) + c, (int32_t)ldY}, Lane<double>{dYdt + c, (int32_t)ldY});
+        feval<float>(M, Ctot, 1.0 / Ctot, K, KR, C, OM,
+                     Lane<double>{const_cast<double*>(Y) + c, (int32_t)ldY}, Lane<double>{dYdt + c, (int32_t)ldY});
     }
 }
 
@@ -187,18 +186,14 @@ cudaError_t launch_sort(Launch& L, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_rates(const MechDev& M, int64_t cells, const double* T, const double* p,
-                         const double* Y, int64_t ldY, double* dYdt, int precision, void* ws,
-                         int64_t nslots, int blocks, int threads, cudaStream_t st)
+cudaError_t launch_rates_f32(const MechDev& M, int64_t cells, const double* T, const double* p,
+                             const double* Y, int64_t ldY, double* dYdt, void* ws, int64_t nslots,
+                             int blocks, int threads, cudaStream_t st)
 {
-    const WsLayout w = ws_layout(M, precision, KIN_SIGMA_GERSHGORIN, 0, nslots, cells);
+    const WsLayout w = ws_layout(M, KIN_MIXED, KIN_SIGMA_GERSHGORIN, 0, nslots, cells);
     char* b = (char*)ws;
-    if (precision == KIN_MIXED)
-        rates_kernel<float><<<blocks, threads, 0, st>>>(M, cells, T, p, Y, ldY, dYdt, b + w.lane_r,
-                                                        b + w.cell_k, nslots);
-    else
-        rates_kernel<double><<<blocks, threads, 0, st>>>(M, cells, T, p, Y, ldY, dYdt, b + w.lane_r,
-                                                         b + w.cell_k, nslots);
+    rates_kernel<<<blocks, threads, 0, st>>>(M, cells, T, p, Y, ldY, dYdt, (float*)(b + w.lane_r),
+                                             (float*)(b + w.cell_k), nslots);
     return cudaGetLastError();
 }
 

@@ -89,6 +89,10 @@ struct MechDev {
     IntDev ig[INT_NTAB];
     const int4* effI;      // [(nS + 1) / 2][nM] integer efficiencies {hi, lo} of two species
     const int32_t* effX;   // [nM] their exponents
+    const double* arr;     // [3][nR] ln A, beta, E / R in permutation order
+    const double* arr0;    // [3][nFO] the low-pressure limits'
+    const unsigned long long* ex2;  // tables of im_exp and im_log
+    const ulonglong2* lnc;
     const ulonglong2* imW; // [nS] 63-bit mantissas of 1 / W and W
     const int2* imWe;      // [nS] their exponents
     int imLow;             // 1: a reaction of fewer than two factors of concentration
@@ -112,6 +116,7 @@ struct MechDev {
     const double* cp;      // [nS] J/(mol K)
     const double* cpW;     // [nS] cp_i / W_i, J/(g K)
     const double* Hf;      // [nS] J/mol at T_REF
+    const double* HfW;     // [nS] Hf_i / W_i, J/g
 };
 
 // One instance of a batched launch (device pointers).
@@ -170,9 +175,11 @@ WsLayout ws_layout(const MechDev& M, int precision, int sigma_method, int energy
 cudaError_t launch_integrate(Launch& L, int staging, int occupancy, int blocks, int threads,
                              cudaStream_t st);
 size_t smem_bytes(const MechDev& M, int precision, int threads, int staging);
-cudaError_t launch_rates(const MechDev& M, int64_t cells, const double* T, const double* p,
-                         const double* Y, int64_t ldY, double* dYdt, int precision, void* ws,
-                         int64_t nslots, int blocks, int threads, cudaStream_t st);
+cudaError_t launch_rates_f32(const MechDev& M, int64_t cells, const double* T, const double* p,
+                             const double* Y, int64_t ldY, double* dYdt, void* ws, int64_t nslots,
+                             int blocks, int threads, cudaStream_t st);
+cudaError_t launch_rates_f64(const MechDev& M, int64_t cells, const double* T, const double* p, const double* Y,
+                             int64_t ldY, double* dYdt, int nsm, cudaStream_t st);
 cudaError_t launch_rkc_table(double* tab, cudaStream_t st);
 // Per method/precision instantiations (inst_*.cu) and the bucket sort.
 cudaError_t launch_rkc_f64(Launch& L, int stg, int occ, int blocks, int threads, cudaStream_t st);

@@ -113,7 +113,7 @@ __host__ __device__ __forceinline__ int warp_smem_elems(const MechDev& M)
 template <typename R, bool EN, int G>
 __host__ __device__ __forceinline__ int warp_f_words(const MechDev& M)
 {
-    return EN || sizeof(R) == 4 ? warp_smem_elems(M) : int_smem_words(M, int_tab<G>(M));
+    return sizeof(R) == 4 ? warp_smem_elems(M) : int_smem_words(M, int_tab<G>(M));
 }
 
 // The cell's rate constants in shared memory too: f reads every k_j once per
@@ -280,10 +280,6 @@ __device__ __forceinline__ void warp_feval(const MechDev& M, const KT* Kc, R* C,
     __syncwarp(mask);  // C and OM are rewritten by the next evaluation
 }
 
-// Element r of a register vector for a warp-uniform r.
-template <int NR>
-__device__ __forceinline__ double reg_get(const double (&v)[NR], int r);
-
 // f with the energy equation (Eqs. (E:mass), (E:energy)) for the warp's cell:
 // state component nS is T (lane nS % 32, slot nS / 32). Each lane computes the
 // rate constants of its reactions from T (they follow T at every
@@ -372,17 +368,6 @@ __device__ __forceinline__ void warp_feval_energy(const MechDev& M, double p, R*
     __syncwarp(mask);  // C and OM are rewritten by the next evaluation
 }
 
-// Element r of a register vector for a warp-uniform r.
-template <int NR>
-__device__ __forceinline__ double reg_get(const double (&v)[NR], int r)
-{
-    double o = v[0];
-#pragma unroll
-    for (int q = 1; q < NR; ++q)
-        if (r == q) o = v[q];
-    return o;
-}
-
 template <typename R, int NR, bool EN, int G>
 struct WarpRKC {
     const Launch& L;
@@ -442,27 +427,31 @@ struct WarpRKC {
 
     __device__ __forceinline__ void f(const double (&in)[NR], double (&o)[NR])
     {
-        if constexpr (EN) warp_feval_energy<R, NR, G>(M, p, C, OM, in, o, lane, mask);
-        else if constexpr (sizeof(R) == 4) warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
-        else f64(in, o);
+        if constexpr (sizeof(R) == 8) f64(in, o);
+        else if constexpr (EN) warp_feval_energy<R, NR, G>(M, p, C, OM, in, o, lane, mask);
+        else warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
         nfe++;
     }
 
-    // The isothermal f of the FP64 path.
+    // f of the FP64 path (with the energy equation Ctot and invCtot hold p / R and
+    // its reciprocal).
     __device__ __forceinline__ void f64(const double (&in)[NR], double (&o)[NR])
     {
         const IntDev& I = int_tab<G>(M);
-        warp_feval_int<NR, G>(M, I, IntSmem(M, I, C64), Kc, kfin, Ctot, invCtot, scale, in, o, lane, grp);
+        const IntSmem S(M, I, C64);
+        if constexpr (EN) warp_feval_int_energy<NR, G>(M, I, S, Ctot, invCtot, scale, in, o, lane, grp);
+        else
+            warp_feval_int<NR, G, false>(M, I, S, RateSource{reinterpret_cast<const double*>(Kc), 0.0, 0.0}, kfin, Ctot,
+                                         invCtot, scale, in, o, lane, grp);
     }
 
     // f in FP64 for the spectral-radius estimates (FP32 rounding noise in
     // f(y + v) - f(y) would swamp the difference; see SIG_SQRT_U).
     __device__ __forceinline__ void fs(const double (&in)[NR], double (&o)[NR])
     {
-        if constexpr (EN) warp_feval_energy<double, NR, G>(M, p, C64, OM64, in, o, lane, mask);
-        else if constexpr (sizeof(R) == 4)
-            warp_feval<double, R, NR, G>(M, Kc, C64, OM64, Ctot, invCtot, in, o, lane, mask);
-        else f64(in, o);
+        if constexpr (sizeof(R) == 8) f64(in, o);
+        else if constexpr (EN) warp_feval_energy<double, NR, G>(M, p, C64, OM64, in, o, lane, mask);
+        else warp_feval<double, R, NR, G>(M, Kc, C64, OM64, Ctot, invCtot, in, o, lane, mask);
         nfe++;
         nfs++;
     }
@@ -966,7 +955,7 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
         const InstDev& I = L.inst[ii];
         const int64_t c = g - L.start[ii];
         const double T = I.T[c], p = I.p[c];
-        W.Ctot = ddiv(p * 1e-6, R_GAS * T);
+        W.Ctot = ddiv(p * 1e-6, EN && sizeof(R) == 8 ? R_GAS : R_GAS * T);
         W.invCtot = ddiv(1.0, W.Ctot);
         W.CtotR = (R)W.Ctot;
         W.invCtotR = (R)W.invCtot;
@@ -1066,13 +1055,14 @@ __device__ __forceinline__ uint8_t warp_load_cell(WarpRKC<R, NR, EN, G>& W, cons
     const uint8_t pre = L.cell_st[g];
     if (pre != 0) return pre;  // Y stays as given
     const double T = I.T[c], p = I.p[c];
-    W.Ctot = ddiv(p * 1e-6, R_GAS * T);
+    W.Ctot = ddiv(p * 1e-6, EN && sizeof(R) == 8 ? R_GAS : R_GAS * T);
     W.invCtot = ddiv(1.0, W.Ctot);
     W.CtotR = (R)W.Ctot;
     W.invCtotR = (R)W.invCtot;
     W.atol = I.atol;
     W.rtol = I.rtol;
     W.p = p;
+    W.scale = 0;
     if constexpr (EN) {
         W.Kc = nullptr;
     } else {
@@ -1085,7 +1075,6 @@ __device__ __forceinline__ uint8_t warp_load_cell(WarpRKC<R, NR, EN, G>& W, cons
                 if (W.Ks) W.Ks[q] = k;  // staged (the last f of the previous cell ended in a sync)
             }
         if (sizeof(R) == 8) W.kfin = W.grp.all(kfin);
-        W.scale = 0;
         if (W.Ks) W.grp.sync();
         W.Kc = W.Ks ? W.Ks : kg;
     }
@@ -1239,11 +1228,17 @@ struct WarpRKCK {
 
     __device__ __forceinline__ void f(const double (&in)[NR], double (&o)[NR])
     {
-        if constexpr (EN) warp_feval_energy<R, NR, G>(M, p, C, OM, in, o, lane, mask);
-        else if constexpr (sizeof(R) == 4) warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
-        else
-            warp_feval_int<NR, G>(M, int_tab<G>(M), IntSmem(M, int_tab<G>(M), base), Kc, kfin, Ctot, invCtot,
-                                     scale, in, o, lane, grp);
+        if constexpr (sizeof(R) == 4) {
+            if constexpr (EN) warp_feval_energy<R, NR, G>(M, p, C, OM, in, o, lane, mask);
+            else warp_feval<R, R, NR, G>(M, Kc, C, OM, CtotR, invCtotR, in, o, lane, mask);
+        } else {
+            const IntDev& I = int_tab<G>(M);
+            const IntSmem S(M, I, base);
+            if constexpr (EN) warp_feval_int_energy<NR, G>(M, I, S, Ctot, invCtot, scale, in, o, lane, grp);
+            else
+                warp_feval_int<NR, G, false>(M, I, S, RateSource{reinterpret_cast<const double*>(Kc), 0.0, 0.0}, kfin,
+                                             Ctot, invCtot, scale, in, o, lane, grp);
+        }
         nfe++;
     }
 
@@ -1339,7 +1334,7 @@ __global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const _
         const InstDev& I = L.inst[ii];
         const int64_t c = g - L.start[ii];
         const double T = I.T[c], p = I.p[c];
-        W.Ctot = ddiv(p * 1e-6, R_GAS * T);
+        W.Ctot = ddiv(p * 1e-6, EN && sizeof(R) == 8 ? R_GAS : R_GAS * T);
         W.invCtot = ddiv(1.0, W.Ctot);
         W.CtotR = (R)W.Ctot;
         W.invCtotR = (R)W.invCtot;
@@ -1470,7 +1465,7 @@ __host__ __device__ inline int warp_nr(int n, int G)
 
 // The instantiation for groups of `lanes` lanes: FN<NR, G>.
 #define KIN_WARP_DISPATCH(FN, n, lanes)                                     \
-    if constexpr (sizeof(R) == 8 && !EN) {                                  \
+    if constexpr (sizeof(R) == 8) {                                         \
         if constexpr (OCC == 0) {                                           \
             if (lanes == 8) return FN(2, 8);                                \
         }                                                                   \

@@ -236,11 +236,28 @@ static __device__ __noinline__ double int_row_dot_slow(const MechDev& M, int row
     return int_row_dot(M, row, [&](int k) { return int_conc(S, k); });
 }
 
+// Where f's rate constants come from: stored (isothermal), or exp(ln A + beta ln T
+// - (E / R) / T) at this temperature (K null).
+struct RateSource {
+    const double* K;
+    double lnT, invT;
+};
+
+// The exponents of reaction position q and falloff ordinal fo.
+__device__ __forceinline__ double rate_exponent(const MechDev& M, int q, const RateSource& k)
+{
+    return fma(-M.arr[2 * M.nR + q], k.invT, fma(M.arr[M.nR + q], k.lnT, M.arr[q]));
+}
+__device__ __forceinline__ double low_exponent(const MechDev& M, int fo, const RateSource& k)
+{
+    return fma(-M.arr0[2 * M.nFO + fo], k.invT, fma(M.arr0[M.nFO + fo], k.lnT, M.arr0[fo]));
+}
+
 // sum_j nu_ij Omega_j of species i in plain FP64, one term after another, from
 // the concentrations c[k + 1] in shared memory (c[0] = 1): for states outside
 // the integer forms' range. Such states are trial points that blew up, so
 // this code is small rather than fast.
-static __device__ __noinline__ double int_general_sum(const MechDev& M, const double* Kc, const double* c, int i)
+static __device__ __noinline__ double int_general_sum(const MechDev& M, const RateSource& k, const double* c, int i)
 {
     const int nP = M.nR - M.nM, nF = M.nR - M.nFO;
     double w = 0.0;
@@ -248,13 +265,14 @@ static __device__ __noinline__ double int_general_sum(const MechDev& M, const do
     for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
         const int q = M.csrp_rxn[e];
         const uint32_t r = M.rxw[q];
-        double v = Kc[q] * c[r & 0xffffu] * c[r >> 16];
+        const double a = k.K ? 0.0 : rate_exponent(M, q, k);
+        double v = (k.K ? k.K[q] : exp(a)) * c[r & 0xffffu] * c[r >> 16];
         if (q >= nP) {
             const double Mc = int_row_dot(M, q - nP, [&](int k) { return c[k]; });
             if (q < nF) {
                 v *= Mc;
             } else {
-                const double Pr = Kc[M.nR + (q - nF)] * Mc;
+                const double Pr = (k.K ? k.K[M.nR + (q - nF)] : exp(low_exponent(M, q - nF, k) - a)) * Mc;
                 v *= ddiv(Pr, 1.0 + Pr);
             }
         }
@@ -274,7 +292,7 @@ __device__ __forceinline__ double falloff_factor(double Pr)
 
 // f of such a state, from its c_k / rho (the group's lanes together).
 template <int NR, int G>
-__device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, const double* Kc, const double (&c)[NR],
+__device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, const RateSource& k, const double (&c)[NR],
                                             double rho, double invrho, double (&out)[NR], int lane, const Group<G>& grp)
 {
     double* cs = reinterpret_cast<double*>(S.CM);
@@ -286,7 +304,7 @@ __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, 
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         const int i = lane + G * r;
-        out[r] = i < M.nS ? __dmul_rn(int_general_sum(M, Kc, cs, i), M.W[i] * invrho) : 0.0;
+        out[r] = i < M.nS ? __dmul_rn(int_general_sum(M, k, cs, i), M.W[i] * invrho) : 0.0;
     }
     grp.sync();
 }
@@ -296,10 +314,11 @@ __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, 
 // (any value at the first); an evaluation whose largest rate is more than
 // IM_GUARD octaves above it or IM_SLACK below is repeated with that rate's. The
 // barriers around the gather carry the two tests. kfin: the cell's rate constants are finite.
-template <int NR, int G>
-__device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I, const IntSmem& S, const double* Kc,
-                                               bool kfin, double Ctot, double invCtot, int& scale,
-                                               const double (&x)[NR], double (&out)[NR], int lane, Group<G>& grp)
+template <int NR, int G, bool AT_T>
+__device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I, const IntSmem& S,
+                                               const RateSource& rk, bool kfin, double Ctot, double invCtot,
+                                               int& scale, const double (&x)[NR], double (&out)[NR], int lane,
+                                               Group<G>& grp)
 {
     const int nS = M.nS, nR = M.nR, nM = M.nM;
     // c_k / rho = Y_k / W_k: in FP64 for the mixture sum, and as mantissa and
@@ -358,7 +377,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         }
     }
     if (grp.sync_any(!in)) {
-        int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
+        int_general<NR, G>(M, S, rk, c, rho, invCtot * s, out, lane, grp);
         return;
     }
     const int nP = nR - nM, nF = nR - M.nFO;
@@ -368,9 +387,8 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         for (int r = 0; r < NR; ++r) acc[r] = im_u128{0ull, 0ull};
         int emax = 0;
         bool over = false, under = false;
-        // K C C of reaction q, from its reactants' word and its rate constant
-        auto product = [&](uint32_t w, double k, im_u64& Q, uint32_t& e) {
-            im_split_k(k, Q, e);
+        // K C C of a reaction, from its reactants' word and its rate constant in Q, e
+        auto product = [&](uint32_t w, im_u64& Q, uint32_t& e) {
             const uint32_t a = w & 0xffffu, b = w >> 16;
             Q = im_mul(im_mul(S.CM[a], S.CM[b]), Q);
             e += S.CE[a] + S.CE[b];
@@ -389,25 +407,36 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         // the lane's reactions follow each other through the chunks, so the
         // next one's words are on their way while this one is formed
         uint32_t wn = 0;
-        double kn = 0.0;
-        if (lane < nR) {
-            wn = M.rxw[lane];
-            kn = Kc[lane];
-        }
+        double kn = 0.0, bn = 0.0, en0 = 0.0;
+        auto fetch = [&](int q) {
+            wn = M.rxw[q];
+            if constexpr (AT_T) {
+                kn = M.arr[q];
+                bn = M.arr[nR + q];
+                en0 = M.arr[2 * nR + q];
+            } else {
+                kn = rk.K[q];
+            }
+        };
+        if (lane < nR) fetch(lane);
 #pragma unroll 1
         for (int ch = 0, q0 = 0; ch < I.nchunk; ++ch, q0 += I.chunk) {
             const int q1 = min(nR, q0 + I.chunk);
 #pragma unroll 1
             for (int q = q0 + lane; q < q1; q += G) {
                 const uint32_t w = wn;
-                const double kq = kn;
-                if (q + G < nR) {
-                    wn = M.rxw[q + G];
-                    kn = Kc[q + G];
-                }
+                const double kq = kn, bq = bn, eq = en0;
+                if (q + G < nR) fetch(q + G);
                 im_u64 Q;
                 uint32_t e;
-                product(w, kq, Q, e);
+                double a = 0.0;
+                if constexpr (AT_T) {
+                    a = fma(-eq, rk.invT, fma(bq, rk.lnT, kq));
+                    if (!im_exp(M.ex2, a, Q, e)) emax = IM_OUT;
+                } else {
+                    im_split_k(kq, Q, e);
+                }
+                product(w, Q, e);
                 if (q >= nP) {
                     const int row = q - nP;
                     const int4* __restrict__ E = M.effI + row;
@@ -445,10 +474,19 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                         const int z = __clzll(U);
                         mm = (im_u64)U << (z - 1);
                         em = (uint32_t)(M.effX[row] + eT + 5 - z);
-                        if (q >= nF) Md = im_round(mm, (int)em - IM_BIAS, false) * rho;
+                        if (!AT_T && q >= nF) Md = im_round(mm, (int)em - IM_BIAS, false) * rho;
                     }
                     if (q >= nF) {
-                        im_split(falloff_factor(__dmul_rn(Kc[nR + (q - nF)], Md)), mm, em);
+                        double Pr;
+                        if constexpr (AT_T) {
+                            im_u64 km;
+                            uint32_t ke;
+                            if (!im_exp(M.ex2, low_exponent(M, q - nF, rk) - a, km, ke)) emax = IM_OUT;
+                            Pr = im_round(im_mul(km, mm), (int)ke + (int)(em & 0x7fffffffu) - 2 * IM_BIAS + 64, (int)em < 0) * rho;
+                        } else {
+                            Pr = __dmul_rn(rk.K[nR + (q - nF)], Md);
+                        }
+                        im_split(falloff_factor(Pr), mm, em);
                         if ((em & 0x7ffu) == 0x7ffu) emax = IM_OUT;
                     }
                     Q = im_mul(Q, mm);
@@ -527,11 +565,59 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         }
         emax = grp.imax(emax);
         if (emax >= IM_OUT) {  // a falloff factor that is not finite
-            int_general<NR, G>(M, S, Kc, c, rho, invCtot * s, out, lane, grp);
+            int_general<NR, G>(M, S, rk, c, rho, invCtot * s, out, lane, grp);
             return;
         }
         scale = emax;
     }
+}
+
+// Element r of a register vector for a warp-uniform r.
+template <int NR>
+__device__ __forceinline__ double reg_get(const double (&v)[NR], int r)
+{
+    double o = v[0];
+#pragma unroll
+    for (int q = 1; q < NR; ++q)
+        if (r == q) o = v[q];
+    return o;
+}
+
+// Rate constants' source at T.
+__device__ __forceinline__ RateSource rates_at(const MechDev& M, double T, double invT)
+{
+    return RateSource{nullptr, T >= 1.0 && T < 65536.0 ? im_log(M.lnc, T) : log(T), invT};
+}
+
+// f with the energy equation (Eqs. (E:mass), (E:energy)) for the group's cell:
+// state component nS is T. pR = p / R and its reciprocal in mol K / cm^3. The
+// species' enthalpies and heat capacities per mass multiply the species' own
+// rates: dT/dt = -(sum_i (Hf_i + cp_i (T - T_REF)) / W_i dY_i/dt) / sum_i Y_i cp_i / W_i.
+template <int NR, int G>
+__device__ __forceinline__ void warp_feval_int_energy(const MechDev& M, const IntDev& I, const IntSmem& S, double pR,
+                                                      double invpR, int& scale, const double (&x)[NR],
+                                                      double (&out)[NR], int lane, Group<G>& grp)
+{
+    const int nS = M.nS;
+    const double T = grp.from(reg_get(x, nS / G), nS % G), invT = Tab<double>::inv(T);
+    warp_feval_int<NR, G, true>(M, I, S, rates_at(M, T, invT), true, pR * invT, invpR * T, scale, x, out, lane, grp);
+    const double dT = T - T_REF;
+    double h[NR], c[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        h[r] = c[r] = 0.0;
+        if (i < nS) {
+            const double w = M.cpW[i];
+            h[r] = __dmul_rn(fma(w, dT, M.HfW[i]), out[r]);
+            c[r] = __dmul_rn(x[r], w);
+        }
+    }
+    const double hw = grp.sum(h), cpm = grp.sum(c);
+    const double dTdt = -hw * Tab<double>::inv(cpm);
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        if (lane + G * r == nS) out[r] = dTdt;
 }
 
 }  // namespace kin
