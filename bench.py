@@ -562,11 +562,12 @@ def run_kin(args):
     roof = roofline(m, method, prec, sigma, stats, energy, kavg, pk, world)
     shape_key = tuple(int(shape[k]) for k in ("block_threads", "blocks_per_sm", "staging", "occupancy",
                                                  "layout"))
-    fname = feval_name(km, prec, shape, cells, layout_name(km, method, shape, cells), energy)
+    lname = layout_name(km, method, shape, cells, prec, energy)
+    fname = feval_name(km, prec, shape, cells, lname, energy)
     tr, tr_shape = traffic_for(name, shape_key, fname, cells)
     roof.update(traffic=tr, traffic_capture_shape=tr_shape,
                 kernel="kin_integrate launch (init + sort + integrate kernels, %s layout, %s f)"
-                       % (layout_name(km, method, shape, cells), fname))
+                       % (lname, fname))
     Yg = Yd.cpu().numpy()
     Tg = Td.cpu().numpy() if energy else None
 
@@ -638,7 +639,7 @@ def run_kin(args):
             "accuracy_vs_oracle": acc,
             "e2e": e2e,
             "gpu_launches": args.steps * (5 if method == synth.RKC else
-                                          (1 if layout_name(km, method, shape, cells) == "warp-per-cell"
+                                          (1 if lname == "warp-per-cell"
                                            else 2)),
             "clocks": clk.summary(),
             "peak_probe": pk,
@@ -903,7 +904,7 @@ def run_divergence(args):
                       "D": divergence.summary(d)}
     print(json.dumps({"mode": "divergence", "workload": name, "cells": cells,
                       "global_steps": args.global_steps, "launch_shape": shape,
-                      "layout": layout_name(km, method, shape, cells),
+                      "layout": layout_name(km, method, shape, cells, prec, energy),
                       "similar_over_random_time": out["similar"]["ms_total"] / out["random"]["ms_total"],
                       **out}))
     km.close()
@@ -911,26 +912,42 @@ def run_divergence(args):
 
 
 def feval_name(km, prec, shape, cells, layout, energy=0):
-    """'generated' where the call runs the generated f (asked for, or the
-    library's automatic choice: lane layout, FP64, isothermal, staging 0, a
-    small mechanism, a large call), else 'tables'."""
+    """'generated' or 'integer' where the call runs the generated f (asked for,
+    or the library's automatic choice: lane layout, FP64, isothermal, staging 0,
+    a small mechanism, a large call) or the f on the integer pipes (a layout left
+    to the library: FP64 in the warp layout, else a small mechanism), else
+    'tables'."""
     from paper_1309_2710_gb300 import kin
     if shape.get("feval", kin.FEVAL_AUTO) != kin.FEVAL_AUTO:
         return "generated" if shape["feval"] == kin.FEVAL_GENERATED else "tables"
+    if shape.get("layout") == kin.LAYOUT_AUTO and prec == synth.FP64:
+        if layout == "warp-per-cell":
+            return "integer"
+        rows = int((km._arrays["type"] != 0).sum())
+        if (not energy and shape.get("staging", 0) == kin.STAGE_GLOBAL and shape.get("block_threads", 0) == 0
+                and shape.get("blocks_per_sm", 0) == 0 and 26 * (km.n_species + 1) + 10 * rows <= 448):
+            return "integer"
     gen = (layout == "lane-per-cell" and prec == synth.FP64 and not energy
            and shape.get("staging", 0) == kin.STAGE_GLOBAL and km.n_species <= kin.GEN_MAX_SPECIES
            and km.n_reactions <= kin.GEN_MAX_REACTIONS and cells >= kin.GEN_MIN_CELLS)
     return "generated" if gen else "tables"
 
 
-def layout_name(km, method, shape, cells):
+def layout_name(km, method, shape, cells, prec=None, energy=0):
+    """The layout of a call: the one asked for, or the library's rule for
+    KIN_LAYOUT_AUTO (include/kin.h)."""
     from paper_1309_2710_gb300 import kin
     import torch
     lay = shape.get("layout", kin.LAYOUT_AUTO)
     if lay == kin.LAYOUT_AUTO:
         nsm = torch.cuda.get_device_properties(0).multi_processor_count
-        small = cells < kin.WARP_MAX_CELLS_PER_SM * nsm
-        lay = kin.LAYOUT_WARP if km.n_reactions > kin.WARP_MIN_REACTIONS or small else kin.LAYOUT_LANE
+        per_sm, n = cells / nsm, km.n_species + energy
+        warp = km.n_reactions > kin.WARP_MIN_REACTIONS or per_sm < kin.WARP_MAX_CELLS_PER_SM
+        free = not any(shape.get(k, 0) for k in ("block_threads", "blocks_per_sm", "staging", "occupancy", "feval"))
+        if free and prec == synth.FP64 and n <= 32:
+            most = kin.WARP_RKC_MAX_CELLS_PER_SM if method == synth.RKC else kin.WARP_RKCK_MAX_CELLS_PER_SM
+            warp = warp or (method == synth.RKC if n > 16 else energy or per_sm < most)
+        lay = kin.LAYOUT_WARP if warp else kin.LAYOUT_LANE
     return "warp-per-cell" if lay == kin.LAYOUT_WARP else "lane-per-cell"
 
 

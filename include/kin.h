@@ -97,11 +97,16 @@ extern "C" {
                              to 256 */
 #define KIN_WARP_MIN_REACTIONS 256
 #define KIN_WARP_MAX_CELLS_PER_SM 64
-#define KIN_WARP_RKC_MAX_CELLS_PER_SM 704
-#define KIN_WARP_RKCK_MAX_CELLS_PER_SM 320
+#define KIN_WARP_RKC_MAX_CELLS_PER_SM 470
+#define KIN_WARP_RKCK_MAX_CELLS_PER_SM 200
 
 /* how the lane-per-cell layout evaluates f (kin_opts.feval) */
-#define KIN_FEVAL_AUTO 0      /* the generated f for an isothermal call of at least
+#define KIN_FEVAL_AUTO 0      /* with KIN_LAYOUT_AUTO, in isothermal KIN_FP64 with
+                                 KIN_STAGE_GLOBAL and at least 480 lanes per SM, f on the
+                                 integer pipes with its sums in shared memory, for small
+                                 mechanisms (26 (n_species + 1) + 10 n_rows <= 448, n_rows
+                                 the third-body and falloff reactions); else
+                                 the generated f for an isothermal call of at least
                                  KIN_GEN_MIN_CELLS cells that it serves (below), else the
                                  tables: the one-time compilation pays for itself on large
                                  calls (with the energy equation the generated form, one

@@ -1,7 +1,8 @@
 """Autotuner for the launch shape of the integrator.
 
 For one mechanism, method and precision it times kin_integrate on a sample
-of the caller's cells over the candidate shapes:
+of the caller's cells with the library's own choice of layout, shape and f,
+and over the candidate shapes:
   block_threads  32 .. 128 lanes per block (one cell per lane),
   blocks_per_sm  persistent blocks per SM (only shapes that fit),
   staging        per-lane rate scratch in the workspace or in shared memory,
@@ -59,6 +60,9 @@ def candidates(full: bool = False, method: int = kin.RKC, n_reactions: int = 0):
     if n_reactions > kin.WARP_MIN_REACTIONS:
         yield from warp_candidates(full, method)
         return
+    # the library's choice: its f on the integer pipes has no shape of its own
+    yield dict(block_threads=0, blocks_per_sm=0, staging=kin.STAGE_GLOBAL, occupancy=kin.OCC_DEFAULT,
+               layout=kin.LAYOUT_AUTO)
     yield from lane_candidates(full)
     yield from warp_candidates(False, method)
 
@@ -100,7 +104,7 @@ def tune(mech: kin.Mechanism, desc, T, p, Y, dt, rtol, atol, method, precision,
     """Best launch shape for this mechanism on the current GPU, timed on the
     given (device) cells: pass the cells of a representative call, since the
     persistent grid's tail depends on the cell count."""
-    key = _key(mech, method, precision, desc) + "|%d|%d|%d|v5" % (int(T.numel()), sigma, energy)
+    key = _key(mech, method, precision, desc) + "|%d|%d|%d|v6" % (int(T.numel()), sigma, energy)
     cache = {}
     if use_cache and os.path.exists(CACHE):
         with open(CACHE) as f:

@@ -72,11 +72,13 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
     if (m->nR > KIN_WARP_MIN_REACTIONS) return KIN_LAYOUT_WARP;
     if (cells < (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return KIN_LAYOUT_WARP;
     // FP64 on small mechanisms: the warp layout's integer f beats a lane per cell
-    // until every lane of the GPU has more than one. GB300, warp against lane:
-    //   13 species RKC: 30,000 cells 14.6 against 39.0 ms, 100,000 51.3 against
-    //     55.3, 131,072 67.4 against 64.3 (generated f from 65,536 cells on);
-    //   9 species RKCK: 20,000 cells 1.85 against 3.24, 40,000 3.51 against 4.20,
-    //     80,000 6.83 against 5.69;
+    // until the cells fill the GPU's lanes (RKC, about 78,000 lanes; half of
+    // them for RKCK, whose cells take equal times). GB300, warp against lane:
+    //   13 species RKC: 30,000 cells 14.6 against 31.4 ms, 70,000 36.0 against
+    //     36.8, 76,000 39.0 against 38.2, 262,144 135 against 97;
+    //   9 species RKCK: 20,000 cells 1.85 against 2.68, 30,000 2.68 against 2.75,
+    //     40,000 3.52 against 2.95, 100,000 8.51 against 5.50;
+    // (plain FP64 lanes, 13 species RKC: 30,000 cells 39.0, 131,072 64.3;)
     //   24 species RKC: 12,000 cells 10.8 against 94.9, 150,000 134 against 185;
     //   energy equation, 13 species RKC: 20,000 cells 13.3 against 68.2, 200,000
     //     128 against 269; 9 species RKCK: 80,000 cells 13.6 against 17.4.
@@ -175,6 +177,30 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
     return KIN_OK;
 }
 
+// Blocks of a lane-layout call's persistent grid that run the integer FP64 f,
+// or 0 where it does not serve: a layout or f evaluation asked for, mixed
+// precision, the energy equation, staged arrays, a mechanism beyond its tables,
+// or fewer than LANE_INT_MIN_LANES lanes per SM, asked for or left by its shared
+// words. Its lanes wait on their own
+// chains, so it needs them: GB300, 13 species RKC, 262,144 cells at 512 and
+// 384 lanes per SM 97 and 116 ms, the generated f 122 and 123; 9 species RKCK,
+// 400,000 cells at 512 lanes 21.4 against 24.9; 20 species RKCK, 150,000 cells
+// at 384 lanes 1.53 against 1.34.
+int lane_int_blocks(const kin_mech* m, const kin_opts* o, const Grid& g, int* blocks)
+{
+    *blocks = 0;
+    if (g.layout != KIN_LAYOUT_LANE || o->layout != KIN_LAYOUT_AUTO || o->feval != KIN_FEVAL_AUTO) return KIN_OK;
+    if (!m->dev.li_rx || o->precision != KIN_FP64 || o->energy || o->staging != KIN_STAGE_GLOBAL) return KIN_OK;
+    int nsm = 0, bps = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
+    e = occ_lane_int(m->dev, o->method, o->occupancy, g.threads, &bps);
+    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    bps = std::min(bps, g.blocks / nsm);
+    if (bps * g.threads >= LANE_INT_MIN_LANES) *blocks = bps * nsm;
+    return KIN_OK;
+}
+
 // Workspace bytes; the warp layout keeps no per-lane arrays.
 int64_t ws_bytes(const kin_mech* m, const kin_opts* o, const Grid& g, int64_t cells)
 {
@@ -265,7 +291,16 @@ int kin::noalloc_opts(const kin_mech* m, const kin_opts* in, int64_t cells, int6
         if (rc) return rc;
         need = ws_bytes(m, &o, g, cells);
         if (need <= cap) {
-            *out = o;
+            // kin_integrate's integer f where it serves, which compiles nothing:
+            // a call whose layout is left to the library and that names its
+            // blocks takes the lane layout again
+            kin_opts a = o;
+            a.layout = in->layout;
+            a.feval = in->feval;
+            int li_blocks = 0;
+            rc = lane_int_blocks(m, &a, g, &li_blocks);
+            if (rc) return rc;
+            *out = li_blocks ? a : o;
             return KIN_OK;
         }
     }
@@ -577,6 +612,13 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     const size_t oEx2 = put(ex2, sizeof(ex2)), oLnc = put(lnc, sizeof(lnc));
     const size_t oImW = put(imW.data(), 8 * imW.size()), oImWe = put(imWe.data(), 4 * imWe.size());
     const size_t oEffI = put(effI.data(), 4 * effI.size()), oEffX = put(effX.data(), 4 * effX.size());
+    // the lane layout's integer FP64 f, for mechanisms whose shared words leave
+    // room for enough lanes
+    const bool use_li = lane_int_bytes(nS, nM) <= LANE_INT_MAX_BYTES;
+    LaneInt li;
+    if (use_li) li = build_lane_int(nS, nR, d->reac, d->prod, d->type, d->eff);
+    const size_t oLiRx = put(li.rx.data(), 4 * li.rx.size());
+    const size_t oLiE = put(li.eff.data(), 4 * li.eff.size()), oLiEx = put(li.effx.data(), 4 * li.effx.size());
     // the segmented FP32 gather of the 32-lane isothermal f, where the packed
     // entries apply and its partial sums fit in the FP32 half of the warp's
     // shared words, past C and Omega
@@ -646,6 +688,11 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.imW = (const ulonglong2*)(b + oImW);
     M.imWe = (const int2*)(b + oImWe);
     M.imLow = imLow;
+    M.li_n = li.n;
+    M.li_tb = li.tb;
+    M.li_rx = use_li ? (const uint4*)(b + oLiRx) : nullptr;
+    M.li_eff = (const int2*)(b + oLiE);
+    M.li_effx = (const int32_t*)(b + oLiEx);
     M.effV64 = (const double*)(b + oEffV64);
     M.effV32 = (const float*)(b + oEffV32);
     M.rxw = (const uint32_t*)(b + oRxw);
@@ -789,13 +836,17 @@ int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, 
     P.cell_st = (uint8_t*)(base + w.st);
     P.order = (int32_t*)(base + w.order);
     if (total > INT32_MAX) return fail(KIN_EINVAL, "more than 2^31-1 cells in one call");
-    // f: tables, or the mechanism's generated code (lane layout, FP64, isothermal)
+    // f: integer arithmetic where it serves, tables, or the mechanism's
+    // generated code (lane layout, FP64, isothermal)
+    int li_blocks = 0;
+    rc = lane_int_blocks(m, o, g, &li_blocks);
+    if (rc) return rc;
     bool gen = false;
     GenKernels gk{};
     // (the automatic choice leaves the energy equation on the tables: with a
     // per-reaction exp inlined, the generated form measured slower)
     if (o->feval == KIN_FEVAL_GENERATED ||
-        (o->feval == KIN_FEVAL_AUTO && total >= KIN_GEN_MIN_CELLS && !o->energy)) {
+        (o->feval == KIN_FEVAL_AUTO && total >= KIN_GEN_MIN_CELLS && !o->energy && !li_blocks)) {
         // (the energy equation comes generated too: the mechanism has cp and
         // Hf, checked above, so its source carries that form of f)
         const bool serves = g.layout == KIN_LAYOUT_LANE && o->precision == KIN_FP64 &&
@@ -826,7 +877,11 @@ int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, 
             {{launch_warp_f64_en_o0, launch_warp_f64_en_o1}, {launch_warp_f32_en_o0, launch_warp_f32_en_o1}}};
         e = fns[o->energy][o->precision == KIN_MIXED][o->occupancy ? 1 : 0](P, blocks, g.threads, st);
     }
-    else if (gen)
+    else if (li_blocks) {
+        blocks = std::min(blocks, li_blocks);
+        P.nslots = (int64_t)blocks * g.threads;
+        e = launch_lane_int(P, o->occupancy, blocks, g.threads, st);
+    } else if (gen)
         e = gen_launch(gk, P, o->occupancy, blocks, g.threads, st);
     else
         e = launch_integrate(P, o->energy ? KIN_STAGE_GLOBAL : o->staging, o->occupancy, blocks,

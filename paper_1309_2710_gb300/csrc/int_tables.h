@@ -151,4 +151,69 @@ inline int int_efficiencies(int nS, const double* eff, int32_t* hi, int32_t* lo)
     return x;
 }
 
+// Tables of the lane layout's f (lane_int.cuh): its reactions in the order
+// third bodies first, without those that change nothing.
+struct LaneInt {
+    int n = 0, tb = 0;
+    std::vector<uint32_t> rx;               // [n + 1][4] records
+    std::vector<int32_t> eff;               // [tb][nS][2] integer efficiencies
+    std::vector<int32_t> effx;              // [tb]
+};
+
+// type: 0 plain, 1 third body, 2 falloff; eff: one row per non-plain reaction,
+// in reaction order.
+inline LaneInt build_lane_int(int nS, int nR, const int32_t* reac, const int32_t* prod,
+                              const int8_t* type, const double* eff)
+{
+    LaneInt t;
+    for (int pass = 0; pass < 2; ++pass) {
+        int row = 0, fo = 0;
+        for (int j = 0; j < nR; ++j) {
+            const int ty = type[j], r = ty ? row++ : -1, f = ty == 2 ? fo++ : 0;
+            if ((ty == 0) != (pass == 1)) continue;
+            // net coefficients by species
+            int sp[4], c[4], m = 0, order = 0;
+            for (int k = 0; k < 4; ++k) {
+                const int s = k < 2 ? prod[2 * j + k] : reac[2 * j + k - 2];
+                if (s < 0) continue;
+                order += k >= 2;
+                int a = 0;
+                while (a < m && sp[a] != s) ++a;
+                if (a == m) {
+                    sp[m] = s;
+                    c[m++] = 0;
+                }
+                c[a] += k < 2 ? 1 : -1;
+            }
+            uint32_t slot[4] = {(uint32_t)nS, (uint32_t)nS, (uint32_t)nS, (uint32_t)nS}, flags = 0;  // p0 p1 n0 n1
+            int np = 0, nn = 0;
+            for (int a = 0; a < m; ++a) {
+                if (c[a] == 0) continue;
+                const int at = c[a] > 0 ? np++ : 2 + nn++;
+                slot[at] = (uint32_t)sp[a];
+                if (c[a] == 2 || c[a] == -2) flags |= 1u << (16 + at);
+            }
+            if (np + nn == 0) continue;
+            const uint32_t ra = reac[2 * j] < 0 ? nS : reac[2 * j], rb = reac[2 * j + 1] < 0 ? nS : reac[2 * j + 1];
+            const int power = order + (ty == 1) - 2;  // of rho, beyond a plain reaction of two
+            t.rx.push_back(ra | rb << 8 | slot[0] << 16 | slot[1] << 24);
+            t.rx.push_back(slot[2] | slot[3] << 8 | flags | (uint32_t)(power + 2) << 20 | (ty == 2 ? 1u << 23 : 0u));
+            t.rx.push_back((uint32_t)j);
+            t.rx.push_back((uint32_t)f);
+            ++t.n;
+            if (ty) {
+                ++t.tb;
+                std::vector<int32_t> hi(nS), lo(nS);
+                t.effx.push_back(int_efficiencies(nS, eff + (size_t)r * nS, hi.data(), lo.data()));
+                for (int k = 0; k < nS; ++k) {
+                    t.eff.push_back(hi[k]);
+                    t.eff.push_back(lo[k]);
+                }
+            }
+        }
+    }
+    for (int k = 0; k < 4; ++k) t.rx.push_back(t.n ? t.rx[4 * (t.n - 1) + k] : 0u);
+    return t;
+}
+
 }  // namespace kin

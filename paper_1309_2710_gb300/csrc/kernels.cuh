@@ -462,6 +462,15 @@ __device__ __forceinline__ double Tab<double>::inv(double a)
     return fma(r, fma(-a, r, 1.0), r);
 }
 
+// Pr / (1 + Pr): the reciprocal by two Newton steps and one correction of the
+// quotient (within an ulp; an IEEE division is a third longer).
+__device__ __forceinline__ double falloff_factor(double Pr)
+{
+    const double d = 1.0 + Pr, r = Tab<double>::inv(d), q = Pr * r;
+    const double z = fma(r, fma(-q, d, Pr), q);
+    return isfinite(z) ? z : ddiv(Pr, d);
+}
+
 struct PowerState {
     int k;
     double prev, dyn, sig;
@@ -526,7 +535,14 @@ __device__ __forceinline__ bool power_post(int nS, Lane<double> Y, Lane<double> 
 // F::eval<R, KT>(M, Ctot, invCtot, K, KR, C, OM, x, out). TableF is feval
 // over the mechanism's device tables (any mechanism, either precision); a
 // generated policy (FP64 only) is f for one mechanism as straight-line code,
-// compiled at run time, with the same arguments.
+// compiled at run time, with the same arguments. A policy in integer arithmetic
+// (IntegerF) also takes the cell's scale, which starts as F::scale0(M, K, KR)
+// and follows from one evaluation to the next.
+template <typename F>
+struct IntegerF {
+    static constexpr bool value = false;
+};
+
 struct TableF {
     template <typename R, typename KT>
     __device__ __forceinline__ static void eval(const MechDev& M, double Ctot, double invCtot, Lane<KT> K,
@@ -544,17 +560,26 @@ struct TableF {
     }
 };
 
+template <typename F, typename R, typename KT>
+__device__ __forceinline__ void eval_f(const MechDev& M, double Ctot, double invCtot, Lane<KT> K, Lane<KT> KR,
+                                       Lane<R> C, Lane<R> OM, Lane<double> x, Lane<double> out, int& scale)
+{
+    if constexpr (IntegerF<F>::value) F::template eval<R, KT>(M, Ctot, invCtot, K, KR, C, OM, x, out, scale);
+    else F::template eval<R, KT>(M, Ctot, invCtot, K, KR, C, OM, x, out);
+}
+
 // f in FP64 for a spectral-radius estimate: the lane's rate scratch in the
 // FP64 path, the separate FP64 scratch in the mixed-precision path (whose
 // rate constants are the same FP32 values, promoted).
 template <typename R, int STG, typename F>
 __device__ __forceinline__ void feval_sig(const Views<R, STG>& W, double Ctot, double invCtot,
-                                          Lane<R> K, Lane<R> KR, Lane<double> x, Lane<double> out)
+                                          Lane<R> K, Lane<R> KR, Lane<double> x, Lane<double> out,
+                                          int& scale)
 {
     if constexpr (sizeof(R) == 4)
-        F::template eval<double, R>(W.M, Ctot, invCtot, K, KR, W.C64, W.OM64, x, out);
+        eval_f<F, double, R>(W.M, Ctot, invCtot, K, KR, W.C64, W.OM64, x, out, scale);
     else
-        F::template eval<double, R>(W.M, Ctot, invCtot, K, KR, W.C, W.OM, x, out);
+        eval_f<F, double, R>(W.M, Ctot, invCtot, K, KR, W.C, W.OM, x, out, scale);
 }
 
 // ------------------------------------------------------------- pre-pass --
@@ -577,17 +602,19 @@ __global__ void __launch_bounds__(128) init_kernel(const __grid_constant__ Launc
         const double Ctot = ddiv(p * 1e-6, R_GAS * T), invCtot = ddiv(1.0, Ctot);
         Lane<R> K = W.K(g), KR = W.KR(g);
         if constexpr (!EN) rate_constants<R>(M, T, K, KR);
+        int scale = 0;
+        if constexpr (IntegerF<F>::value && !EN) scale = F::scale0(M, K, KR);
         // f in the rate type, and f in FP64 for the spectral radius
         auto frate = [&](Lane<double> x, Lane<double> o) {
             if constexpr (EN) F::template eval_energy<R>(M, p, W.C, W.OM, x, o);
-            else F::template eval<R, R>(M, Ctot, invCtot, K, KR, W.C, W.OM, x, o);
+            else eval_f<F, R, R>(M, Ctot, invCtot, K, KR, W.C, W.OM, x, o, scale);
         };
         auto fsig = [&](Lane<double> x, Lane<double> o) {
             if constexpr (EN) {
                 if constexpr (sizeof(R) == 4) F::template eval_energy<double>(M, p, W.C64, W.OM64, x, o);
                 else F::template eval_energy<double>(M, p, W.C, W.OM, x, o);
             } else {
-                feval_sig<R, STG, F>(W, Ctot, invCtot, K, KR, x, o);
+                feval_sig<R, STG, F>(W, Ctot, invCtot, K, KR, x, o, scale);
             }
         };
         Lane<double> Y = W.V(V_Y), F0 = W.F0cell(g), X = W.V(V_X), FX = W.V(V_FX), RS = W.V(V_RS);
@@ -723,6 +750,7 @@ struct LaneState {
     bool last, last_rejected, have_prev, sigma_here;
     int iw1, iw2;  // RKC: slots of w_{j-1}, w_{j-2}
     double t, dt, h, hh, hprev, cprev, sigma, eps, rtol, atol, Ctot, invCtot, invN, p;
+    int scale;        // of the cell's f (integer policies)
     int in_v, out_v;  // vectors read and written by the next f evaluation
     PowerState P;     // RKC power-method sigma in progress
 };
@@ -771,6 +799,7 @@ struct Integrator {
                 const Lane<R> Kc = W.K(g), KRc = W.KR(g);
                 for (int j = 0; j < M.nR; ++j) K[j] = Kc[j];
                 for (int j = 0; j < M.nFO; ++j) KR[j] = KRc[j];
+                if constexpr (IntegerF<F>::value) S.scale = F::scale0(M, K, KR);
             }
             const int n = L.nV;
             Lane<double> Y = V(V_Y), F0 = V(V_F0), F0c = W.F0cell(g);
@@ -1220,10 +1249,10 @@ struct Integrator {
                 else
                     F::template eval_energy<double>(M, S.p, W.C, W.OM, V(S.in_v), V(S.out_v));
             } else if (sizeof(R) == 4 && sig) {
-                F::template eval<double, R>(M, S.Ctot, S.invCtot, K, KR, W.C64, W.OM64, V(S.in_v),
-                                            V(S.out_v));
+                eval_f<F, double, R>(M, S.Ctot, S.invCtot, K, KR, W.C64, W.OM64, V(S.in_v),
+                                     V(S.out_v), S.scale);
             } else {
-                F::template eval<R, R>(M, S.Ctot, S.invCtot, K, KR, W.C, W.OM, V(S.in_v), V(S.out_v));
+                eval_f<F, R, R>(M, S.Ctot, S.invCtot, K, KR, W.C, W.OM, V(S.in_v), V(S.out_v), S.scale);
             }
             S.nfe++;
             S.nfs += sig;
@@ -1251,24 +1280,24 @@ __global__ void __launch_bounds__(128, OCC ? 6 : 4) integrate_kernel(const __gri
 #ifndef __CUDACC_RTC__
 
 // ------------------------------------------------------- launch templates --
-template <int METHOD, typename R, int STG, int OCC, bool EN>
-inline cudaError_t launch_all(Launch& L, int blocks, int threads, cudaStream_t st)
+template <int METHOD, typename R, int STG, int OCC, bool EN, typename F = TableF>
+inline cudaError_t launch_all(Launch& L, int blocks, int threads, cudaStream_t st, size_t f_smem = 0)
 {
-    const size_t sm = smem_bytes(L.M, L.precision, threads, STG);
-    if (STG > 0) {
-        cudaError_t e = cudaFuncSetAttribute(init_kernel<METHOD, R, STG, EN>,
+    const size_t sm = smem_bytes(L.M, L.precision, threads, STG) + f_smem;
+    if (sm > 0) {
+        cudaError_t e = cudaFuncSetAttribute(init_kernel<METHOD, R, STG, EN, F>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(integrate_kernel<METHOD, R, STG, OCC, EN>,
+            e = cudaFuncSetAttribute(integrate_kernel<METHOD, R, STG, OCC, EN, F>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
     }
-    init_kernel<METHOD, R, STG, EN><<<blocks, threads, sm, st>>>(L);
+    init_kernel<METHOD, R, STG, EN, F><<<blocks, threads, sm, st>>>(L);
     if (METHOD == KIN_RKC) {
         const cudaError_t e = launch_sort(L, st);
         if (e != cudaSuccess) return e;
     }
-    integrate_kernel<METHOD, R, STG, OCC, EN><<<blocks, threads, sm, st>>>(L);
+    integrate_kernel<METHOD, R, STG, OCC, EN, F><<<blocks, threads, sm, st>>>(L);
     return cudaGetLastError();
 }
 
@@ -1287,15 +1316,15 @@ inline cudaError_t launch_occ(Launch& L, int stg, int occ, int blocks, int threa
                : launch_staged<METHOD, R, 0>(L, stg, blocks, threads, st);
 }
 
-template <int METHOD, typename R, int STG, int OCC, bool EN = false>
+template <int METHOD, typename R, int STG, int OCC, bool EN = false, typename F = TableF>
 inline cudaError_t occ_one(int threads, size_t sm, int* bps)
 {
-    if (STG > 0) {
-        cudaError_t e = cudaFuncSetAttribute(integrate_kernel<METHOD, R, STG, OCC, EN>,
+    if (sm > 0) {
+        cudaError_t e = cudaFuncSetAttribute(integrate_kernel<METHOD, R, STG, OCC, EN, F>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
     }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, integrate_kernel<METHOD, R, STG, OCC, EN>,
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, integrate_kernel<METHOD, R, STG, OCC, EN, F>,
                                                          threads, sm);
 }
 

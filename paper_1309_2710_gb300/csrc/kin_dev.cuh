@@ -96,6 +96,12 @@ struct MechDev {
     const ulonglong2* imW; // [nS] 63-bit mantissas of 1 / W and W
     const int2* imWe;      // [nS] their exponents
     int imLow;             // 1: a reaction of fewer than two factors of concentration
+    // the lane layout's integer FP64 f (lane_int.cuh): reactions with a net
+    // effect, third bodies first; null where it does not apply
+    int li_n, li_tb;
+    const uint4* li_rx;    // [li_n + 1]
+    const int2* li_eff;    // [li_tb][nS] integer efficiencies {hi, lo}
+    const int32_t* li_effx;  // [li_tb]
     // efficiencies by non-plain reaction in permutation order (row), species
     // in 16-byte groups: [k / V][row][k % V], V = 2 (FP64) or 4 (FP32), the
     // last group zero-padded
@@ -118,6 +124,13 @@ struct MechDev {
     const double* Hf;      // [nS] J/mol at T_REF
     const double* HfW;     // [nS] Hf_i / W_i, J/g
 };
+
+// The lane layout's integer f: shared bytes of a lane (sums, mantissas and
+// exponents of the species and of the empty slot, mantissas and exponents of the
+// third-body factors), the fewest lanes per SM that it runs with (abi.cu has the
+// figures), and the bytes that leave an SM so many.
+constexpr int LANE_INT_MIN_LANES = 480, LANE_INT_MAX_BYTES = 448;
+constexpr int lane_int_bytes(int nS, int rows) { return 26 * (nS + 1) + 10 * rows; }
 
 // One instance of a batched launch (device pointers).
 struct InstDev {
@@ -200,6 +213,9 @@ cudaError_t occ_rkc_f64_en(int occ, int threads, size_t sm, int* bps);
 cudaError_t occ_rkc_f32_en(int occ, int threads, size_t sm, int* bps);
 cudaError_t occ_rkck_f64_en(int occ, int threads, size_t sm, int* bps);
 cudaError_t occ_rkck_f32_en(int occ, int threads, size_t sm, int* bps);
+// The lane layout's integer FP64 f (inst_lane_int.cu, staging 0).
+cudaError_t launch_lane_int(Launch& L, int occ, int blocks, int threads, cudaStream_t st);
+cudaError_t occ_lane_int(const MechDev& M, int method, int occ, int threads, int* bps);
 // Warp-per-cell RKC (inst_warp_*.cu): one warp integrates one cell; one
 // translation unit per rate precision and register budget (occupancy).
 cudaError_t launch_warp_f64_o0(Launch& L, int blocks, int threads, cudaStream_t st);

@@ -281,15 +281,6 @@ static __device__ __noinline__ double int_general_sum(const MechDev& M, const Ra
     return w;
 }
 
-// Pr / (1 + Pr): the reciprocal by two Newton steps and one correction of the
-// quotient (within an ulp; an IEEE division is a third longer).
-__device__ __forceinline__ double falloff_factor(double Pr)
-{
-    const double d = 1.0 + Pr, r = Tab<double>::inv(d), q = Pr * r;
-    const double z = fma(r, fma(-q, d, Pr), q);
-    return isfinite(z) ? z : ddiv(Pr, d);
-}
-
 // f of such a state, from its c_k / rho (the group's lanes together).
 template <int NR, int G>
 __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, const RateSource& k, const double (&c)[NR],

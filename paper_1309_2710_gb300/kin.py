@@ -26,7 +26,7 @@ SIGMA_GERSHGORIN, SIGMA_POWER = 0, 1
 LAYOUT_AUTO, LAYOUT_LANE, LAYOUT_WARP = 0, 1, 2
 WARP_MIN_REACTIONS = 256
 WARP_MAX_CELLS_PER_SM = 64
-WARP_RKC_MAX_CELLS_PER_SM, WARP_RKCK_MAX_CELLS_PER_SM = 704, 320
+WARP_RKC_MAX_CELLS_PER_SM, WARP_RKCK_MAX_CELLS_PER_SM = 470, 200
 FEVAL_AUTO, FEVAL_TABLE, FEVAL_GENERATED = 0, 1, 2
 GEN_MAX_SPECIES, GEN_MAX_REACTIONS, GEN_MIN_CELLS = 32, 256, 65536
 MAX_INSTANCES = 128
