@@ -626,7 +626,11 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     const int group_floats = 2 * ((nS + nR + 3) & ~3);
     const bool use_seg = build_seg_tables(nS, nR, ptr.data(), crxp.data(), cnu.data(), seg) &&
                          nS + nR + seg.nslots <= group_floats;
-    const size_t oSegE = use_seg ? put(seg.ent.data(), 4 * seg.ent.size()) : 0;
+    // four steps of a lane side by side; steps past the last have no flush
+    const int segK4 = (seg.K + 3) / 4;
+    std::vector<uint32_t> segE((size_t)segK4 * 128, 0u);
+    for (size_t k = 0; k < seg.ent.size(); ++k) segE[(k / 128 * 32 + k % 32) * 4 + k / 32 % 4] = seg.ent[k];
+    const size_t oSegE = use_seg ? put(segE.data(), 4 * segE.size()) : 0;
     const size_t oSegF = use_seg ? put(seg.slot0.data(), 4 * seg.slot0.size()) : 0;
     const size_t oSegP = use_seg ? put(seg.part.data(), 4 * seg.part.size()) : 0;
     const size_t oEff = put(d->eff, 8 * (size_t)nM * nS), oEff32 = put(eff32.data(), 4 * (size_t)nM * nS);
@@ -668,10 +672,10 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.ell32 = (const CsrW32*)(b + oEll32);
     M.ell64 = (const CsrW64*)(b + oEll64);
     for (int r = 0; r < ELL_SLOTS; ++r) M.ell_base[r] = ell_base[r];
-    M.seg_ent = use_seg ? (const uint32_t*)(b + oSegE) : nullptr;
+    M.seg_ent = use_seg ? (const uint4*)(b + oSegE) : nullptr;
     M.seg_slot0 = use_seg ? (const int32_t*)(b + oSegF) : nullptr;
     M.seg_part = use_seg ? (const int32_t*)(b + oSegP) : nullptr;
-    M.seg_K = use_seg ? seg.K : 0;
+    M.seg_K4 = use_seg ? segK4 : 0;
     for (int v = 0; v < INT_NTAB; ++v) {
         M.ig[v] = IntDev{};
         if (!ig_use[v]) continue;

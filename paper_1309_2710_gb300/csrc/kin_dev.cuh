@@ -82,10 +82,10 @@ struct MechDev {
     // The segmented FP32 gather of the 32-lane isothermal f (seg_tables.h):
     // the nonzeros cut into 32 equal chunks of seg_K packed entries, one per
     // lane. Null where the packed form does not apply (the ELL gather runs).
-    const uint32_t* seg_ent;   // [seg_K][32] nu's FP32 bits | flush flag | position
+    const uint4* seg_ent;      // [seg_K4][32] four steps: nu's FP32 bits | flush flag | position
     const int32_t* seg_slot0;  // [32] first partial slot of each lane
     const int32_t* seg_part;   // [nS] first slot << 8 | slot count; -1: empty row
-    int seg_K;
+    int seg_K4;
     IntDev ig[INT_NTAB];
     const int4* effI;      // [(nS + 1) / 2][nM] integer efficiencies {hi, lo} of two species
     const int32_t* effX;   // [nM] their exponents

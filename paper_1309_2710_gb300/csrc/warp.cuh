@@ -60,6 +60,7 @@ __device__ __forceinline__ float eff_dot<float>(const MechDev& M, int row, const
     const float4* __restrict__ a = reinterpret_cast<const float4*>(M.effV32) + row;
     const float4* c = reinterpret_cast<const float4*>(C);
     float m0 = 0.0f, m1 = 0.0f;
+#pragma unroll 4
     for (int k = 0; k < n4; ++k) {
         const float4 e = a[(int64_t)k * nM], x = c[k];
         m0 += e.x * x.x;
@@ -84,6 +85,7 @@ __device__ __forceinline__ double eff_dot<double>(const MechDev& M, int row, con
     const double2* __restrict__ a = reinterpret_cast<const double2*>(M.effV64) + row;
     const double2* c = reinterpret_cast<const double2*>(C);
     double m0 = 0.0, m1 = 0.0;
+#pragma unroll 4
     for (int k = 0; k < n2; ++k) {
         const double2 e = a[(int64_t)k * nM], x = c[k];
         m0 += e.x * x.x;
@@ -181,8 +183,33 @@ __device__ __forceinline__ void warp_feval(const MechDev& M, const KT* Kc, R* C,
     // q - nP), then falloff (ordinal q - nF)
     const int nP = nR - nM, nF = nR - M.nFO;
     const uint32_t* __restrict__ rxw = M.rxw;
+    // The evaluation waits on L1, L2 and shared-memory round trips (53 species
+    // / 634 reactions, FP32: FP64 pipe 68 %, load/store 67 %, issue 57 %), so the
+    // loads of four rounds of plain reactions are in flight together, and so
+    // are four steps of the gathers below. GB300, 1,024 cells 10.7 -> 8.5 ms, 65,536
+    // 235 -> 199 ms, the same bits.
+    int q = lane;
 #pragma unroll 1
-    for (int q = lane; q < nR; q += G) {
+    for (; q - lane + 4 * G <= nP; q += 4 * G) {
+        uint32_t w[4];
+        R v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            w[u] = rxw[q + u * G];
+            v[u] = (R)Kc[q + u * G];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r0 = (int)(w[u] & 0xffffu) - 1, r1 = (int)(w[u] >> 16) - 1;
+            const R a = C[max(r0, 0)], b = C[max(r1, 0)];
+            v[u] *= r0 >= 0 ? a : R(1);
+            v[u] *= r1 >= 0 ? b : R(1);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) OM[q + u * G] = v[u];
+    }
+#pragma unroll 1
+    for (; q < nR; q += G) {
         const uint32_t w = rxw[q];
         R v = (R)Kc[q];
         const int r0 = (int)(w & 0xffffu) - 1, r1 = (int)(w >> 16) - 1;
@@ -205,18 +232,28 @@ __device__ __forceinline__ void warp_feval(const MechDev& M, const KT* Kc, R* C,
         if (M.seg_ent) {
             // omega over equal chunks of the nonzeros (seg_tables.h); the
             // partial sums land past Omega, in the FP32 half of the warp's
-            // words that only the FP64 evaluations use
+            // words that only the FP64 evaluations use. Four entries per load, the
+            // next four on their way
             float* P = reinterpret_cast<float*>(OM) + nR;
-            const uint32_t* __restrict__ ent = M.seg_ent + lane;
+            const uint4* __restrict__ ent = M.seg_ent + lane;
             int slot = M.seg_slot0[lane];
             float w = 0.0f;
-            const int K = M.seg_K;
-            for (int k = 0; k < K; ++k) {
-                const uint32_t e = ent[32 * k];
-                w = fmaf(__uint_as_float(e & SEG_NU_MASK), OM[e & SEG_POS_MASK], w);
-                if (e & SEG_FLUSH) {
-                    P[slot++] = w;
-                    w = 0.0f;
+            const int K4 = M.seg_K4;
+            uint4 e4 = ent[0];
+#pragma unroll 2
+            for (int k = 0; k < K4; ++k) {
+                const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+                e4 = ent[32 * min(k + 1, K4 - 1)];
+                float o[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) o[u] = OM[e[u] & SEG_POS_MASK];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    w = fmaf(__uint_as_float(e[u] & SEG_NU_MASK), o[u], w);
+                    if (e[u] & SEG_FLUSH) {
+                        P[slot++] = w;
+                        w = 0.0f;
+                    }
                 }
             }
             __syncwarp(mask);
@@ -255,6 +292,14 @@ __device__ __forceinline__ void warp_feval(const MechDev& M, const KT* Kc, R* C,
                 const int len = M.csr_ptr[i + 1] - M.csr_ptr[i];
                 const auto* __restrict__ p = EllT<R>::tab(M) + M.ell_base[r] + lane;
                 int k = 0;
+                for (; k + 3 < len; k += 4) {
+                    const auto a = p[32 * k], b = p[32 * (k + 1)], c = p[32 * (k + 2)], e = p[32 * (k + 3)];
+                    const R oa = OM[a.pos], ob = OM[b.pos], oc = OM[c.pos], oe = OM[e.pos];
+                    w0 += a.nuW * oa;
+                    w1 += b.nuW * ob;
+                    w0 += c.nuW * oc;
+                    w1 += e.nuW * oe;
+                }
                 for (; k + 1 < len; k += 2) {
                     const auto a = p[32 * k], b = p[32 * (k + 1)];
                     w0 += a.nuW * OM[a.pos];
@@ -933,7 +978,9 @@ struct WarpRKC {
 // these mechanisms waits on L1 and shared-memory round trips, and more
 // resident warps hide more of that latency: on 53 species / 634 reactions,
 // mixed precision, 198 K cells/s at 32 warps per SM (64 registers), 217 K at
-// 36 (56) and 237 K at 40 (48), against 178 K at 24 (80). With the energy
+// 36 (56) and 237 K at 40 (48), against 178 K at 24 (80), before four rounds'
+// loads were in flight together; with them 65,536 cells take 199 ms at 40
+// warps and 202 ms at 16 (128), 1,024 cells 18.9 and 8.5. With the energy
 // equation 74.1 K at 80 registers against 72.1 K at 64.
 template <int NR, int OCC, bool EN>
 struct WarpBounds {
