@@ -920,9 +920,9 @@ def feval_name(km, prec, shape, cells, layout, energy=0):
     from paper_1309_2710_gb300 import kin
     if shape.get("feval", kin.FEVAL_AUTO) != kin.FEVAL_AUTO:
         return "generated" if shape["feval"] == kin.FEVAL_GENERATED else "tables"
-    if shape.get("layout") == kin.LAYOUT_AUTO and prec == synth.FP64:
-        if layout == "warp-per-cell":
-            return "integer"
+    if prec == synth.FP64 and "layout" in shape and layout == "warp-per-cell":
+        return "integer"
+    if prec == synth.FP64 and shape.get("layout") == kin.LAYOUT_AUTO:
         rows = int((km._arrays["type"] != 0).sum())
         if (not energy and shape.get("staging", 0) == kin.STAGE_GLOBAL and shape.get("block_threads", 0) == 0
                 and shape.get("blocks_per_sm", 0) == 0 and 26 * (km.n_species + 1) + 10 * rows <= 448):

@@ -86,8 +86,9 @@ extern "C" {
 #define KIN_LAYOUT_LANE 1 /* one lane integrates one cell (the paper's thread-per-ODE
                              design, Section 3): per-cell arrays in the workspace or in
                              shared memory (kin_opts.staging) */
-#define KIN_LAYOUT_WARP 2 /* one warp (or half of one, or up to four: the library's
-                             choice by the state's size) integrates one cell: its
+#define KIN_LAYOUT_WARP 2 /* one warp (or a quarter or half of one, or up to four: the
+                             library's choice by the state's size, the precision and
+                             the call's cells) integrates one cell: its
                              lanes share the reactions and species of f; the cell's
                              concentrations and rates of progress live in shared
                              memory. staging is ignored; for RKC, occupancy selects the register budget

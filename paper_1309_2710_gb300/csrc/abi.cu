@@ -94,11 +94,12 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
 }
 
 // Lanes that integrate one cell in the warp layout: half a warp for states of
-// at most 16 components (RKCK; RKC in isothermal FP64, there a quarter above
-// 64 cells per SM: 13 species, 4,000 cells 4.0 ms with 16 lanes and 5.6 with
-// 8, 16,000 cells 9.8 and 8.6, 30,000 cells 17.9 and 14.6), a warp, and in
-// isothermal FP64 RKC two warps above 32 components and four above 64. An
-// evaluation is a chain of short phases, so more lanes shorten it, and the
+// at most 16 components (RKCK; RKC in FP64), of which FP64 calls of up to 8
+// cells per SM take a whole one (9 species RKCK, 64 cells 0.348 -> 0.295 ms; 13
+// species RKC, 1,000 cells 3.57 -> 3.05) and FP64 RKC above 64 cells per SM a
+// quarter (13 species, 4,000 cells 4.0 ms with 16 lanes and 5.6 with 8, 16,000
+// cells 9.8 and 8.6, 30,000 cells 17.9 and 14.6); else a warp, and in FP64 RKC
+// two warps above 32 components and four above 64. An evaluation is a chain of short phases, so more lanes shorten it, and the
 // FP64 pipe's vector work per cell stays the same (fewer slots per lane on more
 // warps). Measured on GB300, 2 or 4 warps against 1: 53 species, 256 / 4,096 /
 // 20,000 cells 10.4 against 18.9, 37.7 against 43.9, 157.9 against 159.4 ms;

@@ -5,12 +5,12 @@
 // progress and rate constants: ~(2 n_R + n_S) words per cell, which for
 // hundreds of reactions spills out of L1/L2 and turns every f evaluation into
 // a stream from HBM. Here a group of G lanes integrates one cell (a warp; in
-// isothermal FP64 half a warp to four warps, cell_lanes in abi.cu):
+// FP64 a quarter of a warp to four warps, cell_lanes in abi.cu):
 //  * the lanes split the reactions (rates of progress, rounds of G) and
 //    the species (state vectors in registers: species l + G r in slot r of
 //    lane l);
-//  * f in FP64 runs on the integer pipes (warp_int.cuh); in mixed precision and
-//    with the energy equation its concentrations and rates of progress live in
+//  * f in FP64 runs on the integer pipes (warp_int.cuh); in mixed precision
+//    its concentrations and rates of progress live in
 //    shared memory (n_S + n_R words per warp). A cell's rate constants, computed
 //    once per call since T is fixed, live in the workspace cell-major and are
 //    read coalesced (the working set of the resident cells stays in L2);

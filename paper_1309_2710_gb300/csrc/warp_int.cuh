@@ -1,4 +1,5 @@
-// warp_int.cuh -- the warp layout's isothermal FP64 f on the integer pipes
+// warp_int.cuh -- the warp layout's FP64 f on the integer pipes, isothermal, with
+// the energy equation and alone
 // (intf.cuh has the arithmetic, int_tables.h the tables).
 //
 // One group of G lanes evaluates f for one cell. Concentrations live in
@@ -14,11 +15,13 @@
 // 1780; the FP64 f it replaced took 43 K with one warp, 354 FP64 instructions
 // of 64 cycles among them). So a lane's next reaction words, the gather's next
 // entries and eight efficiencies of a third-body sum are fetched ahead.
-// Whole calls on GB300, before and after: 53 / 634 RKC, 4,096 cells 76.9 ->
-// 38.4 ms; 111 / 1566 RKC, 16 instances of 2,000 cells in all 1067 -> 222 ms;
-// 13 / 54 RKC, 1,000 cells 3.70 -> 3.11 ms; 9 / 38 RKCK, 4,096 cells 0.715 ->
-// 0.457 ms. Error of whole results against plain FP64: unchanged (1e-13, the
-// finite differences of the spectral radius).
+// Whole calls on GB300, before and after: 53 / 634 RKC, 4,096 cells 76.1 ->
+// 38.4 ms; 111 / 1566 RKC, 16 instances of 2,000 cells in all 1061 -> 226 ms;
+// 13 / 54 RKC, 1,000 cells 3.75 -> 3.03 ms, 30,011 cells 38.4 -> 15.3; 9 / 38 RKCK,
+// 4,096 cells 0.716 -> 0.468 ms; energy equation, 13 / 54, 20,000 cells 67.1 -> 13.3;
+// f alone, 53 / 634, 50,000 cells 2.81 -> 0.71 ms. Error of whole results
+// against plain FP64: unchanged (1e-13, the finite differences of the spectral
+// radius).
 #pragma once
 #include "intf.cuh"
 #include "kernels.cuh"
