@@ -592,6 +592,7 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     for (int i = 0; i < nS; ++i) {
         imW[2 * i] = int_split(1.0L / d->W[i], &imWe[2 * i]);
         imW[2 * i + 1] = int_split(d->W[i], &imWe[2 * i + 1]);
+        if (ptr[i + 1] == ptr[i]) imW[2 * i + 1] = 0;  // no reaction changes it
     }
     int imLow = 0;
     for (int j = 0; j < nR; ++j)
@@ -693,6 +694,7 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.imW = (const ulonglong2*)(b + oImW);
     M.imWe = (const int2*)(b + oImWe);
     M.imLow = imLow;
+    int_word_bits(nS, ptr.data(), cnu.data(), &M.imUp, &M.imShort);
     M.li_n = li.n;
     M.li_tb = li.tb;
     M.li_rx = use_li ? (const uint4*)(b + oLiRx) : nullptr;

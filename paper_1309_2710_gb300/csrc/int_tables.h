@@ -108,6 +108,24 @@ inline IntGather build_int_gather(int nS, int nR, const int* ptr, const int* pos
     return t;
 }
 
+// How far up the largest rate's word is shifted, and how many bits a sum needs
+// for its last place to be worth an ulp (intf.cuh), for species-major rows whose
+// longest counts n entries: n words below 2^(61 + up + 8) stay below 2^127, and n
+// units below the sum's 53rd bit. Up to 55 bits, so that a word's shift stays
+// below 64.
+inline void int_word_bits(int nS, const int* ptr, const double* nu, int* up, int* enough)
+{
+    int n = 1, bits = 0;
+    for (int i = 0; i < nS; ++i) {
+        int c = 0;
+        for (int e = ptr[i]; e < ptr[i + 1]; ++e) c += (int)std::abs(nu[e]);
+        n = std::max(n, c);
+    }
+    while (n >> bits) ++bits;
+    *up = std::min(55, 58 - bits);
+    *enough = 53 + bits;
+}
+
 // 63-bit left-aligned mantissa of v > 0 and its exponent as in a double.
 inline uint64_t int_split(long double v, int* e)
 {

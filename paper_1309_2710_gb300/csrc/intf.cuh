@@ -11,9 +11,10 @@
 //    mantissa and an exponent, exact for every normal double; a product
 //    keeps the top 62 bits of the mantissas' product (three IMAD.WIDE, 6
 //    cycles for a DMUL's 64);
-//  * a rate of progress is placed into a 128-bit fixed-point word whose unit
-//    is 2^-99 (at most 2^-83) of the largest rate of the evaluation, so every sum of
-//    rates is exact (four 32-bit adds) but for the words' own last bits;
+//  * a rate of progress is placed into a 128-bit fixed-point word whose unit is
+//    far below the largest rate of the evaluation, so every sum of rates is
+//    exact (four 32-bit adds) but for the words' own last bits; sums that these
+//    bits could matter to are formed again with a lower unit (IM_STEP below);
 //  * a third-body sum multiplies 55-bit integer efficiencies by the
 //    concentrations as 55-bit fractions of the total.
 // Every product, sum and third-body sum is at least as accurate as its FP64
@@ -52,7 +53,8 @@ __device__ __forceinline__ void im_split(double v, im_u64& m, uint32_t& e)
     m = x ? n << 10 : 0ull;
 }
 
-// The same of a positive double; zero and denormals read as about 2^-1023.
+// The same of a positive double; zero and denormals read as about 2^-1023
+// (im_normal_k tells).
 __device__ __forceinline__ void im_split_k(double v, im_u64& m, uint32_t& e)
 {
     const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
@@ -60,6 +62,7 @@ __device__ __forceinline__ void im_split_k(double v, im_u64& m, uint32_t& e)
     m = (((im_u64)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 10;
 }
 
+__device__ __forceinline__ bool im_normal_k(double v) { return ((uint32_t)__double2hiint(v) >> 20) != 0u; }
 __device__ __forceinline__ bool im_finite_k(double v) { return ((uint32_t)__double2hiint(v) >> 20) < 0x7ffu; }
 __device__ __forceinline__ bool im_finite_k(float v) { return (__float_as_uint(v) >> 23) < 0xffu; }
 
@@ -106,7 +109,8 @@ inline void im_sub(im_u128& a, im_u64 lo, im_u64 hi)
 }
 #endif
 
-// Q * 2^L as a 128-bit word, Q < 2^61, L <= 63; bits below the unit drop.
+// Q * 2^L as a 128-bit word, Q < 2^61, L <= 63 (any L gives some word); bits
+// below the unit drop.
 __device__ __forceinline__ im_u128 im_place(im_u64 Q, int L)
 {
     im_u128 r;
@@ -126,6 +130,26 @@ __device__ __forceinline__ double im_round(im_u64 r, int x, bool neg)
     if (n <= 0) b = 0ull;
     if (n >= 0x7ff) b = 0x7ff0000000000000ull;
     return __longlong_as_double((long long)(neg ? b | 0x8000000000000000ull : b));
+}
+
+// a * 2^-d of a signed 128-bit word, d >= 0.
+__device__ __forceinline__ void im_sar(im_u128& a, int d)
+{
+    for (int k = 0; k < 2 && d >= 64; ++k, d -= 64) {
+        a.lo = a.hi;
+        a.hi = (im_u64)((long long)a.hi >> 63);
+    }
+    if (d == 0 || d >= 64) return;
+    a.lo = a.lo >> d | a.hi << (64 - d);
+    a.hi = (im_u64)((long long)a.hi >> d);
+}
+
+// Whether a signed 128-bit word has at most t bits.
+__device__ __forceinline__ bool im_short(im_u128 a, int t)
+{
+    const im_u64 s = (im_u64)((long long)a.hi >> 63);
+    const im_u64 hi = a.hi ^ s, lo = a.lo ^ s;
+    return t < 64 ? (hi | im_shr(lo, (uint32_t)t)) == 0ull : im_shr(hi, (uint32_t)(t - 64)) == 0ull;
 }
 
 // (a 2^x) (u 2^(eu - IM_BIAS)) (v 2^(ev - IM_BIAS)) of a signed 128-bit word and
@@ -213,12 +237,25 @@ __device__ __forceinline__ double im_log(const ulonglong2* __restrict__ tab, dou
     return im_round(l + c.y + (q >> 3), -59, false);
 }
 
-// Bits a word of the largest rate (e = the evaluation's scale) is shifted up:
-// Q < 2^61, so it stays below 2^(61 + 43 + 8) where the scale is IM_GUARD octaves
-// too low, which leaves 15 bits for a row's entries and the sign. The words'
-// unit is 2^-99 of the largest rate (Q >= 2^56), 2^-83 where the scale is
-// IM_SLACK octaves too high.
-constexpr int IM_UP = 43, IM_GUARD = 8, IM_SLACK = 16;
+// A word of the largest rate (e = the evaluation's scale) is shifted up by
+// MechDev::imUp bits (int_word_bits of int_tables.h): Q < 2^61, so it stays below
+// 2^(61 + imUp + 8) where the scale is IM_GUARD octaves too low, which leaves
+// room for the entries of the mechanism's longest row and the sign. The words'
+// unit is 2^-105 of the largest rate for rows of up to 127 entries (Q >= 2^54),
+// 2^-97 where the scale is IM_SLACK octaves too high.
+//
+// A row's sum of fewer than MechDev::imShort = 53 + log2(entries) bits could
+// miss an ulp in the bits below the unit: a species whose rates are all far
+// below the cell's largest, or whose rates cancel. Such rows are summed again on
+// their own: with a unit of their own largest rate (int_row_sum, one lane's
+// work), or in the lane layout, all of them together, with the unit IM_STEP octaves
+// lower, modulo 2^128 (the sum itself fits, the words that do not wrap around), and
+// so on until each has its bits or no rate has bits below the unit, when the sums
+// are exact (lane_int_lower). The workloads' cells have no net rate below 2^-36 of
+// their largest, and a net rate of 2^-37 has its bits, so that they pay for the
+// test alone, 1 to 2 % of a call. Inside the common code the further sums' registers
+// and branches would cost 5 to 38 %.
+constexpr int IM_GUARD = 8, IM_SLACK = 8, IM_STEP = 56;
 
 // Exponent that stands for a rate that is not finite.
 constexpr int IM_OUT = 1 << 20;

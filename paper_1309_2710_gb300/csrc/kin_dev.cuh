@@ -93,9 +93,10 @@ struct MechDev {
     const double* arr0;    // [3][nFO] the low-pressure limits'
     const unsigned long long* ex2;  // tables of im_exp and im_log
     const ulonglong2* lnc;
-    const ulonglong2* imW; // [nS] 63-bit mantissas of 1 / W and W
+    const ulonglong2* imW; // [nS] 63-bit mantissas of 1 / W and W (0: no reaction changes the species)
     const int2* imWe;      // [nS] their exponents
     int imLow;             // 1: a reaction of fewer than two factors of concentration
+    int imUp, imShort;     // shift of the largest rate's word, bits that a sum needs (intf.cuh)
     // the lane layout's integer FP64 f (lane_int.cuh): reactions with a net
     // effect, third bodies first; null where it does not apply
     int li_n, li_tb;

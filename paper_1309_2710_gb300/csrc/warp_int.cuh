@@ -188,11 +188,33 @@ struct Group {
 template <int NR, int G>
 __host__ __device__ constexpr int group_set_words() { return G > 32 ? NR * G : 0; }
 
+// Where f's rate constants come from: stored (isothermal), or exp(ln A + beta ln T
+// - (E / R) / T) at this temperature (K null).
+struct RateSource {
+    const double* K;
+    double lnT, invT;
+};
+
+// The cell's mixture, with mantissas and exponents of rho and 1 / rho.
+struct IntMix {
+    double rho;
+    im_u64 mr, mi;
+    uint32_t er, ei;
+    int eT;  // exponent of the sum of Y_k / W_k
+};
+
+// What int_row_sum reads of the cell beside its concentrations.
+struct IntCell {
+    IntMix mix;
+    RateSource rk;
+};
+
 // The group's shared arrays.
 struct IntSmem {
     ulonglong2* OM;  // [chunk + 1] rates of progress of a chunk, and a zero word
     ulonglong2* P;   // [nslots] partial sums
     int2* CF;        // [nS, even] concentrations as 55-bit fractions: 30 high, 25 low bits
+    IntCell* cell;
     im_u64* CM;      // [nS + 1] mantissas, after the constant 1 that empty slots read
     uint32_t* CE;    // [nS + 1] exponent words
 
@@ -200,8 +222,15 @@ struct IntSmem {
     {
         OM = reinterpret_cast<ulonglong2*>(base);
         P = OM + I.chunk + 1;
-        CF = reinterpret_cast<int2*>(P + I.nslots);
-        CM = reinterpret_cast<im_u64*>(CF + ((M.nS + 1) & ~1));
+        species(M, reinterpret_cast<int2*>(P + I.nslots));
+    }
+    // (without OM and P, from the first of the species' arrays)
+    __device__ IntSmem(const MechDev& M, int2* f) : OM(nullptr), P(nullptr) { species(M, f); }
+    __device__ void species(const MechDev& M, int2* f)
+    {
+        CF = f;
+        cell = reinterpret_cast<IntCell*>(CF + ((M.nS + 1) & ~1));
+        CM = reinterpret_cast<im_u64*>(cell + 1);
         CE = reinterpret_cast<uint32_t*>(CM + M.nS + 1);
     }
 };
@@ -209,7 +238,7 @@ struct IntSmem {
 // Shared FP64 words of a group, a multiple of 4.
 __host__ __device__ __forceinline__ int int_smem_words(const MechDev& M, const IntDev& I)
 {
-    const int w = 2 * (I.chunk + 1 + I.nslots) + ((M.nS + 1) & ~1) + M.nS + 1 + (M.nS + 2) / 2;
+    const int w = 2 * (I.chunk + 1 + I.nslots) + ((M.nS + 1) & ~1) + (int)sizeof(IntCell) / 8 + M.nS + 1 + (M.nS + 2) / 2;
     return (w + 3) & ~3;
 }
 
@@ -238,13 +267,6 @@ static __device__ __noinline__ double int_row_dot_slow(const MechDev& M, int row
 {
     return int_row_dot(M, row, [&](int k) { return int_conc(S, k); });
 }
-
-// Where f's rate constants come from: stored (isothermal), or exp(ln A + beta ln T
-// - (E / R) / T) at this temperature (K null).
-struct RateSource {
-    const double* K;
-    double lnT, invT;
-};
 
 // The exponents of reaction position q and falloff ordinal fo.
 __device__ __forceinline__ double rate_exponent(const MechDev& M, int q, const RateSource& k)
@@ -303,6 +325,138 @@ __device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, 
     grp.sync();
 }
 
+// The rate of progress of the reaction at position q (over a common power of rho) as
+// Q < 2^61 and exponent word, from its reactants' word and its rate constant
+// (kq), or ln A, beta and E / R (AT_T). False where it is not finite. AHEAD: eight
+// efficiencies in flight.
+template <bool AT_T, bool AHEAD>
+__device__ __forceinline__ bool int_rate(const MechDev& M, const IntSmem& S, const RateSource& rk, const IntMix& mix,
+                                         int q, uint32_t w, double kq, double bq, double eq, im_u64& Q, uint32_t& e)
+{
+    const int nS = M.nS, nR = M.nR, nM = M.nM, nP = nR - nM, nF = nR - M.nFO;
+    bool in = true;
+    double a = 0.0;
+    if constexpr (AT_T) {
+        a = fma(-eq, rk.invT, fma(bq, rk.lnT, kq));
+        if (!im_exp(M.ex2, a, Q, e)) in = false;
+    } else {
+        im_split_k(kq, Q, e);
+    }
+    const uint32_t ra = w & 0xffffu, rb = w >> 16;
+    Q = im_mul(im_mul(S.CM[ra], S.CM[rb]), Q);
+    e += S.CE[ra] + S.CE[rb];
+    if (q >= nP) {
+        const int row = q - nP;
+        const int4* __restrict__ E = M.effI + row;
+        const int4* F = reinterpret_cast<const int4*>(S.CF);
+        long long hi = 0, mid = 0;
+        auto term = [&](const int4& u, const int4& f) {
+            hi += (long long)u.x * f.x;
+            mid += (long long)u.x * f.y;
+            mid += (long long)u.y * f.x;
+            hi += (long long)u.z * f.z;
+            mid += (long long)u.z * f.w;
+            mid += (long long)u.w * f.z;
+        };
+        const int n2 = (nS + 1) >> 1;
+        int k = 0;
+#pragma unroll 1
+        for (; AHEAD && k + 7 < n2; k += 8) {
+            int4 u[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) u[j] = E[(int64_t)(k + j) * nM];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) term(u[j], F[k + j]);
+        }
+        if constexpr (AHEAD) {
+#pragma unroll 4
+            for (; k < n2; ++k) term(E[(int64_t)k * nM], F[k]);
+        } else {
+#pragma unroll 1
+            for (; k < n2; ++k) term(E[(int64_t)k * nM], F[k]);
+        }
+        const long long U = hi + (mid >> 25);
+        double Md = 0.0;
+        im_u64 mm;
+        uint32_t em;
+        if (U < (1ll << 54)) {  // small beside its terms: the fractions are too coarse
+            Md = int_row_dot_slow(M, row, S);
+            im_split(Md, mm, em);
+            Md *= mix.rho;
+        } else {
+            const int z = __clzll(U);
+            mm = (im_u64)U << (z - 1);
+            em = (uint32_t)(M.effX[row] + mix.eT + 5 - z);
+            if (!AT_T && q >= nF) Md = im_round(mm, (int)em - IM_BIAS, false) * mix.rho;
+        }
+        if (q >= nF) {
+            double Pr;
+            if constexpr (AT_T) {
+                im_u64 km;
+                uint32_t ke;
+                if (!im_exp(M.ex2, low_exponent(M, q - nF, rk) - a, km, ke)) in = false;
+                Pr = im_round(im_mul(km, mm), (int)ke + (int)(em & 0x7fffffffu) - 2 * IM_BIAS + 64, (int)em < 0) * mix.rho;
+            } else {
+                Pr = __dmul_rn(rk.K[nR + (q - nF)], Md);
+            }
+            im_split(falloff_factor(Pr), mm, em);
+            if ((em & 0x7ffu) == 0x7ffu) in = false;
+        }
+        Q = im_mul(Q, mm);
+        e += em - (uint32_t)(IM_BIAS - 64);
+    }
+    // the rate is rho^2 of what a plain reaction of two gives here
+    if (q >= nP || M.imLow) {
+        int p = (ra != 0u) + (rb != 0u) + (q >= nP && q < nF) - 2;
+        for (; p > 0; --p) {
+            Q = im_mul(Q, mix.mr);
+            e += mix.er - (uint32_t)(IM_BIAS - 64);
+        }
+        for (; p < 0; ++p) {
+            Q = im_mul(Q, mix.mi);
+            e += mix.ei - (uint32_t)(IM_BIAS - 64);
+        }
+    }
+    return in;
+}
+
+// W_i omega_i / rho of a species whose words are too short for it (intf.cuh): its
+// rates once more, one after another, placed by the largest of them so far. One
+// lane's chain, and rarely taken, so it is out of line, with rolled loops, and
+// reads the cell's values from shared memory: with more of its registers around,
+// cells without such species lose up to 8 % (now 2 %; GB300, 53 species / 634
+// reactions, 4,096 cells 20.2 -> 20.4 ms, 21.9 with its third-body sum unrolled).
+template <bool AT_T>
+static __device__ __noinline__ double int_row_sum(const MechDev& M, int2* CF, int i)
+{
+    const IntSmem S(M, CF);
+    const IntMix mix = S.cell->mix;
+    const RateSource rk = S.cell->rk;
+    constexpr int UP = 43;  // 61 + 43 bits and the entries of the longest row, two for each reaction
+    im_u128 acc{0ull, 0ull};
+    int at = -1;
+#pragma unroll 1
+    for (int c = M.csr_ptr[i]; c < M.csr_ptr[i + 1]; ++c) {
+        const int q = M.csrp_rxn[c];
+        const double nu = M.csr_nu[c], kq = AT_T ? M.arr[q] : rk.K[q];
+        im_u64 Q;
+        uint32_t e;
+        int_rate<AT_T, false>(M, S, rk, mix, q, M.rxw[q], kq, AT_T ? M.arr[M.nR + q] : 0.0, AT_T ? M.arr[2 * M.nR + q] : 0.0, Q, e);
+        if (!Q || (!AT_T && !im_normal_k(kq))) continue;
+        const int x = (int)(e & 0x7fffffffu);
+        if (x > at) {
+            im_sar(acc, x - max(at, 0));
+            at = x;
+        }
+        const im_u128 v = im_place(Q, x - at + UP);
+        const bool neg = (e >> 31 != 0u) != (nu < 0.0);
+        for (int n = (int)fabs(nu); n > 0; --n)
+            if (neg) im_sub(acc, v.lo, v.hi);
+            else im_add(acc, v.lo, v.hi);
+    }
+    return im_scaled(acc, at - UP - 3 * IM_BIAS, M.imW[i].y, M.imWe[i].y, mix.mr, (int)mix.er);
+}
+
 // f for the group's cell. `scale` is the exponent that the fixed-point words are
 // placed by, kept by the caller from one evaluation of the cell to the next
 // (any value at the first); an evaluation whose largest rate is more than
@@ -314,7 +468,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                                                int& scale, const double (&x)[NR], double (&out)[NR], int lane,
                                                Group<G>& grp)
 {
-    const int nS = M.nS, nR = M.nR, nM = M.nM;
+    const int nS = M.nS, nR = M.nR;
     // c_k / rho = Y_k / W_k: in FP64 for the mixture sum, and as mantissa and
     // exponent word (64 above the double's, so that 1 / W never takes it below
     // zero) for everything else
@@ -345,14 +499,14 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
     const int eT = (int)(top >> 20);
     // finite, and no species below -2^-9 of the total
     in = in && top - 0x00100000u < 0x7fe00000u && neg + 9 <= eT + 64;
-    im_u64 mr, mi = 0ull;  // rho and 1 / rho
-    uint32_t er, ei = 0u;
-    im_split_k(rho, mr, er);
-    if (M.imLow) im_split_k(s * invCtot, mi, ei);
+    IntMix mix{rho, 0ull, 0ull, 0u, 0u, eT};
+    im_split_k(rho, mix.mr, mix.er);
+    if (M.imLow) im_split_k(s * invCtot, mix.mi, mix.ei);
     if (lane == 0) {
         S.CM[0] = 1ull << 62;
         S.CE[0] = 1023u + 64u;
         S.OM[I.chunk] = make_ulonglong2(0ull, 0ull);
+        *S.cell = IntCell{mix, rk};
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
@@ -360,7 +514,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         if (i < nS) {
             S.CM[i + 1] = m[r];
             S.CE[i + 1] = e[r];
-            if (nM) {
+            if (M.nM) {
                 // 2^55 of twice the total at most: sum |F| < 3 * 2^55
                 long long F = (long long)((im_shr(m[r], (uint32_t)(eT - (int)(e[r] & 0xfffu) + 71)) + 1ull) >> 1);
                 if ((int)e[r] < 0) F = -F;
@@ -374,23 +528,16 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         int_general<NR, G>(M, S, rk, c, rho, invCtot * s, out, lane, grp);
         return;
     }
-    const int nP = nR - nM, nF = nR - M.nFO;
     im_u128 acc[NR];
     for (;;) {
 #pragma unroll
         for (int r = 0; r < NR; ++r) acc[r] = im_u128{0ull, 0ull};
         int emax = 0;
         bool over = false, under = false;
-        // K C C of a reaction, from its reactants' word and its rate constant in Q, e
-        auto product = [&](uint32_t w, im_u64& Q, uint32_t& e) {
-            const uint32_t a = w & 0xffffu, b = w >> 16;
-            Q = im_mul(im_mul(S.CM[a], S.CM[b]), Q);
-            e += S.CE[a] + S.CE[b];
-        };
         auto store = [&](im_u64 Q, uint32_t e, int at) {
             const int x = (int)(e & 0x7fffffffu);
             if (Q) emax = max(emax, x);
-            im_u128 v = im_place(Q, min(x - scale + IM_UP, 63));
+            im_u128 v = im_place(Q, x - scale + M.imUp);
             if (e >> 31) {
                 im_u128 z{0ull, 0ull};
                 im_sub(z, v.lo, v.hi);
@@ -423,81 +570,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                 if (q + G < nR) fetch(q + G);
                 im_u64 Q;
                 uint32_t e;
-                double a = 0.0;
-                if constexpr (AT_T) {
-                    a = fma(-eq, rk.invT, fma(bq, rk.lnT, kq));
-                    if (!im_exp(M.ex2, a, Q, e)) emax = IM_OUT;
-                } else {
-                    im_split_k(kq, Q, e);
-                }
-                product(w, Q, e);
-                if (q >= nP) {
-                    const int row = q - nP;
-                    const int4* __restrict__ E = M.effI + row;
-                    const int4* F = reinterpret_cast<const int4*>(S.CF);
-                    long long hi = 0, mid = 0;
-                    auto term = [&](const int4& u, const int4& f) {
-                        hi += (long long)u.x * f.x;
-                        mid += (long long)u.x * f.y;
-                        mid += (long long)u.y * f.x;
-                        hi += (long long)u.z * f.z;
-                        mid += (long long)u.z * f.w;
-                        mid += (long long)u.w * f.z;
-                    };
-                    const int n2 = (nS + 1) >> 1;
-                    int k = 0;
-#pragma unroll 1
-                    for (; k + 7 < n2; k += 8) {
-                        int4 u[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) u[j] = E[(int64_t)(k + j) * nM];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) term(u[j], F[k + j]);
-                    }
-#pragma unroll 4
-                    for (; k < n2; ++k) term(E[(int64_t)k * nM], F[k]);
-                    const long long U = hi + (mid >> 25);
-                    double Md = 0.0;
-                    im_u64 mm;
-                    uint32_t em;
-                    if (U < (1ll << 54)) {  // small beside its terms: the fractions are too coarse
-                        Md = int_row_dot_slow(M, row, S);
-                        im_split(Md, mm, em);
-                        Md *= rho;
-                    } else {
-                        const int z = __clzll(U);
-                        mm = (im_u64)U << (z - 1);
-                        em = (uint32_t)(M.effX[row] + eT + 5 - z);
-                        if (!AT_T && q >= nF) Md = im_round(mm, (int)em - IM_BIAS, false) * rho;
-                    }
-                    if (q >= nF) {
-                        double Pr;
-                        if constexpr (AT_T) {
-                            im_u64 km;
-                            uint32_t ke;
-                            if (!im_exp(M.ex2, low_exponent(M, q - nF, rk) - a, km, ke)) emax = IM_OUT;
-                            Pr = im_round(im_mul(km, mm), (int)ke + (int)(em & 0x7fffffffu) - 2 * IM_BIAS + 64, (int)em < 0) * rho;
-                        } else {
-                            Pr = __dmul_rn(rk.K[nR + (q - nF)], Md);
-                        }
-                        im_split(falloff_factor(Pr), mm, em);
-                        if ((em & 0x7ffu) == 0x7ffu) emax = IM_OUT;
-                    }
-                    Q = im_mul(Q, mm);
-                    e += em - (uint32_t)(IM_BIAS - 64);
-                }
-                // the rate is rho^2 of what a plain reaction of two gives here
-                if (q >= nP || M.imLow) {
-                    int p = ((w & 0xffffu) != 0u) + (w >> 16 != 0u) + (q >= nP && q < nF) - 2;
-                    for (; p > 0; --p) {
-                        Q = im_mul(Q, mr);
-                        e += er - (uint32_t)(IM_BIAS - 64);
-                    }
-                    for (; p < 0; ++p) {
-                        Q = im_mul(Q, mi);
-                        e += ei - (uint32_t)(IM_BIAS - 64);
-                    }
-                }
+                if (!int_rate<AT_T, true>(M, S, rk, mix, q, w, kq, bq, eq, Q, e)) emax = IM_OUT;
                 store(Q, e, q - q0);
             }
             // the run's first entries, fetched ahead of the barrier
@@ -546,11 +619,24 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
             }
         }
         if (!over && !under) {
+            unsigned left = 0u;
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const int i = lane + G * r;
-                // a word's unit at e = scale: 2^(128 + scale - 2 * 64 - 3 IM_BIAS - IM_UP)
-                out[r] = i < nS ? im_scaled(acc[r], scale - 3 * IM_BIAS - IM_UP, M.imW[i].y, M.imWe[i].y, mr, (int)er) : 0.0;
+                out[r] = 0.0;
+                if (i >= nS) continue;
+                const im_u64 w = M.imW[i].y;  // 0: no reaction changes the species
+                // a word's unit at e = scale: 2^(128 + scale - 2 * 64 - 3 IM_BIAS - imUp)
+                if (w && im_short(acc[r], M.imShort)) left |= 1u << r;
+                out[r] = im_scaled(acc[r], scale - M.imUp - 3 * IM_BIAS, w, M.imWe[i].y, mix.mr, (int)mix.er);
+            }
+#pragma unroll 1
+            for (; left; left &= left - 1u) {
+                const int k = __ffs(left) - 1;
+                const double v = int_row_sum<AT_T>(M, S.CF, lane + G * k);
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (r == k) out[r] = v;
             }
             // the shared words are rewritten by the next evaluation (across
             // warps, only after the barrier of its mixture sum)
