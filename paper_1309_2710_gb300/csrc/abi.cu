@@ -608,6 +608,12 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
         arr0[nFO + fo] = beta0[j];
         arr0[2 * nFO + fo] = Ea0R[j];
     }
+    std::vector<uint32_t> scl(4 * nR);
+    for (int q = 0; q < nR; ++q) {
+        const int j = perm[q];
+        int_scale_table(d->lnA[j], d->beta[j], EaR[j], d->reac + 2 * j, d->type[j], q >= nPlain ? effX[q - nPlain] : 0, &scl[4 * q]);
+    }
+    const size_t oScl = put(scl.data(), 4 * scl.size());
     uint64_t ex2[64], lnc[128];
     int_exp_log_tables(ex2, lnc);
     const size_t oArr = put(arr.data(), 8 * arr.size()), oArr0 = put(arr0.data(), 8 * arr0.size());
@@ -689,6 +695,7 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.effX = (const int32_t*)(b + oEffX);
     M.arr = (const double*)(b + oArr);
     M.arr0 = (const double*)(b + oArr0);
+    M.scl = (const uint4*)(b + oScl);
     M.ex2 = (const unsigned long long*)(b + oEx2);
     M.lnc = (const ulonglong2*)(b + oLnc);
     M.imW = (const ulonglong2*)(b + oImW);

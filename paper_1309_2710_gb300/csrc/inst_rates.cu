@@ -4,9 +4,9 @@
 // A cell of 53 species / 634 reactions takes 659 exponentials and 8,160 other
 // operations; on the FP64 pipe the exponentials alone (some 20 instructions
 // each) take 1.1 ms for 50,000 cells, and the lane-per-cell form streamed its
-// rate constants and rates of progress through L2 besides: 2.80 ms, 0.71 now.
-// The group keeps its scale from cell to cell (warp_feval_int), so the last bits
-// of rates below 2^-83 of a cell's largest may depend on the cell before it.
+// rate constants and rates of progress through L2 besides: 2.80 ms, 0.76 now.
+// Each cell's scale comes from the cell itself (int_first_scale), so its bits do
+// not depend on the call's other cells.
 #include "warp.cuh"
 
 namespace kin {
@@ -21,7 +21,6 @@ __global__ void __launch_bounds__(128, 4)
     const IntSmem S(M, I, base);
     Group<G> grp(nullptr, 0);
     const int lane = threadIdx.x & (G - 1);
-    int scale = 0;
     const int64_t ngroups = (int64_t)gridDim.x * (blockDim.x / G);
     const int64_t first = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     // every group of a warp takes part in every pass; those past the end repeat
@@ -30,6 +29,7 @@ __global__ void __launch_bounds__(128, 4)
         const int64_t c = c0 < cells ? c0 : cells - 1;
         const double t = T[c], pR = p[c] * (1e-6 / R_GAS), invT = Tab<double>::inv(t);
         double x[NR], out[NR];
+        int scale = -1;
 #pragma unroll
         for (int r = 0; r < NR; ++r) x[r] = lane + G * r < M.nS ? Y[(int64_t)(lane + G * r) * ldY + c] : 0.0;
         warp_feval_int<NR, G, true>(M, I, S, rates_at(M, t, invT), true, pR * invT, Tab<double>::inv(pR) * t, scale, x,

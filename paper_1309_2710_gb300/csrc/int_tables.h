@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <vector>
 
 namespace kin {
@@ -167,6 +168,21 @@ inline int int_efficiencies(int nS, const double* eff, int32_t* hi, int32_t* lo)
         lo[k] = (int32_t)(E & ((1 << 25) - 1));
     }
     return x;
+}
+
+// A reaction's entry of the estimate of a cell's largest rate (int_first_scale of
+// warp_int.cuh): three floats, whose sum with weights 1, ln T and -1 / T is the
+// rate's exponent word (a double's exponent) without the concentrations' two (and
+// the third body's eT), and reactants (0: none) | power of rho + 2 << 20 | third body << 23.
+// row: the exponent of its largest efficiency.
+inline void int_scale_table(double lnA, double beta, double EaR, const int32_t* reac, int type, int row, uint32_t* out)
+{
+    const double log2e = 1.4426950408889634;
+    const float f[3] = {(float)(lnA * log2e + 1023 + (type == 1 ? row + 1 - 1021 : type == 2)), (float)(beta * log2e),
+                        (float)(EaR * log2e)};
+    std::memcpy(out, f, sizeof(f));
+    const int power = (reac[0] >= 0) + (reac[1] >= 0) + (type == 1) - 2;
+    out[3] = (uint32_t)(reac[0] + 1) | (uint32_t)(reac[1] + 1) << 10 | (uint32_t)(power + 2) << 20 | (type == 1 ? 1u << 23 : 0u);
 }
 
 // Tables of the lane layout's f (lane_int.cuh): its reactions in the order

@@ -91,6 +91,7 @@ struct MechDev {
     const int32_t* effX;   // [nM] their exponents
     const double* arr;     // [3][nR] ln A, beta, E / R in permutation order
     const double* arr0;    // [3][nFO] the low-pressure limits'
+    const uint4* scl;      // [nR] estimate of the rates' exponents (int_scale_table)
     const unsigned long long* ex2;  // tables of im_exp and im_log
     const ulonglong2* lnc;
     const ulonglong2* imW; // [nS] 63-bit mantissas of 1 / W and W (0: no reaction changes the species)

@@ -426,7 +426,7 @@ struct WarpRKC {
     int lane, nV;  // nV: state length, nS + 1 with the energy equation
     Group<G> grp;
     unsigned mask; // the group's lanes in this warp
-    int scale;     // of the integer FP64 f, kept from one evaluation to the next
+    int scale;     // of the integer FP64 f, kept from one evaluation of a cell to the next
     bool kfin;     // the cell's rate constants are finite
     double Ctot, invCtot, atol, rtol, p;
     R CtotR, invCtotR;   // the same in the rate type
@@ -1039,8 +1039,8 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
             W.grp.sync();
             W.Kc = ks;
             if (sizeof(R) == 8) W.kfin = W.grp.all(kfin);
-            W.scale = 0;
         }
+        W.scale = EN ? -1 : 0;
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const int i = lane + G * r;
@@ -1109,7 +1109,7 @@ __device__ __forceinline__ uint8_t warp_load_cell(WarpRKC<R, NR, EN, G>& W, cons
     W.atol = I.atol;
     W.rtol = I.rtol;
     W.p = p;
-    W.scale = 0;
+    W.scale = EN ? -1 : 0;
     if constexpr (EN) {
         W.Kc = nullptr;
     } else {
@@ -1254,7 +1254,7 @@ struct WarpRKCK {
     int lane, nV;
     Group<G> grp;
     unsigned mask;  // the group's lanes
-    int scale;      // of the integer FP64 f, kept from one evaluation to the next
+    int scale;      // of the integer FP64 f, kept from one evaluation of a cell to the next
     bool kfin;      // the cell's rate constants are finite
     double Ctot, invCtot, atol, rtol, p;
     R CtotR, invCtotR;  // the same in the rate type
@@ -1412,8 +1412,8 @@ __global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const _
             __syncwarp(W.mask);
             W.Kc = kc;
             if (sizeof(R) == 8) W.kfin = __all_sync(W.mask, kfin);
-            W.scale = 0;
         }
+        W.scale = EN ? -1 : 0;
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const int i = lane + G * r;

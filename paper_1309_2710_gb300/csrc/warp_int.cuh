@@ -457,9 +457,36 @@ static __device__ __noinline__ double int_row_sum(const MechDev& M, int2* CF, in
     return im_scaled(acc, at - UP - 3 * IM_BIAS, M.imW[i].y, M.imWe[i].y, mix.mr, (int)mix.er);
 }
 
+// About the largest rate's exponent of the lane's reactions, for the first
+// evaluation of a cell: a few octaves too high where a third-body sum is small
+// beside its largest efficiency, more where a falloff is. A function of the cell
+// alone, in FP32 from a table of its own (int_scale_table) and without the third-body
+// sums; a whole evaluation to find the scale would double kin_rates.
+__device__ __forceinline__ int int_first_scale(const MechDev& M, const IntSmem& S, const RateSource& rk, const IntMix& mix,
+                                               int lane, int lanes)
+{
+    const float lnT = im_f32(rk.lnT), invT = im_f32(rk.invT);
+    const int nP = M.nR - M.nM;
+    int top = 0;
+#pragma unroll 4
+    for (int q = lane; q < M.nR; q += lanes) {
+        const uint4 d = M.scl[q];
+        const float a = fmaf(-__uint_as_float(d.z), invT, fmaf(__uint_as_float(d.y), lnT, __uint_as_float(d.x)));
+        int e = (int)floorf(a) + (int)((S.CE[d.w & 0x3ffu] + S.CE[d.w >> 10 & 0x3ffu]) & 0x7fffffffu);
+        if (q >= nP || M.imLow) {
+            const int p = (int)(d.w >> 20 & 7u) - 2;  // of rho, beyond a plain reaction of two
+            if (d.w >> 23) e += mix.eT;
+            e += p > 0 ? p * ((int)mix.er - (IM_BIAS - 64)) : -p * ((int)mix.ei - (IM_BIAS - 64));
+        }
+        top = max(top, e);
+    }
+    return top;
+}
+
 // f for the group's cell. `scale` is the exponent that the fixed-point words are
 // placed by, kept by the caller from one evaluation of the cell to the next
-// (any value at the first); an evaluation whose largest rate is more than
+// (at the first a value that does not depend on other cells, for the bits of the
+// result not to; AT_T: -1, and int_first_scale gives one); an evaluation whose largest rate is more than
 // IM_GUARD octaves above it or IM_SLACK below is repeated with that rate's. The
 // barriers around the gather carry the two tests. kfin: the cell's rate constants are finite.
 template <int NR, int G, bool AT_T>
@@ -527,6 +554,9 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
     if (grp.sync_any(!in)) {
         int_general<NR, G>(M, S, rk, c, rho, invCtot * s, out, lane, grp);
         return;
+    }
+    if constexpr (AT_T) {
+        if (scale < 0) scale = grp.imax(int_first_scale(M, S, rk, mix, lane, G));
     }
     im_u128 acc[NR];
     for (;;) {

@@ -109,7 +109,7 @@ struct Mech {
     IntGather g;
     LaneInt li;
     std::vector<double> W, invW, arr, arr0, effV64, nu;
-    std::vector<uint32_t> rxw;
+    std::vector<uint32_t> rxw, scl;
     std::vector<int> perm, ptr, pos;
     std::vector<int32_t> effI, effX, imWe, liE;
     std::vector<uint64_t> imW, ex2, lnc;
@@ -171,7 +171,7 @@ extern "C" void* mech_new(int nS, int nR, const double* W, const double* lnA, co
     MechDev& M = m->M;
     M.nS = nS; M.nR = nR; M.nM = nM; M.nFO = nFO;
     for (int j = 0; j < nR; ++j) if ((reac[2 * j] >= 0) + (reac[2 * j + 1] >= 0) + (type[j] == 1) < 2) M.imLow = 1;
-    tables(*m, eff, row.data());
+    tables(*m, eff, row.data(), reac, type);
     M.W = m->W.data(); M.invW = m->invW.data();
     M.csr_ptr = m->ptr.data(); M.csrp_rxn = m->pos.data(); M.csr_nu = m->nu.data();
     M.rxw = m->rxw.data(); M.arr = m->arr.data(); M.arr0 = m->arr0.data(); M.effV64 = m->effV64.data();
@@ -225,7 +225,7 @@ extern "C" int f_lane(Mech* m, double Ctot, double* K, double* KR, double* Y, do
 
 # The tables of abi.cu beside those that the headers build.
 TABLES = r"""
-static void tables(Mech& m, const double* eff, const int* row)
+static void tables(Mech& m, const double* eff, const int* row, const int* reac, const signed char* type)
 {
     const int nS = m.M.nS, nR = m.M.nR, nM = m.M.nM;
     for (int r = 0; r < nM; ++r) {
@@ -237,6 +237,13 @@ static void tables(Mech& m, const double* eff, const int* row)
         }
     }
     m.liE = m.li.eff;
+    m.scl.resize(4 * nR + 4);
+    for (int q = 0; q < nR; ++q) {
+        const int j = m.perm[q];
+        int_scale_table(m.arr[q], m.arr[nR + q], m.arr[2 * nR + q], reac + 2 * j, type[j],
+                        q >= nR - nM ? m.effX[q - (nR - nM)] : 0, &m.scl[4 * q]);
+    }
+    m.M.scl = (const uint4*)m.scl.data();
     int_word_bits(nS, m.ptr.data(), m.nu.data(), &m.M.imUp, &m.M.imShort);
 }
 """

@@ -49,7 +49,7 @@ def test_unburnt(lib, wl, radicals):
         cell = T[c], p[c], Y[:, c]
         bound = ULP * (16 + 4 * (abs(m.lnA) + abs(m.beta) * np.log(T[c]) + m.Ea / (synth.R_GAS * T[c])).max())
         ref, mag = f.reference(*cell)
-        out, scale = f.warp(*cell, 0)
+        out, scale = f.warp(*cell, -(c % 2))  # (-1: the scale is estimated first)
         assert (np.abs(out - ref) <= bound * mag).all(), (c, float((np.abs(out - ref) / np.maximum(mag, 1e-300)).max()))
         if m.n_species > 16:
             continue
