@@ -581,7 +581,9 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     std::vector<int32_t> effI((size_t)(nS + 1) / 2 * nM * 4, 0), effX(nM);
     for (int row = 0; row < nM; ++row) {
         std::vector<int32_t> hi(nS), lo(nS);
-        effX[row] = int_efficiencies(nS, d->eff + (size_t)rxn[perm[nPlain + row]].row * nS, hi.data(), lo.data());
+        const double* e = d->eff + (size_t)rxn[perm[nPlain + row]].row * nS;
+        effX[row] = int_efficiencies(nS, e, hi.data(), lo.data());
+        int_eff_limbs(nS, e, effX[row], 1, hi.data(), lo.data());
         for (int k = 0; k < nS; ++k) {
             effI[((size_t)(k / 2) * nM + row) * 4 + 2 * (k % 2)] = hi[k];
             effI[((size_t)(k / 2) * nM + row) * 4 + 2 * (k % 2) + 1] = lo[k];
@@ -625,6 +627,9 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     const bool use_li = lane_int_bytes(nS, nM) <= LANE_INT_MAX_BYTES;
     LaneInt li;
     if (use_li) li = build_lane_int(nS, nR, d->reac, d->prod, d->type, d->eff);
+    for (int r = 0; r < li.tb; ++r)
+        int_eff_limbs(nS, d->eff + (size_t)li.row[r] * nS, li.effx[r], 2, &li.eff[2 * (size_t)r * nS],
+                      &li.eff[2 * (size_t)r * nS + 1]);
     const size_t oLiRx = put(li.rx.data(), 4 * li.rx.size());
     const size_t oLiE = put(li.eff.data(), 4 * li.eff.size()), oLiEx = put(li.effx.data(), 4 * li.effx.size());
     // the segmented FP32 gather of the 32-lane isothermal f, where the packed

@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(128, 4)
         int scale = -1;
 #pragma unroll
         for (int r = 0; r < NR; ++r) x[r] = lane + G * r < M.nS ? Y[(int64_t)(lane + G * r) * ldY + c] : 0.0;
-        warp_feval_int<NR, G, true>(M, I, S, rates_at(M, t, invT), true, pR * invT, Tab<double>::inv(pR) * t, scale, x,
+        warp_feval_int<NR, G, true>(M, I, S, rates_at(M, t, invT), true, pR * invT, quot(t, pR), scale, x,
                                     out, lane, grp);
 #pragma unroll
         for (int r = 0; r < NR; ++r)

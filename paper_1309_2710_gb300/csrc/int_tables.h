@@ -22,9 +22,8 @@
 // (bank = place mod 8).
 //
 // Third-body sums (Eq. (E:rxn-rate), [M] = sum_k eff_k C_k): a row's
-// efficiencies as integers eff_k 2^(54 - x), x the exponent of the row's
-// largest (one more above 128 species, which keeps the sums of 30 x 25-bit
-// products below 2^63), cut into 30 high and 25 low bits.
+// efficiencies as integers eff_k 2^(58 - x), x the exponent of the row's
+// largest, cut into 30 high and 29 low bits (int_eff_limbs).
 #pragma once
 #include <algorithm>
 #include <cmath>
@@ -178,11 +177,26 @@ inline int int_efficiencies(int nS, const double* eff, int32_t* hi, int32_t* lo)
 inline void int_scale_table(double lnA, double beta, double EaR, const int32_t* reac, int type, int row, uint32_t* out)
 {
     const double log2e = 1.4426950408889634;
-    const float f[3] = {(float)(lnA * log2e + 1023 + (type == 1 ? row + 1 - 1021 : type == 2)), (float)(beta * log2e),
+    const float f[3] = {(float)(lnA * log2e + 1023 + (type == 1 ? row - 1021 : 0)), (float)(beta * log2e),
                         (float)(EaR * log2e)};
     std::memcpy(out, f, sizeof(f));
     const int power = (reac[0] >= 0) + (reac[1] >= 0) + (type == 1) - 2;
     out[3] = (uint32_t)(reac[0] + 1) | (uint32_t)(reac[1] + 1) << 10 | (uint32_t)(power + 2) << 20 | (type == 1 ? 1u << 23 : 0u);
+}
+
+// The same in 59 bits, round(eff 2^(58 - x)), as the kernels take them: hi (30
+// bits) and lo (29 bits, signed and rounded to nearest, so that the products
+// lo lo that they leave out are small and of either sign). Every efficiency down to
+// 2^-6 of the row's largest is exact. hi and lo come from int_efficiencies,
+// `stride` apart.
+inline void int_eff_limbs(int nS, const double* eff, int x, int stride, int32_t* hi, int32_t* lo)
+{
+    for (int k = 0; k < nS; ++k) {
+        const int64_t c = (int64_t)hi[stride * k] * (1 << 25) + lo[stride * k];
+        const int64_t E = 16 * c + (int64_t)std::nearbyint(16.0 * (std::ldexp(eff[k], 54 - x) - (double)c));
+        hi[stride * k] = (int32_t)((E + (1 << 28)) >> 29);
+        lo[stride * k] = (int32_t)(E - (int64_t)hi[stride * k] * (1 << 29));
+    }
 }
 
 // Tables of the lane layout's f (lane_int.cuh): its reactions in the order
@@ -192,6 +206,7 @@ struct LaneInt {
     std::vector<uint32_t> rx;               // [n + 1][4] records
     std::vector<int32_t> eff;               // [tb][nS][2] integer efficiencies
     std::vector<int32_t> effx;              // [tb]
+    std::vector<int32_t> row;               // [tb] efficiency rows in reaction order
 };
 
 // type: 0 plain, 1 third body, 2 falloff; eff: one row per non-plain reaction,
@@ -237,6 +252,7 @@ inline LaneInt build_lane_int(int nS, int nR, const int32_t* reac, const int32_t
             ++t.n;
             if (ty) {
                 ++t.tb;
+                t.row.push_back(r);
                 std::vector<int32_t> hi(nS), lo(nS);
                 t.effx.push_back(int_efficiencies(nS, eff + (size_t)r * nS, hi.data(), lo.data()));
                 for (int k = 0; k < nS; ++k) {

@@ -15,10 +15,15 @@
 //    far below the largest rate of the evaluation, so every sum of rates is
 //    exact (four 32-bit adds) but for the words' own last bits; sums that these
 //    bits could matter to are formed again with a lower unit (IM_STEP below);
-//  * a third-body sum multiplies 55-bit integer efficiencies by the
-//    concentrations as 55-bit fractions of the total.
-// Every product, sum and third-body sum is at least as accurate as its FP64
-// form: 2^-57 per product against 2^-53, no rounding in the sums. States
+//  * a third-body sum multiplies 59-bit integer efficiencies by the
+//    concentrations as 59-bit fractions of the total. Sums below 2^-7 to 2^-5 of
+//    the row's largest efficiency times the total are taken in FP64, where the
+//    fractions would be too coarse.
+// A product of two loses up to 2^-58, one of five (a third body, the density) up to
+// 2^-53, and a sum of rates nothing to the order of its terms. Error of a
+// species' rate over the sum of its |terms|, in units of 2^-53, on mixtures of 13,
+// 53 and 111 species with given rate constants (tests/test_int_f_species.py): rms
+// 1.2 to 2.0, and 1.8 to 2.2 for the plain FP64 form of the same rates. States
 // outside the range of the fixed-point forms (not finite, or a concentration
 // below -2^-9 of the total) take a plain FP64 evaluation instead.
 #pragma once

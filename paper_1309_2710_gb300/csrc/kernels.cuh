@@ -462,13 +462,16 @@ __device__ __forceinline__ double Tab<double>::inv(double a)
     return fma(r, fma(-a, r, 1.0), r);
 }
 
-// Pr / (1 + Pr): the reciprocal by two Newton steps and one correction of the
-// quotient (within an ulp; an IEEE division is a third longer).
-__device__ __forceinline__ double falloff_factor(double Pr)
+// a / b in the evaluation of f: the quotient by that reciprocal and one correction.
+// Both are the nearest double except next to a tie (the seed's 2^-19.9 is 2^-79
+// after two steps; none of 20 million random quotients and reciprocals on the CPU,
+// from an FP32 seed, differed from the division); an IEEE division is a third
+// longer.
+__device__ __forceinline__ double quot(double a, double b)
 {
-    const double d = 1.0 + Pr, r = Tab<double>::inv(d), q = Pr * r;
-    const double z = fma(r, fma(-q, d, Pr), q);
-    return isfinite(z) ? z : ddiv(Pr, d);
+    const double r = Tab<double>::inv(b), q = a * r;
+    const double z = fma(r, fma(-q, b, a), q);
+    return isfinite(z) ? z : ddiv(a, b);
 }
 
 struct PowerState {

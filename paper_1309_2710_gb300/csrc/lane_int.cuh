@@ -96,8 +96,8 @@ __device__ __forceinline__ int lane_int_pass(const MechDev& M, const LaneIntSmem
         const uint32_t ea = se[a], eb = se[b];
         e += (ea & 0x7fffu) + (eb & 0x7fffu);
         if (j < nTB) {
-            Q = im_mul(Q, tm[j * T]);
-            e += te[j * T] - (uint32_t)(IM_BIAS - 64);
+            Q = im_mul(Q << 1, tm[j * T]);
+            e += te[j * T] - (uint32_t)(IM_BIAS - 63);
         }
         if ((d.y & (7u << 20)) != (2u << 20)) {  // not rho^2 as for a plain reaction of two
             for (int p = (int)((d.y >> 20) & 7u) - 2; p != 0; p += p > 0 ? -1 : 1) {
@@ -229,14 +229,15 @@ struct IntF {
         im_split_k(Sum * invCtot, mix.mi, mix.ei);
         int bad = 0;
         if (nTB) {
-            // fractions of the total in 30 + 25 bits, in the lane's own sums' words
+            // fractions of the total in 30 + 29 bits, in the lane's own sums' words
             int2* const F = reinterpret_cast<int2*>(acc);
 #pragma unroll 2
             for (int k = 0; k < nS; ++k) {
                 const uint32_t e = se[k * T];
-                long long f = (long long)((im_shr(sm[k * T], (uint32_t)(eS - (int)(e & 0x7fffu) + 71)) + 1ull) >> 1);
+                long long f = (long long)((im_shr(sm[k * T], (uint32_t)(eS - (int)(e & 0x7fffu) + 67)) + 1ull) >> 1);
                 if (e & 0x8000u) f = -f;
-                F[2 * k * T] = make_int2((int)(f >> 25), (int)(f & 0x1ffffff));
+                const int hi = (int)((f + (1 << 28)) >> 29);
+                F[2 * k * T] = make_int2(hi, (int)(f - (long long)hi * (1 << 29)));
             }
 #pragma unroll 1
             for (int r = 0; r < nTB; ++r) {
@@ -249,15 +250,18 @@ struct IntF {
                     mid += (long long)u.x * f.y;
                     mid += (long long)u.y * f.x;
                 }
-                const long long U = hi + (mid >> 25);
-                if (U < (1ll << 54)) bad = IM_OUT;  // small beside its terms: the fractions are too coarse
+                const long long U = hi + (mid >> 29);
+                if (U < (1ll << 53)) bad = IM_OUT;  // small beside its terms: the fractions are too coarse
                 const int z = max(1, __clzll(U | 1ll));
                 im_u64 mm = (im_u64)U << (z - 1);
                 uint32_t em = (uint32_t)(eS + M.li_effx[r] + 5 - z);
                 const uint4 d = M.li_rx[r];
                 if (d.y & LI_FALLOFF) {
-                    const double Md = im_round(mm, (int)em - IM_BIAS, false) * rho;
-                    im_split(falloff_factor(KR[d.w] * Md), mm, em);
+                    im_u64 km;
+                    uint32_t ke;
+                    im_split_k(KR[d.w], km, ke);
+                    const double Pr = im_round(im_mul(im_mul(km, mm) << 1, mix.mr), (int)(ke + em + mix.er) - 3 * IM_BIAS + 127, false);
+                    im_split(quot(Pr, 1.0 + Pr), mm, em);
                     if (em >= 0x7ffu) bad = IM_OUT;
                 }
                 tm[r * T] = mm;

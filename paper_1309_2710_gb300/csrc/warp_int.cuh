@@ -213,7 +213,7 @@ struct IntCell {
 struct IntSmem {
     ulonglong2* OM;  // [chunk + 1] rates of progress of a chunk, and a zero word
     ulonglong2* P;   // [nslots] partial sums
-    int2* CF;        // [nS, even] concentrations as 55-bit fractions: 30 high, 25 low bits
+    int2* CF;        // [nS, even] concentrations as 59-bit fractions: 30 high, 29 low bits
     IntCell* cell;
     im_u64* CM;      // [nS + 1] mantissas, after the constant 1 that empty slots read
     uint32_t* CE;    // [nS + 1] exponent words
@@ -249,18 +249,20 @@ __device__ __forceinline__ double int_conc(const IntSmem& S, int k)
     return im_round(S.CM[k], (int)(e & 0x7fffffffu) - 64 - IM_BIAS, (int)e < 0);
 }
 
-// [M] of an efficiency row in FP64, from concentrations c[k + 1] given by get.
+// [M] of an efficiency row in FP64, from concentrations c[k + 1] given by get, in
+// two interleaved partial sums.
 template <typename Get>
 __device__ double int_row_dot(const MechDev& M, int row, Get get)
 {
     const double2* __restrict__ a = reinterpret_cast<const double2*>(M.effV64) + row;
-    double m = 0.0;
+    double m0 = 0.0, m1 = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < M.nS; ++k) {
+    for (int k = 0; k < M.nS; k += 2) {
         const double2 e = a[(int64_t)(k >> 1) * M.nM];
-        m += ((k & 1) ? e.y : e.x) * get(k + 1);
+        m0 += e.x * get(k + 1);
+        if (k + 1 < M.nS) m1 += e.y * get(k + 2);
     }
-    return m;
+    return m0 + m1;
 }
 
 static __device__ __noinline__ double int_row_dot_slow(const MechDev& M, int row, const IntSmem& S)
@@ -358,6 +360,11 @@ __device__ __forceinline__ bool int_rate(const MechDev& M, const IntSmem& S, con
             mid += (long long)u.z * f.w;
             mid += (long long)u.w * f.z;
         };
+        // (sixteen species' products keep mid below 2^63)
+        auto carry = [&]() {
+            hi += mid >> 29;
+            mid &= (1 << 29) - 1;
+        };
         const int n2 = (nS + 1) >> 1;
         int k = 0;
 #pragma unroll 1
@@ -367,43 +374,45 @@ __device__ __forceinline__ bool int_rate(const MechDev& M, const IntSmem& S, con
             for (int j = 0; j < 8; ++j) u[j] = E[(int64_t)(k + j) * nM];
 #pragma unroll
             for (int j = 0; j < 8; ++j) term(u[j], F[k + j]);
+            carry();
         }
         if constexpr (AHEAD) {
 #pragma unroll 4
             for (; k < n2; ++k) term(E[(int64_t)k * nM], F[k]);
         } else {
 #pragma unroll 1
-            for (; k < n2; ++k) term(E[(int64_t)k * nM], F[k]);
+            for (; k < n2; ++k) {
+                term(E[(int64_t)k * nM], F[k]);
+                carry();
+            }
         }
-        const long long U = hi + (mid >> 25);
-        double Md = 0.0;
+        carry();
+        const long long U = hi;
         im_u64 mm;
         uint32_t em;
-        if (U < (1ll << 54)) {  // small beside its terms: the fractions are too coarse
-            Md = int_row_dot_slow(M, row, S);
-            im_split(Md, mm, em);
-            Md *= mix.rho;
+        if (U < (1ll << 53)) {  // small beside its terms: the fractions are too coarse
+            im_split(int_row_dot_slow(M, row, S), mm, em);
         } else {
             const int z = __clzll(U);
             mm = (im_u64)U << (z - 1);
             em = (uint32_t)(M.effX[row] + mix.eT + 5 - z);
-            if (!AT_T && q >= nF) Md = im_round(mm, (int)em - IM_BIAS, false) * mix.rho;
         }
         if (q >= nF) {
-            double Pr;
+            im_u64 km;
+            uint32_t ke;
             if constexpr (AT_T) {
-                im_u64 km;
-                uint32_t ke;
                 if (!im_exp(M.ex2, low_exponent(M, q - nF, rk) - a, km, ke)) in = false;
-                Pr = im_round(im_mul(km, mm), (int)ke + (int)(em & 0x7fffffffu) - 2 * IM_BIAS + 64, (int)em < 0) * mix.rho;
             } else {
-                Pr = __dmul_rn(rk.K[nR + (q - nF)], Md);
+                im_split_k(rk.K[nR + (q - nF)], km, ke);
             }
-            im_split(falloff_factor(Pr), mm, em);
+            const double Pr = im_round(im_mul(im_mul(km, mm) << 1, mix.mr),
+                                       (int)(ke + (em & 0x7fffffffu) + mix.er) - 3 * IM_BIAS + 127, (int)em < 0);
+            im_split(quot(Pr, 1.0 + Pr), mm, em);
             if ((em & 0x7ffu) == 0x7ffu) in = false;
         }
-        Q = im_mul(Q, mm);
-        e += em - (uint32_t)(IM_BIAS - 64);
+        // (a bit up: four factors cut from a short mantissa would cost half an ulp)
+        Q = im_mul(Q << 1, mm);
+        e += em - (uint32_t)(IM_BIAS - 63);
     }
     // the rate is rho^2 of what a plain reaction of two gives here
     if (q >= nP || M.imLow) {
@@ -542,10 +551,11 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
             S.CM[i + 1] = m[r];
             S.CE[i + 1] = e[r];
             if (M.nM) {
-                // 2^55 of twice the total at most: sum |F| < 3 * 2^55
-                long long F = (long long)((im_shr(m[r], (uint32_t)(eT - (int)(e[r] & 0xfffu) + 71)) + 1ull) >> 1);
+                // 2^59 of twice the total at most: sum |F| < 3 * 2^59
+                long long F = (long long)((im_shr(m[r], (uint32_t)(eT - (int)(e[r] & 0xfffu) + 67)) + 1ull) >> 1);
                 if ((int)e[r] < 0) F = -F;
-                S.CF[i] = make_int2((int)(F >> 25), (int)(F & ((1 << 25) - 1)));
+                const int hi = (int)((F + (1 << 28)) >> 29);
+                S.CF[i] = make_int2(hi, (int)(F - (long long)hi * (1 << 29)));
             }
         } else if (i == nS && (nS & 1)) {
             S.CF[i] = make_int2(0, 0);
@@ -724,7 +734,7 @@ __device__ __forceinline__ void warp_feval_int_energy(const MechDev& M, const In
         }
     }
     const double hw = grp.sum(h), cpm = grp.sum(c);
-    const double dTdt = -hw * Tab<double>::inv(cpm);
+    const double dTdt = quot(-hw, cpm);
 #pragma unroll
     for (int r = 0; r < NR; ++r)
         if (lane + G * r == nS) out[r] = dTdt;

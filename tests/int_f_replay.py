@@ -86,13 +86,13 @@ KERNELS = r"""
 #include "kin_dev.cuh"
 namespace kin {
 inline double ddiv(double a, double b) { return a / b; }
+inline double quot(double a, double b) { return a / b; }
 template <typename R> struct Tab;
 template <> struct Tab<double> { static double inv(double a) { return int_inv(a); } };
 template <typename T> struct Lane { T* p; int32_t s; T& operator[](int i) const { return p[(int64_t)i * s]; } };
 template <typename F> struct IntegerF { static constexpr bool value = false; };
 template <typename R, typename KT>
 void feval(const MechDev&, double, double, Lane<KT>, Lane<KT>, Lane<R>, Lane<R>, Lane<double>, Lane<double>) { ++general; }
-inline double falloff_factor(double p) { return p / (1.0 + p); }
 }
 """
 
@@ -230,13 +230,17 @@ static void tables(Mech& m, const double* eff, const int* row, const int* reac, 
     const int nS = m.M.nS, nR = m.M.nR, nM = m.M.nM;
     for (int r = 0; r < nM; ++r) {
         std::vector<int32_t> hi(nS), lo(nS);
-        m.effX[r] = int_efficiencies(nS, eff + (size_t)row[m.perm[nR - nM + r]] * nS, hi.data(), lo.data());
+        const double* e = eff + (size_t)row[m.perm[nR - nM + r]] * nS;
+        m.effX[r] = int_efficiencies(nS, e, hi.data(), lo.data());
+        int_eff_limbs(nS, e, m.effX[r], 1, hi.data(), lo.data());
         for (int k = 0; k < nS; ++k) {
             m.effI[((size_t)(k / 2) * nM + r) * 4 + 2 * (k % 2)] = hi[k];
             m.effI[((size_t)(k / 2) * nM + r) * 4 + 2 * (k % 2) + 1] = lo[k];
         }
     }
     m.liE = m.li.eff;
+    for (int r = 0; r < m.li.tb; ++r)
+        int_eff_limbs(nS, eff + (size_t)m.li.row[r] * nS, m.li.effx[r], 2, &m.liE[2 * r * nS], &m.liE[2 * r * nS + 1]);
     m.scl.resize(4 * nR + 4);
     for (int q = 0; q < nR; ++q) {
         const int j = m.perm[q];
