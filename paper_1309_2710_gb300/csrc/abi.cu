@@ -138,8 +138,9 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
         if (threads % 32 != 0 || threads > 256) return fail(KIN_EINVAL, "block_threads must be a multiple of 32 and <= 256");
         lanes = cell_lanes(o, m->nS + o->energy, threads, cells, nsm);
         // the layout's limit on a mechanism: C and Omega of a block's cells in
-        // shared memory (the FP64 f's own words need no more)
-        const size_t sm = (size_t)((m->nS + m->nR + 3) & ~3) * 8 * (threads / std::min(lanes, 32));
+        // shared memory, at half a warp or a warp per cell (the FP64 f's own words
+        // need no more: a group's chunk of a large mechanism takes 2 to 5 KB)
+        const size_t sm = (size_t)((m->nS + m->nR + 3) & ~3) * 8 * (threads / (o->method == KIN_RKCK && lanes < 32 ? 16 : 32));
         if (sm > (size_t)maxsm)
             return fail(KIN_EUNSUPPORTED, "warp layout needs %zu bytes of shared memory per block (max %d)", sm, maxsm);
         const int nV = m->nS + o->energy;
