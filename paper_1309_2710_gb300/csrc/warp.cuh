@@ -1241,7 +1241,7 @@ __global__ void __launch_bounds__(256, WarpBounds<NR, OCC, EN>::min_blocks) warp
 // (cell-major in the workspace, unless they follow T with the energy
 // equation) and integrates it with straight-line control flow; the decisions
 // are those of the lane-per-cell kernel. Every collective of a group names
-// only the group's lanes, so the two halves of a warp may diverge.
+// only the group's lanes.
 template <typename R, int NR, bool EN, int G>
 struct WarpRKCK {
     const Launch& L;
@@ -1289,159 +1289,235 @@ struct WarpRKCK {
         nfe++;
     }
 
-    // Integrate over [0, dt] from y with k[0] = f(y); returns the cell status.
-    __device__ int run(double dt, int& nacc, int& nrej)
+    // Integration state of a cell.
+    struct Cell {
+        double dt, t, h, hh;
+        int attempts, nacc, nrej;
+        bool last, due;  // the flow step's last step; f(y) comes next
+
+        __device__ void start(double dt_)
+        {
+            dt = h = dt_;  // first trial step: the whole flow step
+            t = 0.0;
+            attempts = nacc = nrej = 0;
+            due = true;
+        }
+    };
+
+    __device__ __forceinline__ bool finite(const double (&v)[NR]) const
     {
-        double t = 0.0, h = dt;  // first trial step: the whole flow step
-        int attempts = 0;
-        for (;;) {
-            if (attempts >= L.max_steps) return KIN_CELL_MAXSTEPS;
-            double hh = h;
-            bool last = false;
-            if (hh >= dt - t) {
-                hh = dt - t;
-                last = true;
+        bool fin = true;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) fin &= isfinite(v[r]);
+        return __all_sync(mask, fin);
+    }
+
+    // The next step's size.
+    __device__ __forceinline__ void begin_step(Cell& U)
+    {
+        U.hh = U.h;
+        U.last = false;
+        if (U.hh >= U.dt - U.t) {
+            U.hh = U.dt - U.t;
+            U.last = true;
+        }
+    }
+
+    // Stage point y + hh sum_l b_{st,l} k_l in x (stage indices are resolved
+    // with unrolled selects, so k stays in registers).
+    __device__ __forceinline__ void stage_point(int st, double hh)
+    {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            double acc = 0.0;
+#pragma unroll
+            for (int l = 0; l < 5; ++l)
+                if (l < st) acc += CK_B[st][l] * k[l][r];
+            x[r] = y[r] + hh * acc;
+        }
+    }
+
+    // Error test and step control after the six evaluations. Returns a final
+    // status, or -1.
+    __device__ __forceinline__ int end_step(Cell& U)
+    {
+        const double hh = U.hh;
+        double errmax = 0.0;
+        bool blown = false;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            double s5 = 0.0, e = 0.0;
+#pragma unroll
+            for (int l = 0; l < 6; ++l) {
+                s5 += CK_C[l] * k[l][r];
+                e += CK_E[l] * k[l][r];
             }
-            for (int st = 1; st < 6; ++st) {  // stage points y + hh sum_l b_{st,l} k_l
-                // (stage indices are resolved with unrolled selects, so k stays
-                // in registers)
+            x[r] = y[r] + hh * s5;
+            if (valid(r)) {
+                const double tol = rtol * (fabs(y[r]) + fabs(hh * k[0][r])) + atol;
+                const double q = fabs(hh * e) * rcp_newton(tol);
+                blown |= isnan(q);
+                if (q > errmax) errmax = q;
+            }
+        }
+        // group maximum; a NaN component makes the estimate non-finite
+        errmax = group_max<G>(errmax, mask);
+        if (__any_sync(mask, blown)) errmax = __longlong_as_double(0x7ff8000000000000ll);
+        U.attempts++;
+        if (errmax <= 1.0) {
+            U.nacc++;
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    double acc = 0.0;
+            for (int r = 0; r < NR; ++r) y[r] = x[r];
+            if (U.last) return KIN_CELL_OK;
+            U.t += hh;
+            const double hn = errmax == 0.0 ? 5.0 * hh : 0.9 * hh * rpow5_newton(errmax);
+            U.h = fmin(hn, 5.0 * hh);
+            U.due = true;
+        } else {
+            U.nrej++;
+            const double hn = isfinite(errmax) ? 0.9 * hh * rpow4_newton(errmax) : 0.1 * hh;
+            U.h = fmax(hn, 0.1 * hh);
+            if (U.h < 1e-20 * U.dt) return KIN_CELL_HMIN;
+        }
+        return -1;
+    }
+};
+
+// Take cell g into W: its constants and state.
+template <typename R, int NR, bool EN, int G>
+__device__ __forceinline__ void warp_rkck_load(WarpRKCK<R, NR, EN, G>& W, const InstDev& I, int64_t g, int64_t c)
+{
+    const Launch& L = W.L;
+    const MechDev& M = W.M;
+    const int lane = W.lane, nK = M.nR + M.nFO, nS = M.nS;
+    const double T = I.T[c], p = I.p[c];
+    W.Ctot = ddiv(p * 1e-6, EN && sizeof(R) == 8 ? R_GAS : R_GAS * T);
+    W.invCtot = ddiv(1.0, W.Ctot);
+    W.CtotR = (R)W.Ctot;
+    W.invCtotR = (R)W.invCtot;
+    W.atol = I.atol;
+    W.rtol = I.rtol;
+    W.p = p;
+    W.nfe = 0;
+    if constexpr (!EN) {
+        // formed straight into the staged copy when there is one (the
+        // previous cell's last f ended in a sync of the group)
+        R* kc = W.Ks ? W.Ks : reinterpret_cast<R*>(L.cell_k) + g * nK;
+        const double lnT = log(T), invT = ddiv(1.0, T);
+        bool kfin = true;
+        for (int qq = lane; qq < M.nR; qq += G) {
+            const int j = M.rxn_perm[qq];
+            const double a = M.lnA[j] + M.beta[j] * lnT - M.EaR[j] * invT;
+            const R k = Tab<R>::ex(a);
+            kc[qq] = k;
+            if (sizeof(R) == 8) kfin &= im_finite_k(k);
+            const int fo = M.rxnp[qq].fo;
+            if (fo >= 0) {
+                const double a0 = M.lnA0[j] + M.beta0[j] * lnT - M.Ea0R[j] * invT;
+                const R k0 = Tab<R>::ex(a0 - a);
+                kc[M.nR + fo] = k0;
+                if (sizeof(R) == 8) kfin &= im_finite_k(k0);
+            }
+        }
+        __syncwarp(W.mask);
+        W.Kc = kc;
+        if (sizeof(R) == 8) W.kfin = __all_sync(W.mask, kfin);
+    }
+    W.scale = EN ? -1 : 0;
 #pragma unroll
-                    for (int l = 0; l < 5; ++l)
-                        if (l < st) acc += CK_B[st][l] * k[l][r];
-                    x[r] = y[r] + hh * acc;
-                }
-                f(x, kx);
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        W.y[r] = i < nS ? I.Y[(int64_t)i * I.ldY + c] : (i == nS && EN ? T : 0.0);
+    }
+}
+
+// The cell's result: its state unless f(y) at the start was not finite, the
+// status and the statistics.
+template <typename R, int NR, bool EN, int G>
+__device__ __forceinline__ void warp_rkck_store(const WarpRKCK<R, NR, EN, G>& W, const InstDev& I, int64_t c, bool state,
+                                                int code, int nacc, int nrej)
+{
+    const int lane = W.lane, nS = W.M.nS;
+    if (state) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int i = lane + G * r;
+            if (i < nS) I.Y[(int64_t)i * I.ldY + c] = W.y[r];
+            else if (i == nS && EN) I.T[c] = W.y[r];
+        }
+    }
+    if (lane == 0) {
+        if (I.status) I.status[c] = (uint8_t)code;
+        if (I.stats) {
+            int32_t* st = I.stats + KIN_NSTATS * c;
+            st[0] = W.nfe;
+            st[1] = nacc;
+            st[2] = nrej;
+            st[3] = 0;
+            st[4] = 0;
+        }
+    }
+}
+
+// Two half-warp groups stay together step by step and evaluation by evaluation
+// (a group that has no evaluation due, or no cell, waits): where they only met by
+// the compiler's choice, one build ran the 16-species kernel at a third of its
+// speed.
+template <typename R, int NR, bool EN, int G>
+__global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const __grid_constant__ Launch L)
+{
+    using Warp = WarpRKCK<R, NR, EN, G>;
+    Warp W(L);
+    typename Warp::Cell U;
+    bool have = false, more = true;
+    int ii = 0;
+    int64_t c = 0;
+    for (;;) {
+        if (!have && more) {
+            unsigned long long q = 0;
+            if (W.lane == 0) q = atomicAdd(L.queue, 1ull);
+            q = __shfl_sync(W.mask, q, 0, G);
+            more = q < (unsigned long long)L.total;
+            if (more) {
+                ii = find_inst(L, (int64_t)q);
+                c = (int64_t)q - L.start[ii];
+                warp_rkck_load(W, L.inst[ii], (int64_t)q, c);
+                U.start(L.inst[ii].dt);
+                have = true;
+            }
+        }
+        if (__all_sync(0xffffffffu, !have)) return;
+        if (have && U.due) {
+            W.f(W.y, W.k[0]);
+            U.due = false;
+            if (!W.finite(W.k[0])) {
+                warp_rkck_store(W, L.inst[ii], c, U.nacc > 0, KIN_CELL_NONFINITE, U.nacc, U.nrej);
+                have = false;
+            } else if (U.attempts >= L.max_steps) {
+                warp_rkck_store(W, L.inst[ii], c, true, KIN_CELL_MAXSTEPS, U.nacc, U.nrej);
+                have = false;
+            }
+        }
+        __syncwarp();
+        if (have) W.begin_step(U);
+        for (int st = 1; st < 6; ++st) {
+            if (have) {
+                W.stage_point(st, U.hh);
+                W.f(W.x, W.kx);
 #pragma unroll
                 for (int l = 1; l < 6; ++l)
                     if (l == st)
 #pragma unroll
-                        for (int r = 0; r < NR; ++r) k[l][r] = kx[r];
+                        for (int r = 0; r < NR; ++r) W.k[l][r] = W.kx[r];
             }
-            double errmax = 0.0;
-            bool blown = false;
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                double s5 = 0.0, e = 0.0;
-#pragma unroll
-                for (int l = 0; l < 6; ++l) {
-                    s5 += CK_C[l] * k[l][r];
-                    e += CK_E[l] * k[l][r];
-                }
-                x[r] = y[r] + hh * s5;
-                if (valid(r)) {
-                    const double tol = rtol * (fabs(y[r]) + fabs(hh * k[0][r])) + atol;
-                    const double q = fabs(hh * e) * rcp_newton(tol);
-                    blown |= isnan(q);
-                    if (q > errmax) errmax = q;
-                }
-            }
-            // group maximum; a NaN component makes the estimate non-finite
-            errmax = group_max<G>(errmax, mask);
-            if (__any_sync(mask, blown)) errmax = __longlong_as_double(0x7ff8000000000000ll);
-            attempts++;
-            if (errmax <= 1.0) {
-                nacc++;
-#pragma unroll
-                for (int r = 0; r < NR; ++r) y[r] = x[r];
-                if (last) return KIN_CELL_OK;
-                t += hh;
-                const double hn = errmax == 0.0 ? 5.0 * hh : 0.9 * hh * rpow5_newton(errmax);
-                h = fmin(hn, 5.0 * hh);
-                f(y, k[0]);
-                bool fin = true;
-#pragma unroll
-                for (int r = 0; r < NR; ++r) fin &= isfinite(k[0][r]);
-                if (!__all_sync(mask, fin)) return KIN_CELL_NONFINITE;
-            } else {
-                nrej++;
-                const double hn = isfinite(errmax) ? 0.9 * hh * rpow4_newton(errmax) : 0.1 * hh;
-                h = fmax(hn, 0.1 * hh);
-                if (h < 1e-20 * dt) return KIN_CELL_HMIN;
-            }
+            __syncwarp();
         }
-    }
-};
-
-template <typename R, int NR, bool EN, int G>
-__global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const __grid_constant__ Launch L)
-{
-    WarpRKCK<R, NR, EN, G> W(L);
-    const MechDev& M = L.M;
-    const int lane = W.lane, nK = M.nR + M.nFO, nS = M.nS;
-    for (;;) {
-        unsigned long long q = 0;
-        if (lane == 0) q = atomicAdd(L.queue, 1ull);
-        q = __shfl_sync(W.mask, q, 0, G);
-        if (q >= (unsigned long long)L.total) return;
-        const int64_t g = (int64_t)q;
-        const int ii = find_inst(L, g);
-        const InstDev& I = L.inst[ii];
-        const int64_t c = g - L.start[ii];
-        const double T = I.T[c], p = I.p[c];
-        W.Ctot = ddiv(p * 1e-6, EN && sizeof(R) == 8 ? R_GAS : R_GAS * T);
-        W.invCtot = ddiv(1.0, W.Ctot);
-        W.CtotR = (R)W.Ctot;
-        W.invCtotR = (R)W.invCtot;
-        W.atol = I.atol;
-        W.rtol = I.rtol;
-        W.p = p;
-        W.nfe = 0;
-        if constexpr (!EN) {
-            // formed straight into the staged copy when there is one (the
-            // previous cell's last f ended in a sync of the group)
-            R* kc = W.Ks ? W.Ks : reinterpret_cast<R*>(L.cell_k) + g * nK;
-            const double lnT = log(T), invT = ddiv(1.0, T);
-            bool kfin = true;
-            for (int qq = lane; qq < M.nR; qq += G) {
-                const int j = M.rxn_perm[qq];
-                const double a = M.lnA[j] + M.beta[j] * lnT - M.EaR[j] * invT;
-                const R k = Tab<R>::ex(a);
-                kc[qq] = k;
-                if (sizeof(R) == 8) kfin &= im_finite_k(k);
-                const int fo = M.rxnp[qq].fo;
-                if (fo >= 0) {
-                    const double a0 = M.lnA0[j] + M.beta0[j] * lnT - M.Ea0R[j] * invT;
-                    const R k0 = Tab<R>::ex(a0 - a);
-                    kc[M.nR + fo] = k0;
-                    if (sizeof(R) == 8) kfin &= im_finite_k(k0);
-                }
-            }
-            __syncwarp(W.mask);
-            W.Kc = kc;
-            if (sizeof(R) == 8) W.kfin = __all_sync(W.mask, kfin);
-        }
-        W.scale = EN ? -1 : 0;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const int i = lane + G * r;
-            W.y[r] = i < nS ? I.Y[(int64_t)i * I.ldY + c] : (i == nS && EN ? T : 0.0);
-        }
-        W.f(W.y, W.k[0]);
-        bool fin = true;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) fin &= isfinite(W.k[0][r]);
-        int nacc = 0, nrej = 0, code = KIN_CELL_NONFINITE;
-        if (__all_sync(W.mask, fin)) {
-            code = W.run(I.dt, nacc, nrej);
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int i = lane + G * r;
-                if (i < nS) I.Y[(int64_t)i * I.ldY + c] = W.y[r];
-                else if (i == nS && EN) I.T[c] = W.y[r];
-            }
-        }
-        if (lane == 0) {
-            if (I.status) I.status[c] = (uint8_t)code;
-            if (I.stats) {
-                int32_t* st = I.stats + KIN_NSTATS * c;
-                st[0] = W.nfe;
-                st[1] = nacc;
-                st[2] = nrej;
-                st[3] = 0;
-                st[4] = 0;
+        if (have) {
+            int code = W.end_step(U);
+            if (code < 0 && !U.due && U.attempts >= L.max_steps) code = KIN_CELL_MAXSTEPS;
+            if (code >= 0) {
+                warp_rkck_store(W, L.inst[ii], c, true, code, U.nacc, U.nrej);
+                have = false;
             }
         }
     }

@@ -257,16 +257,18 @@ __device__ double int_row_dot(const MechDev& M, int row, Get get)
     const double2* __restrict__ a = reinterpret_cast<const double2*>(M.effV64) + row;
     double m0 = 0.0, m1 = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < M.nS; k += 2) {
+    for (int k = 0; k < M.nS; ++k) {
         const double2 e = a[(int64_t)(k >> 1) * M.nM];
-        m0 += e.x * get(k + 1);
-        if (k + 1 < M.nS) m1 += e.y * get(k + 2);
+        const double m = m1 + ((k & 1) ? e.y : e.x) * get(k + 1);
+        m1 = m0;
+        m0 = m;
     }
     return m0 + m1;
 }
 
-static __device__ __noinline__ double int_row_dot_slow(const MechDev& M, int row, const IntSmem& S)
+static __device__ __noinline__ double int_row_dot_slow(const MechDev& M, int row, int2* CF)
 {
+    const IntSmem S(M, CF);
     return int_row_dot(M, row, [&](int k) { return int_conc(S, k); });
 }
 
@@ -391,7 +393,7 @@ __device__ __forceinline__ bool int_rate(const MechDev& M, const IntSmem& S, con
         im_u64 mm;
         uint32_t em;
         if (U < (1ll << 53)) {  // small beside its terms: the fractions are too coarse
-            im_split(int_row_dot_slow(M, row, S), mm, em);
+            im_split(int_row_dot_slow(M, row, S.CF), mm, em);
         } else {
             const int z = __clzll(U);
             mm = (im_u64)U << (z - 1);
