@@ -493,6 +493,19 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     const size_t oPerm = put(perm.data(), 4 * nR), oRxp = put(rxnp.data(), sizeof(Rxn) * nR);
     const size_t oRxw = put(rxw.data(), 4 * nR);
     const size_t oCrxp = put(crxp.data(), 4 * nnz);
+    // the rows once more in order of position
+    std::vector<int> crxq(nnz), byPos;
+    std::vector<double> cnuq(nnz);
+    for (int i = 0; i < nS; ++i) {
+        byPos.clear();
+        for (int e2 = ptr[i]; e2 < ptr[i + 1]; ++e2) byPos.push_back(e2);
+        std::sort(byPos.begin(), byPos.end(), [&](int a, int b) { return crxp[a] < crxp[b]; });
+        for (size_t k = 0; k < byPos.size(); ++k) {
+            crxq[ptr[i] + k] = crxp[byPos[k]];
+            cnuq[ptr[i] + k] = cnu[byPos[k]];
+        }
+    }
+    const size_t oCrxq = put(crxq.data(), 4 * nnz), oCnuq = put(cnuq.data(), 8 * nnz);
     const size_t oEffV64 = put(effV64.data(), 8 * effV64.size()), oEffV32 = put(effV32.data(), 4 * effV32.size());
     const size_t oPtr = put(ptr.data(), 4 * (nS + 1)), oCrx = put(crx.data(), 4 * nnz);
     const size_t oNu = put(cnu.data(), 8 * nnz), oNu32 = put(nu32.data(), 4 * nnz);
@@ -683,6 +696,8 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.rxn_perm = (const int*)(b + oPerm);
     M.rxnp = (const Rxn*)(b + oRxp);
     M.csrp_rxn = (const int*)(b + oCrxp);
+    M.csrq_rxn = (const int*)(b + oCrxq);
+    M.csrq_nu = (const double*)(b + oCnuq);
     M.ell32 = (const CsrW32*)(b + oEll32);
     M.ell64 = (const CsrW64*)(b + oEll64);
     for (int r = 0; r < ELL_SLOTS; ++r) M.ell_base[r] = ell_base[r];

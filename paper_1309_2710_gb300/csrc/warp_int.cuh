@@ -282,51 +282,87 @@ __device__ __forceinline__ double low_exponent(const MechDev& M, int fo, const R
     return fma(-M.arr0[2 * M.nFO + fo], k.invT, fma(M.arr0[M.nFO + fo], k.lnT, M.arr0[fo]));
 }
 
-// sum_j nu_ij Omega_j of species i in plain FP64, one term after another, from
-// the concentrations c[k + 1] in shared memory (c[0] = 1): for states outside
-// the integer forms' range. Such states are trial points that blew up, so
-// this code is small rather than fast.
-static __device__ __noinline__ double int_general_sum(const MechDev& M, const RateSource& k, const double* c, int i)
+// A state outside the integer forms' range (a trial point that blew up, as a Cash-Karp
+// step far beyond the stability limit makes them) takes plain FP64, chunk by chunk:
+// the lanes' rates of progress from the concentrations c[k + 1] (c[0] = 1), then
+// each species' sum over its row, whose entries are in order of position, so that
+// the bits depend neither on the lanes nor on the chunks. Out of line; about the
+// time of the plain FP64 f that the integer one replaced (with every row forming
+// its own rates instead, 111 species / 1566 reactions, 500 cells in RKCK took
+// 43.8 ms instead of 12.7; 23.2 in plain FP64 throughout).
+template <bool AT_T>
+static __device__ __noinline__ void int_general_rates(const MechDev& M, int2* CF, double* om, int q0, int q1, int lane, int lanes)
 {
+    const IntSmem S(M, CF);
+    const RateSource k = S.cell->rk;
+    const double* c = reinterpret_cast<const double*>(S.CM);
     const int nP = M.nR - M.nM, nF = M.nR - M.nFO;
-    double w = 0.0;
 #pragma unroll 1
-    for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
-        const int q = M.csrp_rxn[e];
-        const uint32_t r = M.rxw[q];
-        const double a = k.K ? 0.0 : rate_exponent(M, q, k);
-        double v = (k.K ? k.K[q] : exp(a)) * c[r & 0xffffu] * c[r >> 16];
+    for (int q = q0 + lane; q < q1; q += lanes) {
+        const uint32_t w = M.rxw[q];
+        const double a = AT_T ? rate_exponent(M, q, k) : 0.0;
+        double v = (AT_T ? exp(a) : k.K[q]) * c[w & 0xffffu] * c[w >> 16];
         if (q >= nP) {
-            const double Mc = int_row_dot(M, q - nP, [&](int k) { return c[k]; });
+            const double Mc = int_row_dot(M, q - nP, [&](int i) { return c[i]; });
             if (q < nF) {
                 v *= Mc;
             } else {
-                const double Pr = (k.K ? k.K[M.nR + (q - nF)] : exp(low_exponent(M, q - nF, k) - a)) * Mc;
+                const double Pr = (AT_T ? exp(low_exponent(M, q - nF, k) - a) : k.K[M.nR + (q - nF)]) * Mc;
                 v *= ddiv(Pr, 1.0 + Pr);
             }
         }
-        w += M.csr_nu[e] * v;
+        om[q - q0] = v;
     }
-    return w;
+}
+
+// w and the rest of species i's row from entry e on, up to position q1.
+struct IntRow {
+    double w;
+    int e;
+};
+static __device__ __noinline__ IntRow int_general_row(const MechDev& M, const double* om, int i, int q0, int q1, IntRow a)
+{
+    const int end = M.csr_ptr[i + 1];
+#pragma unroll 1
+    for (; a.e < end; ++a.e) {
+        const int q = M.csrq_rxn[a.e];
+        if (q >= q1) break;
+        a.w += M.csrq_nu[a.e] * om[q - q0];
+    }
+    return a;
 }
 
 // f of such a state, from its c_k / rho (the group's lanes together).
-template <int NR, int G>
-__device__ __forceinline__ void int_general(const MechDev& M, const IntSmem& S, const RateSource& k, const double (&c)[NR],
+template <int NR, int G, bool AT_T>
+__device__ __forceinline__ void int_general(const MechDev& M, const IntDev& I, const IntSmem& S, const double (&c)[NR],
                                             double rho, double invrho, double (&out)[NR], int lane, const Group<G>& grp)
 {
     double* cs = reinterpret_cast<double*>(S.CM);
+    double* om = reinterpret_cast<double*>(S.OM);
     if (lane == 0) cs[0] = 1.0;
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-        if (lane + G * r < M.nS) cs[lane + G * r + 1] = c[r] * rho;
-    grp.sync();
+    IntRow row[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         const int i = lane + G * r;
-        out[r] = i < M.nS ? __dmul_rn(int_general_sum(M, k, cs, i), M.W[i] * invrho) : 0.0;
+        row[r] = IntRow{0.0, i < M.nS ? M.csr_ptr[i] : 0};
+        if (i < M.nS) cs[i + 1] = c[r] * rho;
     }
     grp.sync();
+#pragma unroll 1
+    for (int q0 = 0; q0 < M.nR; q0 += I.chunk) {
+        const int q1 = min(M.nR, q0 + I.chunk);
+        int_general_rates<AT_T>(M, S.CF, om, q0, q1, lane, G);
+        grp.sync();
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            if (lane + G * r < M.nS) row[r] = int_general_row(M, om, lane + G * r, q0, q1, row[r]);
+        grp.sync();
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        out[r] = i < M.nS ? __dmul_rn(row[r].w, M.W[i] * invrho) : 0.0;
+    }
 }
 
 // The rate of progress of the reaction at position q (over a common power of rho) as
@@ -564,7 +600,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         }
     }
     if (grp.sync_any(!in)) {
-        int_general<NR, G>(M, S, rk, c, rho, invCtot * s, out, lane, grp);
+        int_general<NR, G, AT_T>(M, I, S, c, rho, invCtot * s, out, lane, grp);
         return;
     }
     if constexpr (AT_T) {
@@ -687,7 +723,7 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
         }
         emax = grp.imax(emax);
         if (emax >= IM_OUT) {  // a falloff factor that is not finite
-            int_general<NR, G>(M, S, rk, c, rho, invCtot * s, out, lane, grp);
+            int_general<NR, G, AT_T>(M, I, S, c, rho, invCtot * s, out, lane, grp);
             return;
         }
         scale = emax;

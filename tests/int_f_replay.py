@@ -108,9 +108,9 @@ struct Mech {
     IntDev I{};
     IntGather g;
     LaneInt li;
-    std::vector<double> W, invW, arr, arr0, effV64, nu;
+    std::vector<double> W, invW, arr, arr0, effV64, nu, nuq;
     std::vector<uint32_t> rxw, scl;
-    std::vector<int> perm, ptr, pos;
+    std::vector<int> perm, ptr, pos, posq;
     std::vector<int32_t> effI, effX, imWe, liE;
     std::vector<uint64_t> imW, ex2, lnc;
 };
@@ -152,6 +152,14 @@ extern "C" void* mech_new(int nS, int nR, const double* W, const double* lnA, co
         m->ptr.push_back((int)m->pos.size());
         m->invW.push_back(1.0 / W[i]);
     }
+    for (int i = 0; i < nS; ++i) {
+        std::vector<std::pair<int, double>> row;
+        for (int k = m->ptr[i]; k < m->ptr[i + 1]; ++k) row.push_back({m->pos[k], m->nu[k]});
+        std::sort(row.begin(), row.end());
+        for (auto& e : row) m->posq.push_back(e.first), m->nuq.push_back(e.second);
+    }
+    m->M.csrq_rxn = m->posq.data();
+    m->M.csrq_nu = m->nuq.data();
     const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, 256));
     m->g = build_int_gather(nS, nR, m->ptr.data(), m->pos.data(), m->nu.data(), chunk, LANES);
     m->I = IntDev{m->g.nchunk, chunk, m->g.nslots, m->g.step0.data(), m->g.ent.data(), m->g.slot0.data(), m->g.part.data()};

@@ -117,3 +117,25 @@ def test_third_body_error(lib, nS, n, top, rtype):
     # two rms values of some 3,000 samples each: 5 % between them by chance (3 sigma)
     for k, v in rms.items():
         assert v <= 1.1 * rms["plain"], {k: v / ULP for k, v in rms.items()}
+
+
+@pytest.mark.parametrize("wl", ["h2_9sp_rkck", "h2co_13sp_rkc", "ch4_53sp_rkc_mixed"])
+def test_plain_path(lib, wl):
+    """States outside the integer forms' range (a species at -0.05 to -300 of the
+    total, as in a step that blew up): plain FP64, whose sums of up to 64 terms and
+    species add their roundings to the bound."""
+    m = synth.workload_mechanism(wl)
+    f = int_f_replay.Mech(lib, m)
+    T, p, Y = unburnt(wl, m, 8, (-6, -2))
+    for c in range(8):
+        Y[c % m.n_species, c] = -10.0 ** (c / 2.0 - 1.3) * Y[:, c].sum()
+        if c % 2:
+            Y[(c + 3) % m.n_species, c] = 1.5 * abs(Y[:, c]).sum()
+        cell = T[c], p[c], Y[:, c] / Y[:, c].sum()
+        bound = ULP * (16 + 64 + m.n_species + 4 * (abs(m.lnA) + abs(m.beta) * np.log(T[c]) + m.Ea / (synth.R_GAS * T[c])).max())
+        ref, _ = f.reference(*cell)
+        _, mag = f.reference(cell[0], cell[1], abs(cell[2]))
+        # (the terms' size at these concentrations; the mixture sum cancels)
+        w = abs(cell[2] / m.W).sum() / abs((cell[2] / m.W).sum())
+        out, _ = f.warp(*cell, 0)
+        assert (np.abs(out - ref) <= bound * w ** 4 * mag).all(), c
