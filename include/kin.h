@@ -94,8 +94,10 @@ extern "C" {
                              memory. staging is ignored; for RKC, occupancy selects the register budget
                              (KIN_OCC_HIGH: for up to 64 state components 48
                              registers and 40 warps per SM, or 80 registers and 24
-                             warps with the energy equation); block_threads may be up
-                             to 256 */
+                             warps with the energy equation; in KIN_FP64 only where
+                             blocks_per_sm asks for more than the default budget
+                             holds, since the FP64 f is slower with it); block_threads
+                             may be up to 256 */
 #define KIN_WARP_MIN_REACTIONS 256
 #define KIN_WARP_MAX_CELLS_PER_SM 64
 #define KIN_WARP_RKC_MAX_CELLS_PER_SM 470

@@ -61,6 +61,7 @@ struct Grid {
     int64_t nslots;
     int layout;           // KIN_LAYOUT_LANE or KIN_LAYOUT_WARP (resolved)
     int lanes;            // lanes per cell (1 in the lane layout)
+    int occupancy;        // register budget (resolved)
 };
 
 // Automatic layout: one warp per cell for large mechanisms (a lane's working
@@ -95,24 +96,24 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
 
 // Lanes that integrate one cell in the warp layout: half a warp for states of
 // at most 16 components (RKCK; RKC in FP64), of which FP64 calls of up to 8
-// cells per SM take a whole one (9 species RKCK, 64 cells 0.348 -> 0.295 ms; 13
-// species RKC, 1,000 cells 3.57 -> 3.05) and FP64 RKC above 64 cells per SM a
-// quarter (13 species, 4,000 cells 4.0 ms with 16 lanes and 5.6 with 8, 16,000
+// cells per SM take a whole one (9 species RKCK, 64 cells 0.348 ms with half a
+// warp, 0.295 with a whole one; 13 species RKC, 1,000 cells 3.57 and 3.05) and
+// FP64 RKC above 64 cells per SM a quarter (13 species, 4,000 cells 4.0 ms with 16 lanes and 5.6 with 8, 16,000
 // cells 9.8 and 8.6, 30,000 cells 17.9 and 14.6); else a warp, and in FP64 RKC
 // two warps above 32 components and four above 64. An evaluation is a chain of short phases, so more lanes shorten it, and the
 // FP64 pipe's vector work per cell stays the same (fewer slots per lane on more
 // warps). Measured on GB300, 2 or 4 warps against 1: 53 species, 256 / 4,096 /
 // 20,000 cells 10.4 against 18.9, 37.7 against 43.9, 157.9 against 159.4 ms;
 // 111 species, 200 / 8,000 cells 42 against 175, 231 against 323 ms. One warp
-// where the block size does not hold whole groups, and with KIN_OCC_HIGH, whose
-// 48-register kernels exist for single warps.
-int cell_lanes(const kin_opts* o, int nV, int threads, int64_t cells, int nsm)
+// where the block size does not hold whole groups, and with the small register
+// budget, whose kernels exist for single warps.
+int cell_lanes(const kin_opts* o, int occupancy, int nV, int threads, int64_t cells, int nsm)
 {
     const bool int_f = o->precision == KIN_FP64, f64 = int_f && o->method == KIN_RKC;
-    if (nV <= 16 && int_f && !o->occupancy && cells <= 8 * (int64_t)nsm) return 32;
-    if (nV <= 16 && f64 && !o->occupancy && cells > (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return 8;
+    if (nV <= 16 && int_f && !occupancy && cells <= 8 * (int64_t)nsm) return 32;
+    if (nV <= 16 && f64 && !occupancy && cells > (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return 8;
     if (nV <= 16) return o->method == KIN_RKCK || f64 ? 16 : 32;
-    if (!f64 || o->occupancy || nV <= 32) return 32;
+    if (!f64 || occupancy || nV <= 32) return 32;
     const int g = nV <= 64 ? 64 : 128;
     return threads % g ? 32 : g;
 }
@@ -133,10 +134,25 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
         return fail(KIN_EUNSUPPORTED, "the energy equation needs the mechanism's cp and Hf");
     const int layout = resolve_layout(m, o, cells, nsm);
     int threads = o->block_threads > 0 ? o->block_threads : 128;
-    int occ = 0, cap = 0, lanes = 1;
+    int occ = 0, cap = 0, lanes = 1, budget = o->occupancy;
     if (layout == KIN_LAYOUT_WARP) {
         if (threads % 32 != 0 || threads > 256) return fail(KIN_EINVAL, "block_threads must be a multiple of 32 and <= 256");
-        lanes = cell_lanes(o, m->nS + o->energy, threads, cells, nsm);
+        // The small register budget does not serve the FP64 f, which spills at it
+        // (GB300, RKC, default against KIN_OCC_HIGH with it: 13 species, 64 / 1,000 /
+        // 9,000 cells 2.5 against 4.9, 3.2 against 5.8, 6.2 against 9.3 ms; 24 species,
+        // 8,000 cells 20.9 against 22.2; 53 species, 8,000 / 20,000 cells 15.0
+        // against 18.7, 90 against 101): it is left to calls that name more blocks per
+        // SM than the other holds.
+        if (o->precision == KIN_FP64 && o->method == KIN_RKC && budget != KIN_OCC_DEFAULT) {
+            kin_opts d = *o;
+            d.occupancy = KIN_OCC_DEFAULT;
+            d.blocks_per_sm = 0;
+            d.layout = KIN_LAYOUT_WARP;
+            Grid gd;
+            if (grid_for(m, &d, cells, &gd) == KIN_OK && o->blocks_per_sm <= gd.blocks / nsm) budget = KIN_OCC_DEFAULT;
+            g_err[0] = 0;
+        }
+        lanes = cell_lanes(o, budget, m->nS + o->energy, threads, cells, nsm);
         // the layout's limit on a mechanism: C and Omega of a block's cells in
         // shared memory, at half a warp or a warp per cell (the FP64 f's own words
         // need no more: a group's chunk of a large mechanism takes 2 to 5 KB)
@@ -153,7 +169,7 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
             static const OccFn fns[2][2][2] = {
                 {{occ_warp_f64_o0, occ_warp_f64_o1}, {occ_warp_f32_o0, occ_warp_f32_o1}},
                 {{occ_warp_f64_en_o0, occ_warp_f64_en_o1}, {occ_warp_f32_en_o0, occ_warp_f32_en_o1}}};
-            e = fns[o->energy][o->precision == KIN_MIXED][o->occupancy ? 1 : 0](m->dev, nV, lanes, threads, &occ);
+            e = fns[o->energy][o->precision == KIN_MIXED][budget ? 1 : 0](m->dev, nV, lanes, threads, &occ);
         }
         cap = occ;  // as many as fit
     } else {
@@ -176,6 +192,7 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
     g->nslots = (int64_t)g->blocks * threads;
     g->layout = layout;
     g->lanes = lanes;
+    g->occupancy = budget;
     return KIN_OK;
 }
 
@@ -910,7 +927,7 @@ int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, 
         static const LaunchFn fns[2][2][2] = {
             {{launch_warp_f64_o0, launch_warp_f64_o1}, {launch_warp_f32_o0, launch_warp_f32_o1}},
             {{launch_warp_f64_en_o0, launch_warp_f64_en_o1}, {launch_warp_f32_en_o0, launch_warp_f32_en_o1}}};
-        e = fns[o->energy][o->precision == KIN_MIXED][o->occupancy ? 1 : 0](P, blocks, g.threads, st);
+        e = fns[o->energy][o->precision == KIN_MIXED][g.occupancy ? 1 : 0](P, blocks, g.threads, st);
     }
     else if (li_blocks) {
         blocks = std::min(blocks, li_blocks);
