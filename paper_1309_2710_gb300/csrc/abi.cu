@@ -94,6 +94,15 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
     return o->energy || cells < most * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
 }
 
+// The mechanism as the small register budget's FP64 kernels see it.
+MechDev small_chunks(const MechDev& d)
+{
+    MechDev s = d;
+    if (d.ig[INT_G16S].ent) s.ig[INT_G16] = d.ig[INT_G16S];
+    if (d.ig[INT_G32S].ent) s.ig[INT_G32] = d.ig[INT_G32S];
+    return s;
+}
+
 // Lanes that integrate one cell in the warp layout: half a warp for states of
 // at most 16 components (RKCK; RKC in FP64), of which FP64 calls of up to 8
 // cells per SM take a whole one (9 species RKCK, 64 cells 0.348 ms with half a
@@ -169,7 +178,8 @@ int grid_for(const kin_mech* m, const kin_opts* o, int64_t cells, Grid* g)
             static const OccFn fns[2][2][2] = {
                 {{occ_warp_f64_o0, occ_warp_f64_o1}, {occ_warp_f32_o0, occ_warp_f32_o1}},
                 {{occ_warp_f64_en_o0, occ_warp_f64_en_o1}, {occ_warp_f32_en_o0, occ_warp_f32_en_o1}}};
-            e = fns[o->energy][o->precision == KIN_MIXED][budget ? 1 : 0](m->dev, nV, lanes, threads, &occ);
+            e = fns[o->energy][o->precision == KIN_MIXED][budget ? 1 : 0](budget ? small_chunks(m->dev) : m->dev, nV, lanes,
+                                                                          threads, &occ);
         }
         cap = occ;  // as many as fit
     } else {
@@ -598,11 +608,16 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     // cost more than the shared memory
     IntGather ig[INT_NTAB];
     size_t oIg[INT_NTAB][4];
-    const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128};
-    const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS >= 32 && nS <= 64, nS >= 64};
+    const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128, 16, 32};
+    const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS >= 32 && nS <= 64, nS >= 64, nS <= 16, nS <= 64};
     for (int v = 0; v < INT_NTAB; ++v) {
         if (!ig_use[v]) continue;
-        const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, (ig_lanes[v] > 32 ? 16 : 8) * ig_lanes[v])));
+        int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, (ig_lanes[v] > 32 ? 16 : 8) * ig_lanes[v])));
+        if (v == INT_G16S || v == INT_G32S) {
+            // (with the rate constants that may be staged beside them)
+            const int words = INT_SMALL_WARP_WORDS * ig_lanes[v] / 32 - (nS + 2 * nR <= 256 ? nR + nFO : 0);
+            while (chunk > 32 && int_group_words(nS, chunk, 2 * nS + ig_lanes[v]) > words) chunk -= 32;
+        }
         ig[v] = build_int_gather(nS, nR, ptr.data(), crxp.data(), cnu.data(), chunk, ig_lanes[v]);
         oIg[v][0] = put(ig[v].step0.data(), 4 * ig[v].step0.size());
         oIg[v][1] = put(ig[v].ent.data(), 4 * ig[v].ent.size());
@@ -923,6 +938,7 @@ int kin_integrate_batch(const kin_mech* m, int32_t n, const kin_instance* inst, 
                                       : launch_warp_rkck_f64(P, blocks, g.threads, st);
     } else if (g.layout == KIN_LAYOUT_WARP) {
         using LaunchFn = cudaError_t (*)(Launch&, int, int, cudaStream_t);
+        if (g.occupancy) P.M = small_chunks(m->dev);
         // [energy][precision][occupancy]
         static const LaunchFn fns[2][2][2] = {
             {{launch_warp_f64_o0, launch_warp_f64_o1}, {launch_warp_f32_o0, launch_warp_f32_o1}},

@@ -235,11 +235,12 @@ struct IntSmem {
     }
 };
 
+static_assert(sizeof(IntCell) == 8 * INT_CELL_WORDS, "int_group_words counts it");
+
 // Shared FP64 words of a group, a multiple of 4.
 __host__ __device__ __forceinline__ int int_smem_words(const MechDev& M, const IntDev& I)
 {
-    const int w = 2 * (I.chunk + 1 + I.nslots) + ((M.nS + 1) & ~1) + (int)sizeof(IntCell) / 8 + M.nS + 1 + (M.nS + 2) / 2;
-    return (w + 3) & ~3;
+    return int_group_words(M.nS, I.chunk, I.nslots);
 }
 
 // A c_k / rho back from its mantissa.

@@ -10,10 +10,15 @@ torch = pytest.importorskip("torch")
 from paper_1309_2710_gb300 import kin, synth  # noqa: E402
 
 
-@pytest.mark.parametrize("wl,most", [("h2co_13sp_rkc", 10), ("h2co_13sp_rkc_energy", 6)])
+@pytest.mark.parametrize("wl,most", [("h2co_13sp_rkc", 10), ("ch4_53sp_rkc_mixed", 10), ("h2co_13sp_rkc_energy", 6),
+                                     ((16, 250), 10), ((32, 250), 10)])
 def test_budgets(wl, most):
-    m = synth.workload_mechanism(wl)
-    state = synth.workload_states(wl, m, cells=700)
+    if isinstance(wl, str):
+        m = synth.workload_mechanism(wl)
+        state = synth.workload_states(wl, m, cells=700)
+    else:
+        m = synth.make_mechanism(*wl, ("H", "O", "C", "N"), 0.1, 0.04, seed=1)
+        state = synth.make_states(m, 700, T_range=(900.0, 2000.0), seed=2)
     en = int(m.cp is not None)
     T, p, Y = (torch.as_tensor(a).cuda() for a in state)
     km = kin.Mechanism(m)
