@@ -1464,7 +1464,7 @@ __device__ __forceinline__ void warp_rkck_store(const WarpRKCK<R, NR, EN, G>& W,
 // the compiler's choice, one build ran the 16-species kernel at a third of its
 // speed.
 template <typename R, int NR, bool EN, int G>
-__global__ void __launch_bounds__(256, NR == 8 || (NR == 4 && sizeof(R) == 8) ? 1 : 2) warp_rkck_kernel(const __grid_constant__ Launch L)
+__global__ void __launch_bounds__(256, NR == 8 ? 1 : 2) warp_rkck_kernel(const __grid_constant__ Launch L)
 {
     using Warp = WarpRKCK<R, NR, EN, G>;
     Warp W(L);

@@ -290,7 +290,7 @@ __device__ __forceinline__ double low_exponent(const MechDev& M, int fo, const R
 // the bits depend neither on the lanes nor on the chunks. Out of line; about the
 // time of the plain FP64 f that the integer one replaced (with every row forming
 // its own rates instead, 111 species / 1566 reactions, 500 cells in RKCK took
-// 43.8 ms instead of 12.7; 23.2 in plain FP64 throughout).
+// 43.8 ms instead of 17.4; 23.2 in plain FP64 throughout).
 template <bool AT_T>
 static __device__ __noinline__ void int_general_rates(const MechDev& M, int2* CF, double* om, int q0, int q1, int lane, int lanes)
 {
