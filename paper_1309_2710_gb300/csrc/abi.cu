@@ -608,8 +608,9 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     // cost more than the shared memory
     IntGather ig[INT_NTAB];
     size_t oIg[INT_NTAB][4];
-    const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128, 16, 32};
-    const bool ig_use[INT_NTAB] = {nS <= 16, nS <= 16, true, nS >= 32 && nS <= 64, nS >= 64, nS <= 16, nS <= 64};
+    const int ig_lanes[INT_NTAB] = {8, 16, 32, 64, 128, 16, 32, 4};
+    const bool ig_use[INT_NTAB] = {nS <= 32, nS <= 16, true, nS >= 32 && nS <= 64, nS >= 64,
+                                  nS <= 16, nS <= 64, nS <= 16};
     for (int v = 0; v < INT_NTAB; ++v) {
         if (!ig_use[v]) continue;
         int chunk = std::max(32, std::min((nR + 31) / 32 * 32, std::max(64, (ig_lanes[v] > 32 ? 16 : 8) * ig_lanes[v])));

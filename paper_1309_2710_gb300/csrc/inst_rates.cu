@@ -58,7 +58,17 @@ static cudaError_t launch_nr(const MechDev& M, int64_t cells, const double* T, c
 cudaError_t launch_rates_f64(const MechDev& M, int64_t cells, const double* T, const double* p, const double* Y,
                              int64_t ldY, double* dYdt, int nsm, cudaStream_t st)
 {
+    // Lanes per cell by the mechanism alone, so that a cell's bits do not depend on
+    // the call. With few reactions more lanes would only wait; GB300, 400,000 cells,
+    // plain FP64 with a lane per cell / more lanes / these: 5 species / 8 reactions
+    // 0.223 / 0.291 / 0.189 ms, 10 / 12 0.321 / 0.360 / 0.243, 14 / 20 0.491 / 0.409 /
+    // 0.344, 17 / 20 0.515 / 0.941 / 0.455, 20 / 30 0.722 / 0.968 / 0.525; more lanes
+    // for 9 / 38 (0.423; 2,000 cells 0.026 against 0.031) and 32 / 80 (1.59; 2,000 cells
+    // 0.031 against 0.039).
+    if (M.nS <= 8 && M.nR < 24) return launch_nr<2, 4>(M, cells, T, p, Y, ldY, dYdt, nsm, st);
+    if (M.nS <= 16 && M.nR < 24) return launch_nr<4, 4>(M, cells, T, p, Y, ldY, dYdt, nsm, st);
     if (M.nS <= 16) return launch_nr<2, 8>(M, cells, T, p, Y, ldY, dYdt, nsm, st);
+    if (M.nS <= 32 && M.nR < 40) return launch_nr<4, 8>(M, cells, T, p, Y, ldY, dYdt, nsm, st);
     switch (warp_nr(M.nS, 32)) {
     case 1: return launch_nr<1, 32>(M, cells, T, p, Y, ldY, dYdt, nsm, st);
     case 2: return launch_nr<2, 32>(M, cells, T, p, Y, ldY, dYdt, nsm, st);

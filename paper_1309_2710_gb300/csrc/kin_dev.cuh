@@ -54,10 +54,10 @@ __host__ __device__ constexpr int int_group_words(int nS, int chunk, int nslots)
 {
     return (2 * (chunk + 1 + nslots) + ((nS + 1) & ~1) + INT_CELL_WORDS + nS + 1 + (nS + 2) / 2 + 3) & ~3;
 }
-// One set per number of lanes that share a cell (8 and 16: states of at most
-// 16 components; 64 and 128: more than 32 and 64), and two with chunks small
+// One set per number of lanes that share a cell (4, 8 and 16: states of at most
+// 16 components, 8 also f alone on up to 32; 64 and 128: more than 32 and 64), and two with chunks small
 // enough for the 40 warps per SM of the small register budget.
-enum IntTab : int { INT_G8 = 0, INT_G16, INT_G32, INT_G64, INT_G128, INT_G16S, INT_G32S, INT_NTAB };
+enum IntTab : int { INT_G8 = 0, INT_G16, INT_G32, INT_G64, INT_G128, INT_G16S, INT_G32S, INT_G4, INT_NTAB };
 constexpr int INT_SMALL_WARP_WORDS = 720;  // shared FP64 words of a warp's cells, 40 of them in 227 KB
 
 // Species slots of 32 in the warp layout's ELL gather tables.

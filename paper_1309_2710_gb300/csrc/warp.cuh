@@ -99,7 +99,7 @@ __device__ __forceinline__ double eff_dot<double>(const MechDev& M, int row, con
 template <int G>
 __host__ __device__ __forceinline__ const IntDev& int_tab(const MechDev& M)
 {
-    return M.ig[G == 8 ? INT_G8 : G == 16 ? INT_G16 : G == 32 ? INT_G32 : G == 64 ? INT_G64 : INT_G128];
+    return M.ig[G == 4 ? INT_G4 : G == 8 ? INT_G8 : G == 16 ? INT_G16 : G == 32 ? INT_G32 : G == 64 ? INT_G64 : INT_G128];
 }
 
 // Shared FP64 words of C [nS] and Omega [nR] in the energy and FP32 forms of
