@@ -82,7 +82,8 @@ extern "C" {
                              with the energy equation on at most 16, and isothermal
                              calls on at most 16 species below
                              KIN_WARP_RKC_MAX_CELLS_PER_SM or
-                             KIN_WARP_RKCK_MAX_CELLS_PER_SM; else KIN_LAYOUT_LANE */
+                             KIN_WARP_RKCK_MAX_CELLS_PER_SM, each up to fewer cells for
+                             mechanisms of few reactions; else KIN_LAYOUT_LANE */
 #define KIN_LAYOUT_LANE 1 /* one lane integrates one cell (the paper's thread-per-ODE
                              design, Section 3): per-cell arrays in the workspace or in
                              shared memory (kin_opts.staging) */

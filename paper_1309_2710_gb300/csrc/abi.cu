@@ -73,25 +73,43 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
     if (m->nR > KIN_WARP_MIN_REACTIONS) return KIN_LAYOUT_WARP;
     if (cells < (int64_t)KIN_WARP_MAX_CELLS_PER_SM * nsm) return KIN_LAYOUT_WARP;
     // FP64 on small mechanisms: the warp layout's integer f beats a lane per cell
-    // until the cells fill the GPU's lanes (RKC, about 78,000 lanes; half of
-    // them for RKCK, whose cells take equal times). GB300, warp against lane:
-    //   13 species RKC: 30,000 cells 14.6 against 31.4 ms, 70,000 36.0 against
-    //     36.8, 76,000 39.0 against 38.2, 262,144 135 against 97;
-    //   9 species RKCK: 20,000 cells 1.85 against 2.68, 30,000 2.68 against 2.75,
-    //     40,000 3.52 against 2.95, 100,000 8.51 against 5.50;
-    // (plain FP64 lanes, 13 species RKC: 30,000 cells 39.0, 131,072 64.3;)
-    //   24 species RKC: 12,000 cells 10.8 against 94.9, 150,000 134 against 185;
-    //   energy equation, 13 species RKC: 20,000 cells 13.3 against 68.2, 200,000
-    //     128 against 269; 9 species RKCK: 80,000 cells 13.6 against 17.4.
+    // until the cells fill the GPU's lanes (about 78,000; half of them for RKCK, whose
+    // cells take equal times), and at any size where a cell's work fills its
+    // group's lanes. Cells per SM up to which it does, from runs at 10,000 to
+    // 262,144 cells on GB300, warp against lane in ms:
+    //   up to 16 components, by reactions. RKC: 5 / 8, 20,000 cells 0.33 against 0.22;
+    //     10 / 12, 40,000 1.44 against 2.15, 71,000 2.4 against 2.3; 13 / 54, 20,000 3.1
+    //     against 11, 262,144 35 against 26 (integer f of the lane layout). RKCK: 10 /
+    //     12, 20,000 0.24 against 0.20; 14 / 20, 20,000 0.27 against 0.29, 40,000 0.46
+    //     against 0.34; 9 / 38, 20,000 0.56 against 0.87, 40,000 1.01 against 0.99.
+    //     Energy equation, RKC: 5 / 8, 20,000 0.39 against 0.31; 10 / 12 131,072 6.5
+    //     against 6.7, 262,144 12.7 against 9.4; 9 / 38, 262,144 131 against 224.
+    //     RKCK: 10 / 12, 20,000 0.32 against 0.30; 14 / 20, 40,000 0.60 against 0.59;
+    //     9 / 38, 262,144 9.6 against 10.3.
+    //   17 to 32 components, RKC, by reactions + 2 species: 17 / 20, 40,000 16.5
+    //     against 19.3, 71,000 29 against 21; 20 / 90, 71,000 36 against 42, 131,072 66
+    //     against 56; 28 / 90, 131,072 19.8 against 20.7, 262,144 39 against 36; 32 / 100,
+    //     262,144 376 against 387; 24 / 150 578 against 836. Energy equation: 20 / 30,
+    //     50,000 7.1 against 9.4, 131,072 18 against 15; 24 / 60, 131,072 16.8 against
+    //     17.0; 24 / 100, 262,144 1065 against 1537.
     // A call that names a shape or form of the lane layout keeps it.
     const bool free_shape = o->block_threads == 0 && o->blocks_per_sm == 0 && o->staging == KIN_STAGE_GLOBAL &&
                             o->occupancy == KIN_OCC_DEFAULT && o->feval == KIN_FEVAL_AUTO;
-    const int nV = m->nS + o->energy;
+    const int nV = m->nS + o->energy, nR = m->nR, any = INT_MAX;
     if (!full || !free_shape || o->precision != KIN_FP64 || nV > 32) return KIN_LAYOUT_LANE;
-    const bool rkc = o->method == KIN_RKC;
-    if (nV > 16) return rkc ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
-    const int64_t most = rkc ? KIN_WARP_RKC_MAX_CELLS_PER_SM : KIN_WARP_RKCK_MAX_CELLS_PER_SM;
-    return o->energy || cells < most * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
+    const bool rkc = o->method == KIN_RKC, en = o->energy != 0;
+    int most = KIN_WARP_MAX_CELLS_PER_SM;  // cells per SM
+    if (nV > 16) {
+        const int work = nR + 2 * m->nS;
+        if (rkc) most = work < 100 ? 330 : work < 135 ? (en ? 800 : 400) : work < 160 && !en ? 600 : any;
+    } else if (nR >= 30) {
+        most = en ? any : rkc ? KIN_WARP_RKC_MAX_CELLS_PER_SM : KIN_WARP_RKCK_MAX_CELLS_PER_SM;
+    } else if (nR >= 16) {
+        most = rkc ? (en ? 860 : KIN_WARP_RKC_MAX_CELLS_PER_SM) : en ? 260 : 150;
+    } else if (nR >= 10) {
+        most = rkc ? (en ? 860 : KIN_WARP_RKC_MAX_CELLS_PER_SM) : en ? 100 : 70;
+    }
+    return most == any || cells < (int64_t)most * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
 }
 
 // The mechanism as the small register budget's FP64 kernels see it.
