@@ -77,7 +77,8 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
     // cells take equal times), and at any size where a cell's work fills its
     // group's lanes. Cells per SM up to which it does, from runs at 10,000 to
     // 262,144 cells on GB300, warp against lane in ms:
-    //   up to 16 components, by reactions. RKC: 5 / 8, 20,000 cells 0.33 against 0.22;
+    //   up to 16 components, by reactions. RKC: 5 / 8, 10,000 cells 0.23 against 0.19,
+    //     20,000 0.33 against 0.22;
     //     10 / 12, 40,000 1.44 against 2.15, 71,000 2.4 against 2.3; 13 / 54, 20,000 3.1
     //     against 11, 262,144 35 against 26 (integer f of the lane layout). RKCK: 10 /
     //     12, 20,000 0.24 against 0.20; 14 / 20, 20,000 0.27 against 0.29, 40,000 0.46
@@ -108,6 +109,8 @@ int resolve_layout(const kin_mech* m, const kin_opts* o, int64_t cells, int nsm,
         most = rkc ? (en ? 860 : KIN_WARP_RKC_MAX_CELLS_PER_SM) : en ? 260 : 150;
     } else if (nR >= 10) {
         most = rkc ? (en ? 860 : KIN_WARP_RKC_MAX_CELLS_PER_SM) : en ? 100 : 70;
+    } else if (rkc && !en) {
+        most = 100;
     }
     return most == any || cells < (int64_t)most * nsm ? KIN_LAYOUT_WARP : KIN_LAYOUT_LANE;
 }
@@ -539,18 +542,18 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     const size_t oRxw = put(rxw.data(), 4 * nR);
     const size_t oCrxp = put(crxp.data(), 4 * nnz);
     // the rows once more in order of position
-    std::vector<int> crxq(nnz), byPos;
+    std::vector<int> crxq(nnz + 1, 0), byPos;
     std::vector<double> cnuq(nnz);
     for (int i = 0; i < nS; ++i) {
         byPos.clear();
         for (int e2 = ptr[i]; e2 < ptr[i + 1]; ++e2) byPos.push_back(e2);
         std::sort(byPos.begin(), byPos.end(), [&](int a, int b) { return crxp[a] < crxp[b]; });
         for (size_t k = 0; k < byPos.size(); ++k) {
-            crxq[ptr[i] + k] = crxp[byPos[k]];
+            crxq[ptr[i] + k] = crxp[byPos[k]] << 3 | ((int)cnu[byPos[k]] + 4);
             cnuq[ptr[i] + k] = cnu[byPos[k]];
         }
     }
-    const size_t oCrxq = put(crxq.data(), 4 * nnz), oCnuq = put(cnuq.data(), 8 * nnz);
+    const size_t oCrxq = put(crxq.data(), 4 * (nnz + 1)), oCnuq = put(cnuq.data(), 8 * nnz);
     const size_t oEffV64 = put(effV64.data(), 8 * effV64.size()), oEffV32 = put(effV32.data(), 4 * effV32.size());
     const size_t oPtr = put(ptr.data(), 4 * (nS + 1)), oCrx = put(crx.data(), 4 * nnz);
     const size_t oNu = put(cnu.data(), 8 * nnz), oNu32 = put(nu32.data(), 4 * nnz);
@@ -747,7 +750,7 @@ int kin_create_mechanism(const kin_mech_desc* d, kin_mech** out)
     M.rxn_perm = (const int*)(b + oPerm);
     M.rxnp = (const Rxn*)(b + oRxp);
     M.csrp_rxn = (const int*)(b + oCrxp);
-    M.csrq_rxn = (const int*)(b + oCrxq);
+    M.csrq = (const int*)(b + oCrxq);
     M.csrq_nu = (const double*)(b + oCnuq);
     M.ell32 = (const CsrW32*)(b + oEll32);
     M.ell64 = (const CsrW64*)(b + oEll64);

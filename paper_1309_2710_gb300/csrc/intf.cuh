@@ -260,15 +260,15 @@ __device__ __forceinline__ double im_log(const ulonglong2* __restrict__ tab, dou
 //
 // A row's sum of fewer than MechDev::imShort = 53 + log2(entries) bits could
 // miss an ulp in the bits below the unit: a species whose rates are all far
-// below the cell's largest, or whose rates cancel. Such rows are summed again on
-// their own: with a unit of their own largest rate (int_row_sum, one lane's
-// work), or in the lane layout, all of them together, with the unit IM_STEP octaves
-// lower, modulo 2^128 (the sum itself fits, the words that do not wrap around), and
-// so on until each has its bits or no rate has bits below the unit, when the sums
-// are exact (lane_int_lower). The workloads' cells have no net rate below 2^-36 of
-// their largest, and a net rate of 2^-37 has its bits, so that they pay for the
-// test alone, 1 to 2 % of a call. Inside the common code the further sums' registers
-// and branches would cost 5 to 38 %.
+// below the cell's largest, or whose rates cancel. Such rows are summed again: with
+// the unit of their own largest rate (int_short), or in the lane layout, all of
+// them together, with the unit IM_STEP octaves lower, modulo 2^128 (the sum itself
+// fits, the words that do not wrap around), and so on until each has its bits or no
+// rate has bits below the unit, when the sums are exact (lane_int_lower). The
+// workloads' cells have no net rate below 2^-36 of their largest, and a net rate
+// of 2^-37 has its bits, so that they pay for the test alone, 2 to 5 % of a call.
+// Inside the common code the further sums' registers and branches would cost 5 to
+// 38 %.
 constexpr int IM_GUARD = 8, IM_SLACK = 8, IM_STEP = 56;
 
 // Exponent that stands for a rate that is not finite.

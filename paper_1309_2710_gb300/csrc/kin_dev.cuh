@@ -99,8 +99,8 @@ struct MechDev {
     const int32_t* effX;   // [nM] their exponents
     const double* arr;     // [3][nR] ln A, beta, E / R in permutation order
     const double* arr0;    // [3][nFO] the low-pressure limits'
-    const int* csrq_rxn;   // [nnz] the species' rows in order of position, and their nu
-    const double* csrq_nu;
+    const int* csrq;       // [nnz + 1] the species' rows in order of position: position << 3 | nu + 4
+    const double* csrq_nu; // [nnz] their nu
     const uint4* scl;      // [nR] estimate of the rates' exponents (int_scale_table)
     const unsigned long long* ex2;  // tables of im_exp and im_log
     const ulonglong2* lnc;

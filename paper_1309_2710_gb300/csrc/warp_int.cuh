@@ -326,7 +326,7 @@ static __device__ __noinline__ IntRow int_general_row(const MechDev& M, const do
     const int end = M.csr_ptr[i + 1];
 #pragma unroll 1
     for (; a.e < end; ++a.e) {
-        const int q = M.csrq_rxn[a.e];
+        const int q = M.csrq[a.e] >> 3;
         if (q >= q1) break;
         a.w += M.csrq_nu[a.e] * om[q - q0];
     }
@@ -468,41 +468,93 @@ __device__ __forceinline__ bool int_rate(const MechDev& M, const IntSmem& S, con
     return in;
 }
 
-// W_i omega_i / rho of a species whose words are too short for it (intf.cuh): its
-// rates once more, one after another, placed by the largest of them so far. One
-// lane's chain, and rarely taken, so it is out of line, with rolled loops, and
-// reads the cell's values from shared memory: with more of its registers around,
-// cells without such species lose up to 8 % (now 2 %; GB300, 53 species / 634
-// reactions, 4,096 cells 20.2 -> 20.4 ms, 21.9 with its third-body sum unrolled).
+// Sums that are too short for their last bits (intf.cuh), once more: the lanes'
+// rates of a chunk of reactions as mantissas and exponents, then each such species'
+// sum over its row (csrq, in order of position), placed by the largest of them so
+// far. Rarely taken, so it is out of line with rolled loops, and reads the cell's
+// values from shared memory: with more of its registers around, cells without such
+// species lose up to 12 % (now 2 to 5 %). A cell with such species takes two to three
+// times as long, about the plain FP64 f's time or less: GB300, 53 species / 634
+// reactions, unburnt mixtures, 4,096 cells with radicals of zero 2.9 ms (without
+// these sums, and wrong, 1.35; plain FP64 2.5), of 1e-22 to 1e-9 7.0 (5.3, 11.5); f
+// alone, 50,000 cells 2.1 and 1.4 (0.69, 0.85; 2.8). Row by row with each row's rates
+// formed anew it was 12, 11, 10 and 1.9 ms.
+// Shift of the largest rate's word there: 61 + 43 bits, the entries of the longest
+// row (two for each reaction) and the sign.
+constexpr int INT_SHORT_UP = 43;
+
 template <bool AT_T>
-static __device__ __noinline__ double int_row_sum(const MechDev& M, int2* CF, int i)
+static __device__ __noinline__ void int_short_rates(const MechDev& M, int2* CF, ulonglong2* om, int q0, int q1, int lane, int lanes)
 {
     const IntSmem S(M, CF);
     const IntMix mix = S.cell->mix;
     const RateSource rk = S.cell->rk;
-    constexpr int UP = 43;  // 61 + 43 bits and the entries of the longest row, two for each reaction
-    im_u128 acc{0ull, 0ull};
-    int at = -1;
 #pragma unroll 1
-    for (int c = M.csr_ptr[i]; c < M.csr_ptr[i + 1]; ++c) {
-        const int q = M.csrp_rxn[c];
-        const double nu = M.csr_nu[c], kq = AT_T ? M.arr[q] : rk.K[q];
+    for (int q = q0 + lane; q < q1; q += lanes) {
+        const double kq = AT_T ? M.arr[q] : rk.K[q];
         im_u64 Q;
         uint32_t e;
         int_rate<AT_T, false>(M, S, rk, mix, q, M.rxw[q], kq, AT_T ? M.arr[M.nR + q] : 0.0, AT_T ? M.arr[2 * M.nR + q] : 0.0, Q, e);
-        if (!Q || (!AT_T && !im_normal_k(kq))) continue;
-        const int x = (int)(e & 0x7fffffffu);
-        if (x > at) {
-            im_sar(acc, x - max(at, 0));
-            at = x;
-        }
-        const im_u128 v = im_place(Q, x - at + UP);
-        const bool neg = (e >> 31 != 0u) != (nu < 0.0);
-        for (int n = (int)fabs(nu); n > 0; --n)
-            if (neg) im_sub(acc, v.lo, v.hi);
-            else im_add(acc, v.lo, v.hi);
+        if (!AT_T && !im_normal_k(kq)) Q = 0ull;
+        om[q - q0] = make_ulonglong2(Q, e);
     }
-    return im_scaled(acc, at - UP - 3 * IM_BIAS, M.imW[i].y, M.imWe[i].y, mix.mr, (int)mix.er);
+}
+
+// A species' sum, its scale (-1: no rate so far) and the next entry of its row.
+struct IntSum {
+    im_u128 w;
+    int at, e;
+};
+// The sum with the row's entries up to position q1.
+static __device__ __noinline__ IntSum int_short_row(const MechDev& M, const ulonglong2* om, int q0, int q1, int end, IntSum a)
+{
+    int next = M.csrq[a.e];  // (the table ends in a word past the last row)
+#pragma unroll 1
+    for (; a.e < end; ++a.e) {
+        const int q = next >> 3, nu = (next & 7) - 4;
+        if (q >= q1) break;
+        next = M.csrq[a.e + 1];
+        const ulonglong2 v = om[q - q0];
+        if (v.x == 0ull) continue;
+        const int x = (int)(v.y & 0x7fffffffull);
+        if (x > a.at) {
+            im_sar(a.w, x - max(a.at, 0));
+            a.at = x;
+        }
+        const im_u128 u = im_place(v.x, x - a.at + INT_SHORT_UP);
+        const bool neg = (v.y >> 31 != 0ull) != (nu < 0);
+        for (int n = abs(nu); n > 0; --n)
+            if (neg) im_sub(a.w, u.lo, u.hi);
+            else im_add(a.w, u.lo, u.hi);
+    }
+    return a;
+}
+
+// The group's species in `left` (a bit per slot).
+template <int NR, int G, bool AT_T>
+__device__ __forceinline__ void int_short(const MechDev& M, const IntDev& I, const IntSmem& S, unsigned left,
+                                          double (&out)[NR], int lane, const Group<G>& grp)
+{
+    IntSum a[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) a[r] = IntSum{{0ull, 0ull}, -1, lane + G * r < M.nS ? M.csr_ptr[lane + G * r] : 0};
+#pragma unroll 1
+    for (int q0 = 0; q0 < M.nR; q0 += I.chunk) {
+        const int q1 = min(M.nR, q0 + I.chunk);
+        int_short_rates<AT_T>(M, S.CF, S.OM, q0, q1, lane, G);
+        grp.sync();
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            if (left >> r & 1u) a[r] = int_short_row(M, S.OM, q0, q1, M.csr_ptr[lane + G * r + 1], a[r]);
+        grp.sync();
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + G * r;
+        if (left >> r & 1u)
+            out[r] = im_scaled(a[r].w, a[r].at - INT_SHORT_UP - 3 * IM_BIAS, M.imW[i].y, M.imWe[i].y, S.cell->mix.mr,
+                               (int)S.cell->mix.er);
+    }
 }
 
 // About the largest rate's exponent of the lane's reactions, for the first
@@ -536,7 +588,9 @@ __device__ __forceinline__ int int_first_scale(const MechDev& M, const IntSmem& 
 // (at the first a value that does not depend on other cells, for the bits of the
 // result not to; AT_T: -1, and int_first_scale gives one); an evaluation whose largest rate is more than
 // IM_GUARD octaves above it or IM_SLACK below is repeated with that rate's. The
-// barriers around the gather carry the two tests. kfin: the cell's rate constants are finite.
+// barriers around the gather carry the two tests, the one at the end whether a
+// sum is too short for its last bits (int_short). kfin: the cell's rate constants
+// are finite.
 template <int NR, int G, bool AT_T>
 __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I, const IntSmem& S,
                                                const RateSource& rk, bool kfin, double Ctot, double invCtot,
@@ -709,17 +763,8 @@ __device__ __forceinline__ void warp_feval_int(const MechDev& M, const IntDev& I
                 if (w && im_short(acc[r], M.imShort)) left |= 1u << r;
                 out[r] = im_scaled(acc[r], scale - M.imUp - 3 * IM_BIAS, w, M.imWe[i].y, mix.mr, (int)mix.er);
             }
-#pragma unroll 1
-            for (; left; left &= left - 1u) {
-                const int k = __ffs(left) - 1;
-                const double v = int_row_sum<AT_T>(M, S.CF, lane + G * k);
-#pragma unroll
-                for (int r = 0; r < NR; ++r)
-                    if (r == k) out[r] = v;
-            }
-            // the shared words are rewritten by the next evaluation (across
-            // warps, only after the barrier of its mixture sum)
-            if constexpr (G <= 32) grp.sync();
+            // (the shared words are rewritten after this barrier)
+            if (grp.sync_any(left != 0u)) int_short<NR, G, AT_T>(M, I, S, left, out, lane, grp);
             return;
         }
         emax = grp.imax(emax);

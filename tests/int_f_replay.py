@@ -156,9 +156,10 @@ extern "C" void* mech_new(int nS, int nR, const double* W, const double* lnA, co
         std::vector<std::pair<int, double>> row;
         for (int k = m->ptr[i]; k < m->ptr[i + 1]; ++k) row.push_back({m->pos[k], m->nu[k]});
         std::sort(row.begin(), row.end());
-        for (auto& e : row) m->posq.push_back(e.first), m->nuq.push_back(e.second);
+        for (auto& e : row) m->posq.push_back(e.first << 3 | ((int)e.second + 4)), m->nuq.push_back(e.second);
     }
-    m->M.csrq_rxn = m->posq.data();
+    m->posq.push_back(0);
+    m->M.csrq = m->posq.data();
     m->M.csrq_nu = m->nuq.data();
     const int chunk = std::max(32, std::min((nR + 31) / 32 * 32, 256));
     m->g = build_int_gather(nS, nR, m->ptr.data(), m->pos.data(), m->nu.data(), chunk, LANES);
