@@ -71,15 +71,6 @@ __device__ __forceinline__ bool im_normal_k(double v) { return ((uint32_t)__doub
 __device__ __forceinline__ bool im_finite_k(double v) { return ((uint32_t)__double2hiint(v) >> 20) < 0x7ffu; }
 __device__ __forceinline__ bool im_finite_k(float v) { return (__float_as_uint(v) >> 23) < 0xffu; }
 
-// v cut to FP32, without the FP64 pipe's conversion (beyond its range: 0, or infinite).
-__device__ __forceinline__ float im_f32(double v)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), s = hi & 0x80000000u;
-    const int x = (int)((hi >> 20) & 0x7ffu) - 896;
-    if (x <= 0) return 0.0f;
-    return __uint_as_float(s | (x >= 255 ? 0x7f800000u : (uint32_t)x << 23 | (hi & 0xfffffu) << 3 | lo >> 29));
-}
-
 struct im_u128 {
     im_u64 lo, hi;
 };

@@ -557,6 +557,15 @@ __device__ __forceinline__ void int_short(const MechDev& M, const IntDev& I, con
     }
 }
 
+// v cut to FP32, without the FP64 pipe's conversion (beyond its range: 0, or infinite).
+__device__ __forceinline__ float im_f32(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), s = hi & 0x80000000u;
+    const int x = (int)((hi >> 20) & 0x7ffu) - 896;
+    if (x <= 0) return 0.0f;
+    return __uint_as_float(s | (x >= 255 ? 0x7f800000u : (uint32_t)x << 23 | (hi & 0xfffffu) << 3 | lo >> 29));
+}
+
 // About the largest rate's exponent of the lane's reactions, for the first
 // evaluation of a cell: a few octaves too high where a third-body sum is small
 // beside its largest efficiency, more where a falloff is. A function of the cell
