@@ -335,8 +335,10 @@ int kin_integrate_noalloc(const kin_mech *m, int64_t cells, double *T, const dou
  * (KIN_FP64 or KIN_MIXED), enqueued on `stream`. T, p, Y, dYdt and workspace
  * are device pointers; dYdt has the layout of Y. The workspace rule is that of
  * kin_integrate with method KIN_RKC, the same precision, layout
- * KIN_LAYOUT_LANE, default launch shape and `cells` cells. Errors:
- * KIN_EINVAL, KIN_ENOMEM, KIN_ECUDA. */
+ * KIN_LAYOUT_LANE, default launch shape and `cells` cells. In KIN_FP64 every
+ * species' rate has FP64 accuracy relative to the sum of its own |nu_ij Omega_j|,
+ * however far below the cell's largest rate, and a cell's bits do not depend on
+ * the call's other cells. Errors: KIN_EINVAL, KIN_ENOMEM, KIN_ECUDA. */
 int kin_rates(const kin_mech *m, int64_t cells, const double *T, const double *p,
               const double *Y, int64_t ldY, double *dYdt, int32_t precision, void *stream,
               void *workspace, int64_t workspace_bytes);

@@ -4,7 +4,7 @@
 // A cell of 53 species / 634 reactions takes 659 exponentials and 8,160 other
 // operations; on the FP64 pipe the exponentials alone (some 20 instructions
 // each) take 1.1 ms for 50,000 cells, and the lane-per-cell form streamed its
-// rate constants and rates of progress through L2 besides: 2.80 ms, 0.76 now.
+// rate constants and rates of progress through L2 besides: 2.80 ms, 0.755 now.
 // Each cell's scale comes from the cell itself (int_first_scale), so its bits do
 // not depend on the call's other cells.
 #include "warp.cuh"

@@ -12,8 +12,9 @@
 // warps per SM that its registers and shared words leave: 17 K instructions of a
 // full warp per evaluation at 0.44 per cycle and scheduler. The plain FP64 code
 // that it replaces kept the FP64 pipe 85 % busy, 64 cycles per instruction.
-// GB300, 13 species / 54 reactions RKC: 262,144 cells 122 -> 97 ms, 131,072
-// 64.3 -> 49.3; 9 / 38 RKCK, 60,000 cells 4.7 -> 3.2. Loops over the state's
+// GB300, 13 species / 54 reactions RKC: 262,144 cells 122 -> 100 ms (97 without the
+// test of the sums' length and the wider limbs), 131,072 64.3 -> 50; 9 / 38 RKCK,
+// 60,000 cells 4.7 -> 3.2. Loops over the state's
 // vectors unrolled (104 ms) or their loads batched (102 to 139, spills) are
 // slower, tables in constant memory no faster (96).
 #pragma once

@@ -15,13 +15,15 @@
 // 1780; the FP64 f it replaced took 43 K with one warp, 354 FP64 instructions
 // of 64 cycles among them). So a lane's next reaction words, the gather's next
 // entries and eight efficiencies of a third-body sum are fetched ahead.
-// Whole calls on GB300, before and after: 53 / 634 RKC, 4,096 cells 76.1 ->
-// 38.4 ms; 111 / 1566 RKC, 16 instances of 2,000 cells in all 1061 -> 226 ms;
-// 13 / 54 RKC, 1,000 cells 3.75 -> 3.03 ms, 30,011 cells 38.4 -> 15.3; 9 / 38 RKCK,
-// 4,096 cells 0.716 -> 0.468 ms; energy equation, 13 / 54, 20,000 cells 67.1 -> 13.3;
-// f alone, 53 / 634, 50,000 cells 2.81 -> 0.71 ms. Error of whole results
-// against plain FP64: unchanged (1e-13, the finite differences of the spectral
-// radius).
+// (Cycles from a build without the test of the sums' length and the wider limbs,
+// which add 2 to 5 %.)
+// Whole calls on GB300, plain FP64 f and this one: 53 / 634 RKC, 4,096 cells 77.0 and
+// 40.0 ms; 111 / 1566 RKC, 16 instances of 2,000 cells in all 1061 and 231 ms;
+// 13 / 54 RKC, 1,000 cells 3.75 and 3.08 ms, 30,011 cells 38.4 and 15.9; 9 / 38 RKCK,
+// 4,096 cells 0.716 and 0.489 ms; energy equation, 13 / 54, 20,000 cells 66.8 and
+// 14.1 (54.6 to 69 from state to state before); f alone, 53 / 634, 50,000 cells 2.80
+// and 0.755 ms. Error of whole results against 64 bits: that of plain FP64 (1e-13
+// and below, the finite differences of the spectral radius).
 #pragma once
 #include "intf.cuh"
 #include "kernels.cuh"
